@@ -483,6 +483,9 @@ int assemble_impl(cps_ctx ctx, const double* xy, int64_t nv, const int32_t* tri,
             const int g3 = grid_for(ctx, 3 * nt);
             const int g1 = grid_for(ctx, nt);
             const int gf = grid_for(ctx, nf);
+            // the arrival counters of the grid reductions start at zero (memory
+            // a freed system gave back need not be)
+            cudaMemsetAsync(s->st, 0, sizeof(CgState) * 2, stream);
             cudaMemsetAsync(keys, 0xFF, sizeof(unsigned long long) * cap, stream);
             cudaMemsetAsync(id0, 0xFF, sizeof(int32_t) * cap, stream);
             cudaMemsetAsync(id1, 0xFF, sizeof(int32_t) * cap, stream);

@@ -97,3 +97,25 @@ def test_tiny_systems_batched(ctx):
             assert _err(x, xo) < tol
     for s in systems:
         s.free()
+
+
+def test_systems_in_memory_given_back_by_others(ctx):
+    """The iteration state of a new system starts from zero even where its
+    memory held another, freed system's arrays: small systems are solved and
+    freed in turn, and a larger one solved on every streaming kernel after
+    them converges."""
+    for seed, n in enumerate((12, 33, 5, 64, 21)):
+        p = synth.centred_block_problem(n, seed=seed)
+        s = _assemble(ctx, p)
+        s.set_solver_path(cps.PATH_STREAM)
+        s.solve(torch.as_tensor(synth.rhs(p.mesh, seed), device="cuda"), rtol=1e-8)
+        s.free()
+    p = synth.channel_block_problem(48, seed=1)
+    b = synth.rhs(p.mesh, 2)
+    xo, _, _ = oracle.solve_problem(p, b, rtol=1e-13)
+    s = _assemble(ctx, p)
+    for path in (cps.PATH_STREAM, cps.PATH_STREAM_1RED, cps.PATH_AUTO):
+        s.set_solver_path(path)
+        x, _ = s.solve(torch.as_tensor(b, device="cuda"), rtol=1e-10)
+        assert _err(x, xo) < 1e-9
+    s.free()
