@@ -109,8 +109,17 @@ def traffic_for(tf: dict, n: int):
     return None
 
 
+# CG on the Schur complement S of one colour (half of the cells), per row and
+# step: the row of S (diagonal 8, six values 48, six columns 24) and x, r, p, q
+# read and written once (64); one step is two Jacobi iterations of all cells.
+BYTES_PER_ROW_STEP_SCHUR = 144
+
+
 def loop_name(tf: dict) -> str:
     """The FP64 Jacobi loop the tuner chose, with its kernels."""
+    if tf.get("two_cyclic"):
+        return ("k_schur_cg (two-cyclic form of Jacobi-PCG: CG on the explicit Schur complement "
+                "of one colour in one cooperative launch, two Jacobi iterations a step)")
     if tf.get("persistent_single_reduction"):
         kname = ("k_persistent_gear (whole Jacobi-PCG solve in one cooperative launch, "
                  "Chronopoulos-Gear recurrences)")
@@ -141,8 +150,21 @@ def loop_name(tf: dict) -> str:
 
 def loop_bytes(tf: dict) -> int:
     """Bytes per cell per iteration the chosen FP64 Jacobi loop moves."""
+    if tf.get("two_cyclic"):
+        return BYTES_PER_ROW_STEP_SCHUR // 4
     single = tf["stream_single_reduction"] or tf.get("persistent_single_reduction")
     return BYTES_PER_CELL_ITER_FP64_1RED if single else BYTES_PER_CELL_ITER_FP64
+
+
+def method_bytes(name: str, tf: dict) -> float:
+    """Bytes per cell per iteration of a FP64 solve variant's method, each array
+    once: on all cells, or on the Schur complement of one colour."""
+    if name == "jacobi":
+        return BYTES_PER_ROW_STEP_SCHUR / 4 if tf.get("two_cyclic") else BYTES_PER_CELL_ITER_METHOD
+    if name == "ic0":      # scaled rows: no diagonal
+        return (BYTES_PER_ROW_STEP_SCHUR - 8) / 2 if tf["ic0_persistent"] else \
+            BYTES_PER_CELL_ITER_METHOD + 40
+    return BYTES_PER_ROW_STEP_SCHUR / 2 if tf["reduced_single_reduction"] else 160 / 2
 
 
 def roofline(tf: dict, nt: int, iters: int, seconds: float, peak: float, peak_kind: str,
@@ -153,6 +175,18 @@ def roofline(tf: dict, nt: int, iters: int, seconds: float, peak: float, peak_ki
     true residual included), so the per-iteration figure is a lower bound."""
     per_iter = seconds / max(iters, 1)
     bpc = loop_bytes(tf)
+    if tf.get("two_cyclic"):
+        # the method's bytes are those of CG on S: half of the rows, and half
+        # of the steps that the iteration count says
+        achieved = bpc * nt / per_iter / 1e9
+        return {"bound": "fp64 issue (matrix and vectors stay in L2 and shared memory at this "
+                         "size); bytes are CG's on S", "kernel": loop_name(tf),
+                "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
+                "peak_kind": peak_kind, "bytes_per_cell_iter": bpc,
+                "algorithmic_bytes_per_iter": bpc * nt, "us_per_iter": 1e6 * per_iter,
+                "iterations": "Jacobi-PCG iterations, two per step on S",
+                "us_per_step": 2e6 * per_iter, "traffic": None,
+                "traffic_source": "no capture of this loop and configuration"}
     achieved = BYTES_PER_CELL_ITER_METHOD * nt / per_iter / 1e9
     loop_achieved = bpc * nt / per_iter / 1e9
     traffic = traffic_for(tf, n)
@@ -713,8 +747,7 @@ def sequence_summary(n: int, rtol: float, iters: int = 200) -> dict:
     after one untimed solve that also tunes); the reduced system, the fastest
     FP64 solver here, is timed to rtol on a second right-hand side,
     warm-started from the first one's solution.  GB/s are the method's
-    algorithmic bytes (108 B/cell/iter Jacobi, 60.5 mixed inner, 148 IC(0),
-    80 reduced) over the measured copy bandwidth.  `bench.py --sequence`
+    algorithmic bytes (method_bytes; 60.5 B/cell/iter mixed inner) over the measured copy bandwidth.  `bench.py --sequence`
     runs the longer sequence of solves to rtol."""
     import torch
     import paper_2309_03543_gb300 as cps
@@ -745,6 +778,8 @@ def sequence_summary(n: int, rtol: float, iters: int = 200) -> dict:
         x.zero_()
         t, st = timed(lambda: s.solve(rhs[0], x=x, rtol=rtol, max_iter=iters, precision=prec,
                                       check=False)[1], stream)
+        if prec == cps.FP64:
+            bpc = method_bytes(name.split("_")[0], s.tuning(cps.FP64))
         gbs = bpc * nt * st.iters / t / 1e9
         out[name] = {"iters": st.iters, "us_per_iter": 1e6 * t / max(st.iters, 1),
                      "bytes_per_cell_iter": bpc, "algorithmic_gbs": gbs, "frac": gbs / peak}
@@ -754,11 +789,12 @@ def sequence_summary(n: int, rtol: float, iters: int = 200) -> dict:
     x.zero_()
     s.solve(rhs[0], x=x, rtol=rtol, max_iter=iters, check=False)      # tunes its path
     t, st = timed(lambda: s.solve(rhs[1], x=x, rtol=rtol, check=False)[1], stream)
-    gbs = 80 * nt * st.iters / t / 1e9
+    bpc = method_bytes("reduced", s.tuning(cps.FP64))
+    gbs = bpc * nt * st.iters / t / 1e9
     out["reduced_fp64_to_rtol"] = {
         "time_to_rtol_s": t, "iters": st.iters, "rel_res": st.rel_res, "status": st.status,
         "warm_start": "from the solution of a capped solve of the first right-hand side",
-        "us_per_iter": 1e6 * t / max(st.iters, 1), "bytes_per_cell_iter": 80,
+        "us_per_iter": 1e6 * t / max(st.iters, 1), "bytes_per_cell_iter": bpc,
         "algorithmic_gbs": gbs, "frac": gbs / peak}
     s.free()
     ctx.close()
@@ -814,6 +850,8 @@ def run_sequence(args):
             rel.append(st.rel_res)
             status.append(st.status)
             per.append(dt_)
+        if prec == cps.FP64:
+            bpc = method_bytes(name, s.tuning(cps.FP64))
         # reduced system: iterations run over the black half of the cells
         units = nt // 2 if pc == cps.PC_REDUCED else nt
         gbs = bpc * nt * it_tot / t_tot / 1e9
@@ -1006,11 +1044,12 @@ def run_graded(args):
             if name == "jacobi":
                 tf = s.tuning(cps.FP64)
                 bpc = loop_bytes(tf)
-                gbs = BYTES_PER_CELL_ITER_METHOD * cells / (t / st.iters) / 1e9
+                mpc = method_bytes("jacobi", tf)
+                gbs = mpc * cells / (t / st.iters) / 1e9
                 entry.update({"algorithmic_gbs": gbs, "frac": gbs / peak,
-                              "bytes_per_cell_iter": BYTES_PER_CELL_ITER_METHOD,
+                              "bytes_per_cell_iter": mpc,
                               "loop_bytes_per_cell_iter": bpc,
-                              "loop_frac": bpc / BYTES_PER_CELL_ITER_METHOD * gbs / peak,
+                              "loop_frac": bpc / mpc * gbs / peak,
                               "path": tf})
             res[f"{order}_{name}"] = entry
         s.free()

@@ -339,7 +339,12 @@ int cps_cp2_kernel_times(cps_sys sys, float* ms);
 
 /* Choose how FP64 Jacobi and reduced-system solves run:
  *   CPS_PATH_AUTO (default): the autotuner times the applicable paths on the
- *     system's first solve of that kind and keeps the fastest;
+ *     system's first solve of that kind and keeps the fastest.  FP64 Jacobi
+ *     solves of a CP2 system whose cell graph has two colours may then run in
+ *     two-cyclic form: from a zero residual on one colour, two Jacobi-PCG
+ *     iterations are one CG iteration on the other colour's Schur complement
+ *     (half the unknowns), and stats->iters counts two for each (max_iter
+ *     bounds that count);
  *   CPS_PATH_STREAM: graph-replayed streaming kernels, any size;
  *   CPS_PATH_CLUSTER (FP64 Jacobi only): the whole solve in one launch of a
  *     single thread-block cluster whose shared memory holds the system;
@@ -383,14 +388,12 @@ int cps_cp2_kernel_times(cps_sys sys, float* ms);
  *   CPS_PATH_PERSISTENT_1RED, CPS_PATH_PERSISTENT_1RED_L2 (FP64 Jacobi,
  *     FP64 IC(0) in a two-colour order, and the reduced system): the
  *     persistent launch with the single-reduction recurrences -- per
- *     iteration one grid reduction and waits on the neighbouring blocks only
- *     (Jacobi: one; IC(0): two, in Eisenstat's form of the preconditioned
- *     iteration, which applies the two-colour IC(0) factor and the matrix in
- *     one pass over the matrix, with the same iterates; reduced system: two,
- *     around the two halves of the Schur product) -- without / with its
- *     vectors in persisting L2 (Jacobi and the reduced system: five,
- *     CPS_ERR_ARG when the set-aside cannot hold them; IC(0): six where they
- *     fit, else five, else none).
+ *     iteration one grid reduction and one wait on the neighbouring blocks
+ *     (IC(0) and the reduced system on explicit rows of the Schur complement,
+ *     for IC(0) scaled by its diagonal: from a zero residual on the
+ *     eliminated colour the same iterates) -- without / with its five vectors
+ *     in persisting L2 (CPS_ERR_ARG when the set-aside cannot hold them;
+ *     IC(0): then without).
  * FP64 IC(0) in a two-colour order runs on the streaming kernels for every
  * other pin, and CPS_PATH_AUTO times both ways on the first such solve; with
  * more colours it always streams.
@@ -453,7 +456,7 @@ int cps_test_inject(cps_sys sys, int fault);
  * single-reduction loop), single-reduction
  * streaming chosen, single-reduction persistent launch chosen, IC(0):
  * persistent single-reduction launch chosen (0 no, 1 without a window, 2
- * with its first five vectors, 3 with all six in persisting L2)}, flags
+ * with its five vectors in persisting L2)}, flags
  * then taking 8 entries; probe_us (may be
  * NULL, 18 entries) the microseconds per iteration measured for {streaming,
  * one cluster (the best of its three recurrences), streaming + matrix in L2, persistent, streaming + vectors in
@@ -477,6 +480,13 @@ int cps_get_gear_shape(cps_sys sys, int32_t* unroll, int32_t* grid, int32_t* blo
 
 int cps_get_tuning(cps_sys sys, int precision, int32_t* unroll, int32_t* grid, int32_t* block,
                    int32_t* flags, double* probe_us);
+
+/* Whether FP64 Jacobi solves of this system run in the two-cyclic form (see
+ * CPS_PATH_AUTO), and the microseconds per CG iteration on the Schur
+ * complement its probe measured (0 before the first such solve, or where it
+ * was not timed on this system's mesh size).  Either output may be NULL.
+ * Errors: CPS_ERR_ARG. */
+int cps_get_two_cyclic(cps_sys sys, int32_t* taken, double* us_per_iter);
 
 /* Allocation-free solve of a matrix the caller already holds in the padded
  * ELL form that cps_export_matrix writes (no counterpart in the paper; it is

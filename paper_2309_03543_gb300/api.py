@@ -152,7 +152,11 @@ class System:
         self.ctx.check(self.ctx.lib.cps_get_gear_shape(self.handle, ctypes.byref(gu),
                                                       ctypes.byref(gg), ctypes.byref(gb)),
                        "cps_get_gear_shape")
+        tc, tus = ctypes.c_int32(), ctypes.c_double()
+        self.ctx.check(self.ctx.lib.cps_get_two_cyclic(self.handle, ctypes.byref(tc),
+                                                      ctypes.byref(tus)), "cps_get_two_cyclic")
         return {"unroll": list(u), "grid": list(g), "block": list(bl),
+                "two_cyclic": bool(tc.value), "two_cyclic_us_per_iter": tus.value,
                 "cluster": bool(f[0]),
                 "cluster_recurrence": (None, "textbook", "single_reduction", "pipelined", "s_step2",
                                        "s_step3")[f[0]],
@@ -163,7 +167,7 @@ class System:
                 "stream_single_reduction": bool(f[5]),
                 "persistent_single_reduction": bool(f[6]),
                 "ic0_persistent": bool(f[7]),
-                "ic0_l2_window": ("none", "none", "vectors5", "vectors6")[f[7]],
+                "ic0_l2_window": ("none", "none", "vectors5")[f[7]],
                 "update_1red": [gu.value, gg.value, gb.value],
                 "probe_us_per_iter": {
                     "stream": pr[0], "cluster": pr[1], "stream_l2_matrix": pr[2],

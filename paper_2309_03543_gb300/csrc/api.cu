@@ -51,6 +51,9 @@ int cps_create(cps_ctx* out, int device) {
     int l2 = 0;
     cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, device);
     c->l2_bytes = (size_t)l2;
+    int so = 0;
+    cudaDeviceGetAttribute(&so, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
+    c->smem_optin = (size_t)so;
     int lp = 0;
     cudaDeviceGetAttribute(&lp, cudaDevAttrMaxPersistingL2CacheSize, device);
     c->l2_persist_max = (size_t)lp;
@@ -223,21 +226,21 @@ int cps_set_batch_path(cps_ctx ctx, int path) {
 int cps_set_solver_path(cps_sys sys, int path) {
     if (!sys) return CPS_ERR_ARG;
     cps::Tuning& t = sys->tune[CPS_FP64];
+    t.pinned = path != CPS_PATH_AUTO;
     if (path >= CPS_PATH_STREAM && path <= CPS_PATH_PERSISTENT_1RED_L2) {
         // IC(0) in a two-colour order: the persistent single-reduction loop
         // for the CPS_PATH_PERSISTENT_1RED pins, the streaming kernels for
         // the others
         t.ic0_done = true;
         t.ic0_path = (path == CPS_PATH_PERSISTENT_1RED || path == CPS_PATH_PERSISTENT_1RED_L2) ? 1 : 0;
-        t.ic0_win = path != CPS_PATH_PERSISTENT_1RED_L2 ? 0
-                    : cps::l2_window_fits_mode(sys, 4) ? 4
-                    : cps::l2_window_fits_mode(sys, 3) ? 3 : 0;
+        t.ic0_win = path == CPS_PATH_PERSISTENT_1RED_L2 && cps::l2_window_fits_mode(sys, 3) ? 3 : 0;
     }
     if (path == CPS_PATH_AUTO) {
         t.ic0_done = false;
         t.ic0_path = 0;
         t.path_done = false;
         t.path = 0;
+        t.tc = 0;
         t.red_done = false;
         t.red_path = 0;
     } else if (path == CPS_PATH_STREAM) {
@@ -382,7 +385,7 @@ int cps_get_tuning(cps_sys sys, int precision, int32_t* unroll, int32_t* grid, i
         flags[5] = t.path_done && t.path == 3;
         flags[6] = t.path_done && t.path == 4;
         flags[7] = (t.ic0_done && t.ic0_path == 1 && sys->ncolours == 2)
-                       ? (t.ic0_win == 4 ? 3 : (t.ic0_win == 3 ? 2 : 1))
+                       ? (t.ic0_win ? 2 : 1)
                        : 0;
     }
     if (probe_us) {
@@ -407,6 +410,14 @@ int cps_get_gear_shape(cps_sys sys, int32_t* unroll, int32_t* grid, int32_t* blo
     *unroll = t.done ? (c.block == 1024 && c.unroll > 2 ? 2 : c.unroll) : 0;
     *grid = t.done ? c.grid : 0;
     *block = t.done ? c.block : 0;
+    return CPS_OK;
+}
+
+int cps_get_two_cyclic(cps_sys sys, int32_t* taken, double* us_per_iter) {
+    if (!sys) return CPS_ERR_ARG;
+    const cps::Tuning& t = sys->tune[CPS_FP64];
+    if (taken) *taken = t.tc == 1 && !t.pinned && sys->sch.buf ? 1 : 0;
+    if (us_per_iter) *us_per_iter = t.tc_us;
     return CPS_OK;
 }
 

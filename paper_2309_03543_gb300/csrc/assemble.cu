@@ -347,6 +347,7 @@ void free_sys(cps_sys s) {
     if (!s) return;
     free_cp2(s);
     free_cp1(s);
+    free_schur(s);
     // s->col lives inside s->a's allocation (one range for the L2 window)
     void* bufs[] = {s->s,     s->diag,  s->a,     s->a32,     s->s32,      s->gfac,
                     s->dxi,   s->slot_kind, s->perm, s->iperm, s->pa,  s->pcol,     s->pl,

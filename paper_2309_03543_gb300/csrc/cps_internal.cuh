@@ -88,8 +88,13 @@ struct Tuning {
     // FP64 IC(0) in a two-colour order: 0 graph-replayed streaming kernels,
     // 1 one persistent launch of the single-reduction recurrences
     int ic0_path = 0;
-    int ic0_win = 0;         // persisting L2 window of the persistent IC(0) loop (0 or 4)
+    int ic0_win = 0;         // persisting L2 window of the persistent IC(0) loop (0 or 3)
     bool ic0_done = false;
+    bool pinned = false;     // cps_set_solver_path chose the path (not CPS_PATH_AUTO)
+    // FP64 Jacobi on a two-coloured graph, two-cyclic form (schur.cu): 0 not
+    // timed, 1 taken by CPS_PATH_AUTO, 2 slower than the loop above
+    int tc = 0;
+    double tc_us = 0.0;      // us per CG iteration on the Schur complement
     double ic0_probe_us[2] = {0, 0};   // us/iteration: streaming, persistent (best window)
 };
 
@@ -180,6 +185,25 @@ struct Cp2Data {
     float kernel_ms[3] = {0.f, 0.f, 0.f};   // last step: mean flux, tangential, update
 };
 
+// The black cells' Schur complement of a two-coloured system, explicit rows,
+// and the vectors of CG on it (schur.cu); every array is a slice of buf.
+struct SchurData {
+    void* buf = nullptr;
+    double* r = nullptr;      // [ld] each; r, w, p, s, y contiguous
+    double* w = nullptr;
+    double* p = nullptr;
+    double* s = nullptr;
+    double* y = nullptr;
+    double* v = nullptr;      // [6][ld] off-diagonals
+    double* d = nullptr;      // [ld] diagonal of S (form 1: the rows'; form 2: before scaling)
+    double* wt = nullptr;     // [ld] weight of the stop test
+    double* dsc = nullptr;    // [ld] D^-1/2 (form 2)
+    int32_t* c = nullptr;     // [6][ld] columns (= row for an unused slot)
+    unsigned long long* pb = nullptr;   // tagged block totals of the reductions
+    int64_t ld = 0, nB = 0;
+    int form = 0;             // 0 not built, 1 S, 2 D^-1/2 S D^-1/2
+};
+
 // Block-wide sum of v[0..NV) over BS threads (BS = blockDim.x); on return
 // every thread holds the totals.  GB300 issues FP64 adds at 1/64 of the FP32
 // rate, so the adds are kept few: every thread stores its values to shared
@@ -247,6 +271,7 @@ struct cps_ctx_s {
     int num_sms = 0;
     int max_threads_per_sm = 2048;
     size_t l2_bytes = 0;
+    size_t smem_optin = 0;       // shared memory a block may opt in to
     size_t l2_persist_max = 0;   // cudaDevAttrMaxPersistingL2CacheSize
     size_t l2_persist_set = 0;   // persisting L2 limit this process has set
     std::string last_error;
@@ -297,7 +322,11 @@ struct cps_sys_s {
     double* dxi = nullptr;      // [nt]
     int32_t* slot_kind = nullptr;   // [3*nt] 0 no-flux, 1 interior, 2 Dirichlet
 
-    // IC(0) in colour order (scaled matrix, unit diagonal), set up on demand.
+    // Colour order of the cells (perm, iperm; ncolours 0: not ordered, -1:
+    // two colours do not suffice and no other order was asked for) and IC(0)
+    // in it (scaled matrix, unit diagonal), each set up on demand.
+    bool factored = false;
+    cps::SchurData sch;
     int ncolours = 0;
     int64_t colour_start[17] = {0};
     int32_t* perm = nullptr;    // [nt] colour order -> mesh order
@@ -373,6 +402,15 @@ int assemble_impl(cps_ctx ctx, const double* xy, int64_t nv, const int32_t* tri,
                   int field_loc, int kind, double nu, double dt, cps_sys* out,
                   cudaStream_t stream);
 int precond_impl(cps_sys sys, int precond, cudaStream_t stream);
+int two_colour_order(cps_sys s, cudaStream_t stream, bool* ok);
+void free_schur(cps_sys s);
+int schur_setup(cps_sys s, bool scaled, cudaStream_t stream);
+int schur_grid(cps_sys s);
+int schur_init(cps_sys s, const double* b, const double* x, double rtol, long long budget,
+               cudaStream_t stream);
+int schur_back(cps_sys s, const double* b, cudaStream_t stream);
+int schur_run(cps_sys s, int grid, bool window, cudaStream_t stream);
+size_t schur_window_bytes(cps_sys s);
 int solve_impl(cps_sys sys, const double* b, double* x, double rtol, int64_t max_iter,
                int precision, cps_stats* stats, cudaStream_t stream);
 int solve_batch_impl(const cps_sys* systems, int nsys, const double* const* b,
@@ -389,8 +427,7 @@ int cluster_solve(cps_sys s, const double* b, const double* x, double* y, double
 int persistent_solve(cps_sys s, int reduced, const double* a, const int32_t* col,
                      const double* sc, double* y, double* r, double* p, double* q, double* t,
                      int64_t n, int64_t nR, const void* win_base, size_t win_bytes, int grid,
-                     cudaStream_t stream, double* z = nullptr, const double* dinv = nullptr,
-                     const double* dpiv = nullptr);
+                     cudaStream_t stream);
 int persistent_max_grid(cps_sys s, int reduced);
 bool l2_vectors_fit(cps_sys s);
 bool l2_window_fits_mode(cps_sys s, int mode);

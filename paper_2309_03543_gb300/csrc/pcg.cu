@@ -356,6 +356,8 @@ static int autotune(cps_sys s, int prec, const Run<V>& v, cudaStream_t stream) {
                 c.grid = grid_for(s->ctx, s->nt * kBlock / sh.block, sh.per_sm);
                 if (c.unroll == keep.unroll && c.block == keep.block && c.grid == keep.grid)
                     continue;
+                // a trip that no thread fills runs one row at a time, as unroll 1
+                if (c.unroll > 1 && (int64_t)c.unroll * c.grid * c.block > s->nt) continue;
                 t.k[kind] = c;
                 const float ms = time_loop();
                 if (ms < best) {
@@ -421,13 +423,14 @@ static int64_t enqueue_iteration(cps_sys s, const Run<V>& v, int prec, bool norm
 // million cells either fits GB300's 129 MB L2 next to the streamed rest.
 // Mode 3, for the single-reduction loop, holds r, p, q (= s), y and p1
 // (= w): every vector that loop reads and writes (five contiguous slices);
-// mode 4, for the single-reduction IC(0) loop, also z (six slices).
+// mode 5 the five vectors of the explicit Schur loop (schur.cu).
 static void* l2_window_base(cps_sys s, int mode) {
     return mode == 1 ? (void*)s->a : (void*)s->wr;
 }
 static size_t l2_window_bytes(cps_sys s, int mode) {
     if (mode == 1) return s->mat_bytes;
-    return (size_t)(mode == 4 ? 6 : (mode == 3 ? 5 : 3)) * s->vec_stride * sizeof(double);
+    if (mode == 5) return schur_window_bytes(s);
+    return (size_t)(mode == 3 ? 5 : 3) * s->vec_stride * sizeof(double);
 }
 static bool l2_window_fits(cps_sys s, int mode) {
     return s->ctx->l2_persist_max > 0 && l2_window_bytes(s, mode) <= s->ctx->l2_persist_max;
@@ -797,22 +800,127 @@ static int choose_fp64_path(cps_sys s, const Run<double>& v, const double* b,
     return rc;
 }
 
-// One persistent single-reduction IC(0) run from the state k_init64 left
-// (colour order, two colours), with persisting L2 window `win` (the caller
-// holds its set-aside) on `grid` blocks (0: all that stay resident).
-static int persistent_ic0(cps_sys s, int win, cudaStream_t stream) {
-    return persistent_solve(s, 3, s->pa, s->pcol, s->ps, s->wy, s->wr, s->wp0, s->wq, s->wp1,
-                            s->nt, s->colour_start[1], win ? l2_window_base(s, win) : nullptr,
-                            win ? l2_window_bytes(s, win) : 0, 0, stream, s->wz, s->pdinv,
-                            s->pdiag);
+// Microseconds per iteration of the explicit Schur loop (schur.cu) over a
+// short run from x = 0 on `grid` blocks (0: the default), with or without its
+// vectors in persisting L2; 0 where it cannot run here.
+static int probe_schur(cps_sys s, const double* b, long long probe, int grid, bool window,
+                       cudaEvent_t e0, cudaEvent_t e1, cudaStream_t stream, double* us) {
+    *us = 0.0;
+    int rc = l2_set_aside(s, window ? 5 : 0, stream);
+    if (rc) return rc;
+    CPS_CUDA_TRY(s->ctx, cudaMemsetAsync(s->wx, 0, sizeof(double) * s->nt, stream));
+    for (int rep = 0; rep < 2; ++rep) {          // the first one warms up
+        CPS_CUDA_TRY(s->ctx, cudaEventRecord(e0, stream));
+        rc = schur_init(s, b, s->wx, 0.0, probe, stream);
+        if (rc == CPS_OK) rc = schur_run(s, grid, window, stream);
+        CgState h{};
+        if (rc == CPS_OK) rc = read_state(s, stream, &h);
+        if (rc) return rc;
+        if (h.status != CPS_OK) return CPS_OK;                 // not usable here
+        CPS_CUDA_TRY(s->ctx, cudaEventRecord(e1, stream));
+        CPS_CUDA_TRY(s->ctx, cudaEventSynchronize(e1));
+        float ms = 0.f;
+        cudaEventElapsedTime(&ms, e0, e1);
+        *us = 1e3 * ms / (double)(h.iter > 0 ? h.iter : 1);
+    }
+    return CPS_OK;
+}
+
+// A whole solve on the explicit Schur rows (schur.cu; the caller has set them
+// up): `per` iterations of the solve's method per CG iteration on S (2 for
+// Jacobi, 1 for IC(0) and the reduced system).
+static int solve_two_cyclic(cps_sys s, const double* b, double* x, double rtol, int64_t max_iter,
+                            int per, int grid, bool window, cps_stats* stats,
+                            cudaStream_t stream) {
+    const int64_t n = s->nt;
+    int64_t total = 0, launches = 0;
+    if (window) {
+        int rc = l2_set_aside(s, 5, stream);
+        if (rc) return rc;
+    }
+    CgState h{};
+    int status = CPS_OK;
+    // restarts from the true residual, as in solve_fp64
+    for (int restart = 0; restart < 8; ++restart) {
+        const int64_t left = max_iter - total;
+        int rc = schur_init(s, b, x, rtol, left / per + (left % per ? 1 : 0), stream);
+        if (rc == CPS_OK) rc = schur_run(s, grid, window, stream);
+        if (rc == CPS_OK) rc = schur_back(s, b, stream);
+        if (rc) return rc;
+        k_final64<<<s->grid, kBlock, 0, stream>>>(b, s->wy, s->s, s->a, s->col, n, x, s->partials,
+                                                  s->st);
+        launches += 5;
+        CPS_CUDA_TRY(s->ctx, cudaGetLastError());
+        rc = read_state(s, stream, &h);
+        if (rc) return rc;
+        const int64_t done = h.iter * per;
+        total += done < left ? done : left;
+        status = h.status;
+        if (status != CPS_OK || h.rnorm2 <= h.thresh2 || total >= max_iter) break;
+    }
+    if (window) {
+        int rc = l2_set_aside(s, 0, stream);
+        if (rc) return rc;
+    }
+    const double rel = h.bnorm2 > 0 ? std::sqrt(h.rnorm2 / h.bnorm2) : 0.0;
+    if (status == CPS_OK && h.bnorm2 > 0 && !(rel <= rtol)) status = CPS_ERR_NOT_CONVERGED;
+    fill_stats(stats, total, rel, status, 1, launches);
+    if (status == CPS_ERR_NOT_SPD)
+        cps::set_error(s->ctx, "solve: p.Ap <= 0 (matrix not SPD or NaN input)");
+    if (status == CPS_ERR_TIMEOUT) cps::set_error(s->ctx, "solve: a grid barrier wait ran out");
+    if (status == CPS_ERR_NOT_CONVERGED)
+        cps::set_error(s->ctx, total >= max_iter
+                                   ? "solve: max_iter reached"
+                                   : "solve: the true residual stays above rtol (FP64 rounding "
+                                     "floor of this system and right-hand side)");
+    return status;
+}
+
+// FP64 Jacobi under CPS_PATH_AUTO: whether the two-cyclic form is taken, its
+// rows then set up.  Taken on two-colourable CP2 systems (no mass term: a
+// solve is hundreds of iterations, against which the colouring and the rows
+// cost nothing; a CP1 system converges in about eight) where one CG iteration
+// on S costs less than two of the loop the tuner chose.
+static int choose_two_cyclic(cps_sys s, const double* b, cudaStream_t stream, bool* take) {
+    *take = false;
+    Tuning& t = s->tune[CPS_FP64];
+    if (t.pinned || s->kind != CPS_KIND_CP2 || t.tc == 2) return CPS_OK;
+    bool two = false;
+    int rc = two_colour_order(s, stream, &two);
+    if (rc == CPS_OK && two) rc = schur_setup(s, false, stream);
+    if (rc == CPS_ERR_NOMEM) {              // no room for the rows: the loop on all cells
+        cudaGetLastError();
+        return CPS_OK;
+    }
+    if (rc || !two) return rc;
+    if (t.tc == 0) {
+        cudaEvent_t e0, e1;
+        CPS_CUDA_TRY(s->ctx, cudaEventCreate(&e0));
+        CPS_CUDA_TRY(s->ctx, cudaEventCreate(&e1));
+        double us = 0.0, best = 0.0;
+        rc = probe_schur(s, b, s->nt >= kTuneMinRows ? 256 : 64, 0, false, e0, e1, stream, &us);
+        cudaEventDestroy(e0);
+        cudaEventDestroy(e1);
+        if (rc) return rc;
+        for (double p : t.probe_us)
+            if (p > 0.0 && (best == 0.0 || p < best)) best = p;
+        t.tc = us > 0.0 && (best == 0.0 || us < 2.0 * best) ? 1 : 2;
+        t.tc_us = us;
+        update_cached_tuning(s, CPS_FP64, [&](Tuning& c) {
+            c.tc = t.tc;
+            c.tc_us = t.tc_us;
+        });
+    }
+    *take = t.tc == 1;
+    return CPS_OK;
 }
 
 // For IC(0) on a two-colour order: times a short run (64 iterations; 256 on
 // large systems) of the graph-replayed streaming kernels and of the
-// persistent single-reduction launch (without and, where the set-aside holds
-// them, with its six vectors in persisting L2) and keeps the fastest.  bb is
-// the right-hand side in colour order.
-static int choose_ic0_path(cps_sys s, const Run<double>& v, const double* bb,
+// persistent single-reduction launch on the scaled Schur rows (without and,
+// where the set-aside holds them, with its vectors in persisting L2) and keeps
+// the fastest.  bb is the right-hand side b in colour order.
+static int choose_ic0_path(cps_sys s, const Run<double>& v, const double* b, const double* bb,
                            cudaStream_t stream) {
     Tuning& t = s->tune[CPS_FP64];
     t.ic0_done = true;
@@ -826,12 +934,9 @@ static int choose_ic0_path(cps_sys s, const Run<double>& v, const double* bb,
     Cand cands[3];
     int nc = 0;
     cands[nc++] = {0, 0};
-    if (persistent_max_grid(s, 3) > 0) {
+    if (schur_setup(s, true, stream) == CPS_OK) {
         cands[nc++] = {1, 0};
-        // six vectors in persisting L2 where they fit, else the first five
-        // (xh, rh, p, s, w: all but v / z)
-        if (s->nt >= kTuneMinRows && l2_window_fits(s, 4)) cands[nc++] = {1, 4};
-        else if (s->nt >= kTuneMinRows && l2_window_fits(s, 3)) cands[nc++] = {1, 3};
+        if (s->nt >= kTuneMinRows && l2_window_fits(s, 3)) cands[nc++] = {1, 3};
     }
     cudaEvent_t e0, e1;
     CPS_CUDA_TRY(s->ctx, cudaEventCreate(&e0));
@@ -843,9 +948,10 @@ static int choose_ic0_path(cps_sys s, const Run<double>& v, const double* bb,
     int64_t dummy = 0;
     for (int ci = 0; ci < nc && rc == CPS_OK; ++ci) {
         const Cand c = cands[ci];
-        rc = l2_set_aside(s, c.win, stream);
         double us = 0.0;
-        for (int rep = 0; rep < 2 && rc == CPS_OK; ++rep) {    // the first one warms up
+        if (c.path == 1) rc = probe_schur(s, b, probe, 0, c.win != 0, e0, e1, stream, &us);
+        else rc = l2_set_aside(s, c.win, stream);
+        for (int rep = 0; rep < 2 && rc == CPS_OK && c.path == 0; ++rep) {   // the first warms up
             if (cudaMemsetAsync(s->wx, 0, sizeof(double) * s->nt, stream) != cudaSuccess ||
                 cudaEventRecord(e0, stream) != cudaSuccess) {
                 rc = CPS_ERR_CUDA;
@@ -854,15 +960,9 @@ static int choose_ic0_path(cps_sys s, const Run<double>& v, const double* bb,
             k_init64<<<s->grid, kBlock, 0, stream>>>(bb, s->wx, v.s, v.a, v.col, s->nt, v.y, v.r,
                                                      v.p0, 0.0, probe, 0, s->partials, s->st);
             CgState h{};
-            if (c.path == 1) {
-                rc = persistent_ic0(s, c.win, stream);
-                if (rc == CPS_OK) rc = read_state(s, stream, &h);
-                if (rc == CPS_OK && h.status != CPS_OK) rc = CPS_ERR_ARG;   // not usable here
-            } else {
-                enqueue_precond<double>(s, v, stream);
-                k_copy<double><<<s->grid, kBlock, 0, stream>>>(v.p0, v.z, s->nt);
-                rc = run_chunks<double>(s, CPS_FP64, v, stream, &h, &dummy);
-            }
+            enqueue_precond<double>(s, v, stream);
+            k_copy<double><<<s->grid, kBlock, 0, stream>>>(v.p0, v.z, s->nt);
+            rc = run_chunks<double>(s, CPS_FP64, v, stream, &h, &dummy);
             if (cudaEventRecord(e1, stream) != cudaSuccess ||
                 cudaEventSynchronize(e1) != cudaSuccess) {
                 rc = CPS_ERR_CUDA;
@@ -922,6 +1022,12 @@ static int solve_fp64(cps_sys s, const double* b, double* x, double rtol, int64_
         int rc = choose_fp64_path(s, v, b, stream);
         if (rc) return rc;
     }
+    if (!ic0) {
+        bool take = false;
+        int rc = choose_two_cyclic(s, b, stream, &take);
+        if (rc) return rc;
+        if (take) return solve_two_cyclic(s, b, x, rtol, max_iter, 2, 0, false, stats, stream);
+    }
     const bool cluster = !ic0 && s->tune[CPS_FP64].path == 1;
     const bool persistent = !ic0 && (s->tune[CPS_FP64].path == 2 || s->tune[CPS_FP64].path == 4);
     const bool pgear = !ic0 && s->tune[CPS_FP64].path == 4;
@@ -940,18 +1046,16 @@ static int solve_fp64(cps_sys s, const double* b, double* x, double rtol, int64_
             // the probe runs from x = 0 in wx: keep the caller's start in wbest
             CPS_CUDA_TRY(s->ctx, cudaMemcpyAsync(s->wbest, s->wx, sizeof(double) * n,
                                                  cudaMemcpyDeviceToDevice, stream));
-            int rc = choose_ic0_path(s, v, bb, stream);
+            int rc = choose_ic0_path(s, v, b, bb, stream);
             if (rc) return rc;
             CPS_CUDA_TRY(s->ctx, cudaMemcpyAsync(s->wx, s->wbest, sizeof(double) * n,
                                                  cudaMemcpyDeviceToDevice, stream));
         }
     }
-    const bool pic0 = ic0 && s->ncolours == 2 && s->tune[CPS_FP64].ic0_path == 1;
-    const int ic0_window = pic0 ? s->tune[CPS_FP64].ic0_win : 0;
-    if (ic0_window) {
-        int rc = l2_set_aside(s, ic0_window, stream);
-        if (rc) return rc;
-    }
+    if (ic0 && s->ncolours == 2 && s->tune[CPS_FP64].ic0_path == 1 &&
+        schur_setup(s, true, stream) == CPS_OK)
+        return solve_two_cyclic(s, b, x, rtol, max_iter, 1, 0, s->tune[CPS_FP64].ic0_win != 0,
+                                stats, stream);
     CgState h{};
     int status = CPS_OK;
     // A restart recomputes r = b - A x when the recursively updated residual
@@ -979,24 +1083,6 @@ static int solve_fp64(cps_sys s, const double* b, double* x, double rtol, int64_
         k_init64<<<g, kBlock, 0, stream>>>(bb, xx, v.s, v.a, v.col, n, v.y, v.r, v.p0, rtol,
                                             budget, ic0 ? 0 : 1, s->partials, s->st);
         ++launches;
-        if (pic0) {
-            // one launch runs to the stop (it returns at once if init stopped)
-            int rc = persistent_ic0(s, ic0_window, stream);
-            if (rc) return rc;
-            ++launches;
-            rc = read_state(s, stream, &h);
-            if (rc) return rc;
-            total += h.iter;
-            status = h.status;
-            k_final64<<<g, kBlock, 0, stream>>>(bb, v.y, v.s, v.a, v.col, n, xx, s->partials,
-                                                s->st);
-            ++launches;
-            CPS_CUDA_TRY(s->ctx, cudaGetLastError());
-            rc = read_state(s, stream, &h);
-            if (rc) return rc;
-            if (status != CPS_OK || h.rnorm2 <= h.thresh2 || total >= max_iter) break;
-            continue;
-        }
         if (persistent) {
             if (pgear) {
                 k_gear_start<<<g, kBlock, 0, stream>>>(v.a, v.col, v.r, v.p1, v.p0, v.q, n,
@@ -1056,7 +1142,7 @@ static int solve_fp64(cps_sys s, const double* b, double* x, double rtol, int64_
         CPS_CUDA_TRY(s->ctx, cudaGetLastError());
         CPS_CUDA_TRY(s->ctx, cudaStreamSynchronize(stream));
     }
-    if (window || ic0_window) {
+    if (window) {
         // release the lines and the set-aside: later work gets the whole L2
         int rc = l2_set_aside(s, 0, stream);
         if (rc) return rc;
@@ -1088,8 +1174,6 @@ static int solve_reduced(cps_sys s, const double* b, double* x, double rtol, int
     const double* S = s->ps;
     double *y = s->wy, *r = s->wr, *p = s->wp0, *q = s->wq, *t = s->wz;
     int64_t total = 0, launches = 0;
-    k_permute_in<<<g, kBlock, 0, stream>>>(b, x, s->perm, n, s->wb, s->wx);
-    ++launches;
     const double* bb = s->wb;
     double* xx = s->wx;
     // black-range views for the shared update kernels
@@ -1148,15 +1232,13 @@ static int solve_reduced(cps_sys s, const double* b, double* x, double rtol, int
     };
     // Runs CG from the state k_black_init left, on the graph-replayed kernels
     // (kind 0) or in one persistent grid-synchronised launch of pgrid blocks
-    // (kind 1 the textbook recurrences, 2 the single-reduction ones, with
-    // s = S p in q and w = S r in p1), with window win (the caller holds its
-    // set-aside); state into *hh.
+    // (kind 1), with window win (the caller holds its set-aside); state into
+    // *hh.
     auto run_cg = [&](int kind, int win, int pgrid, CgState* hh) -> int {
         if (kind) {
-            int rc = persistent_solve(s, kind == 2 ? 4 : 1, A, col, S, y, r, p, q, t, n, nR,
+            int rc = persistent_solve(s, 1, A, col, S, y, r, p, q, t, n, nR,
                                       win ? l2_window_base(s, win) : nullptr,
-                                      win ? l2_window_bytes(s, win) : 0, pgrid, stream,
-                                      kind == 2 ? s->wp1 : nullptr);
+                                      win ? l2_window_bytes(s, win) : 0, pgrid, stream);
             if (rc) return rc;
             ++launches;
             return read_state(s, stream, hh);
@@ -1183,8 +1265,9 @@ static int solve_reduced(cps_sys s, const double* b, double* x, double rtol, int
     if (!tu.red_done) {
         // time a short run of each way from x = 0 and keep the fastest:
         // slot 0 graph, 1 persistent, 2 graph + window, 3 persistent + window,
-        // 4 persistent single-reduction, 5 the same + its five vectors in
-        // persisting L2 (persistent at a few grid sizes)
+        // 4 persistent single-reduction on the explicit rows, 5 the same + its
+        // five vectors in persisting L2 (persistent at a few grid sizes)
+        k_permute_in<<<g, kBlock, 0, stream>>>(b, x, s->perm, n, s->wb, s->wx);
         const long long probe = nB >= kTuneMinRows ? 256 : 64;
         const bool try_win = nB >= kTuneMinRows && l2_window_fits(s, 2);
         const bool try_win5 = nB >= kTuneMinRows && l2_window_fits(s, 3);
@@ -1195,8 +1278,12 @@ static int solve_reduced(cps_sys s, const double* b, double* x, double rtol, int
         int nc = 0;
         cands[nc++] = {0, 0, 0};
         if (try_win) cands[nc++] = {2, 2, 0};
-        for (int kind = 1; kind <= 2; ++kind) {
-            const int gmax = persistent_max_grid(s, kind == 2 ? 4 : 1);
+        if (schur_setup(s, false, stream) == CPS_OK) {
+            cands[nc++] = {4, 0, 0};
+            if (try_win5) cands[nc++] = {5, 3, 0};
+        }
+        {
+            const int gmax = persistent_max_grid(s, 1);
             int grids[3] = {gmax, (int)((nB + 8191) / 8192), (int)((nB + 2047) / 2048)};
             for (int i = 0; i < 3; ++i) {
                 const int gi = grids[i] < 1 ? 1 : (grids[i] > gmax ? gmax : grids[i]);
@@ -1204,13 +1291,8 @@ static int solve_reduced(cps_sys s, const double* b, double* x, double rtol, int
                 for (int j = 0; j < i; ++j) dup = dup || grids[j] == gi;
                 grids[i] = gi;
                 if (dup) continue;
-                if (kind == 1) {
-                    cands[nc++] = {1, 0, gi};
-                    if (try_win) cands[nc++] = {3, 2, gi};
-                } else {
-                    cands[nc++] = {4, 0, gi};
-                    if (try_win5) cands[nc++] = {5, 3, gi};
-                }
+                cands[nc++] = {1, 0, gi};
+                if (try_win) cands[nc++] = {3, 2, gi};
             }
         }
         cudaEvent_t e0, e1;
@@ -1225,9 +1307,10 @@ static int solve_reduced(cps_sys s, const double* b, double* x, double rtol, int
             const Cand c = cands[ci];
             const int kind = kind_of(c.slot);
             const bool pers = kind != 0;
-            rc = l2_set_aside(s, c.win, stream);
             double us = 0.0;
-            for (int rep = 0; rep < 2 && rc == CPS_OK; ++rep) {
+            if (kind == 2) rc = probe_schur(s, b, probe, 0, c.win != 0, e0, e1, stream, &us);
+            else rc = l2_set_aside(s, c.win, stream);
+            for (int rep = 0; rep < 2 && rc == CPS_OK && kind != 2; ++rep) {
                 CPS_CUDA_TRY(s->ctx, cudaMemsetAsync(xx, 0, sizeof(double) * n, stream));
                 if (!pers) rc = build_graph(c.win);        // outside the timed region
                 if (rc) break;
@@ -1276,8 +1359,14 @@ static int solve_reduced(cps_sys s, const double* b, double* x, double rtol, int
             for (int k = 0; k < 6; ++k) c.red_probe_us[k] = tu.red_probe_us[k];
         });
     }
-    const int kind = tu.red_path;
+    int kind = tu.red_path;
     const int win = tu.red_win;
+    if (kind == 2 && schur_setup(s, false, stream) != CPS_OK) kind = 1;   // no room for the rows
+    if (kind == 2) {
+        return solve_two_cyclic(s, b, x, rtol, max_iter, 1, tu.red_pgrid, win != 0, stats, stream);
+    }
+    k_permute_in<<<g, kBlock, 0, stream>>>(b, x, s->perm, n, s->wb, s->wx);
+    ++launches;
     if (win) {
         int rc = l2_set_aside(s, win, stream);
         if (rc) return rc;

@@ -31,67 +31,13 @@
 // waiting on it then run out too, so the kernel always ends.
 #include "cps_internal.cuh"
 #include "exact_sum.cuh"
+#include "grid_sync.cuh"
 
 #include <cmath>
 #include <cstddef>
 
 namespace cps {
 namespace {
-
-constexpr int kPBlock = 1024;
-constexpr long long kSpinCap = 1LL << 26;           // polls; each one an L2 round trip
-constexpr unsigned long long kWaitNs = 1000000000ull;
-constexpr int kFlagStride = 16;                      // one 128-byte line per block flag
-constexpr int kMaxDeps = 8;
-constexpr int kPartialSlots = 4;                     // quantities per reduction buffer
-
-struct GridSync {
-    unsigned long long count;   // arrivals since the launch
-    int timeout;
-    int pad[29];
-    unsigned long long flag[kMaxGrid * kFlagStride];   // per-block iteration flags
-};
-
-__device__ __forceinline__ void red_release_add(unsigned long long* p, unsigned long long v) {
-    asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-
-__device__ __forceinline__ void st_release(unsigned long long* p, unsigned long long v) {
-    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-
-__device__ __forceinline__ unsigned long long ld_acquire(const unsigned long long* p) {
-    unsigned long long v;
-    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
-}
-
-// Hint: fetch the line holding p into this SM's L1 (no register result).
-__device__ __forceinline__ void prefetch_l1(const void* p) {
-    asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
-}
-
-__device__ __forceinline__ unsigned long long global_ns() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
-// Bounded wait until *p >= target (one thread).  False if it ran out, or if
-// another block has already recorded a timeout.
-__device__ bool wait_geq(const unsigned long long* p, unsigned long long target, GridSync* gs) {
-    if (ld_acquire(p) < target) {
-        const unsigned long long t0 = global_ns();
-        for (long long spins = 1;; ++spins) {
-            if (ld_acquire(p) >= target) break;
-            if (spins > kSpinCap || ((spins & 255) == 0 && global_ns() - t0 > kWaitNs)) {
-                atomicExch(&gs->timeout, 1);
-                return false;
-            }
-        }
-    }
-    return *(volatile int*)&gs->timeout == 0;
-}
 
 // Barriers passed by this block: reductions (k picks the partial buffer) and
 // the arrival count that completes the latest barrier (every barrier adds its
@@ -200,28 +146,6 @@ __device__ bool grid_barrier(GridSync* gs, Epoch& ep) {
     return s_ok != 0;
 }
 
-// This block has finished phase `slot` (0: direction update, 1: the reduced
-// system's red phase) `it` times.
-__device__ __forceinline__ void halo_post(GridSync* gs, unsigned long long it, int slot = 0) {
-    __syncthreads();
-    if (threadIdx.x == 0) st_release(&gs->flag[blockIdx.x * kFlagStride + slot], it);
-}
-
-// Wait until the blocks [dlo, dhi] (other than this one) have posted `it`
-// in `slot`.
-__device__ bool halo_wait(GridSync* gs, int dlo, int dhi, unsigned long long it, int slot = 0) {
-    __shared__ int s_ok;
-    if (threadIdx.x == 0) {
-        int ok = 1;
-        for (int d = dlo; d <= dhi && ok; ++d)
-            if (d != (int)blockIdx.x && !wait_geq(&gs->flag[d * kFlagStride + slot], it, gs))
-                ok = 0;
-        s_ok = ok;
-    }
-    __syncthreads();
-    return s_ok != 0;
-}
-
 // Range [*lo, *hi] of blocks owning the columns that rows [r0, r1) read
 // (the self column of an empty slot excluded), where block k owns rows
 // base + [k R, (k+1) R) of the columns' range; this block if there is none.
@@ -269,9 +193,6 @@ struct PersistArgs {
     CgState* st;
     int stall;          // test hook: 1 makes every barrier wait for one arrival too many
     double dmin;        // single-reduction loops: smallest diagonal entry (stop-test gate)
-    double* z;          // IC(0): preconditioned residual
-    const double* dinv; // IC(0): inverse pivots
-    const double* dpiv; // IC(0), Eisenstat form: the pivots themselves
 };
 
 // Rows per block for m rows over the grid: a multiple of 32.
@@ -673,329 +594,6 @@ __global__ void __launch_bounds__(kPBlock, 1) k_persistent_gear(PersistArgs P) {
     }
 }
 
-// FP64 IC(0)-PCG in a two-colour order by Eisenstat's form of the
-// preconditioned iteration (S. C. Eisenstat, SIAM J. Sci. Stat. Comput. 2,
-// 1981), in one persistent launch with the single-reduction recurrences.
-// With Ahat = [[I, E], [E^T, I]] (red rows [0, nR) first), the strictly lower
-// part Lt = [[0, 0], [E^T, 0]] and Dt = diag(I, D_B), the IC(0) factor is
-// M = (Dt + Lt) Dt^-1 (Dt + Lt^T).  PCG on Ahat with M gives the same
-// iterates as PCG on T = (Dt + Lt)^-1 Ahat (Dt + Lt^T)^-1 (symmetric) with
-// the diagonal preconditioner Dt, under xh = (Dt + Lt^T) y and
-// rh = (Dt + Lt)^-1 r; and from Ahat = (Dt + Lt) + (Dt + Lt^T) - (2 Dt - I),
-//   T = diag(I, D_B^-1 (I - E^T E) D_B^-1):
-// the red block is the identity, the black one needs E then E^T once.  One
-// pass over the matrix per iteration instead of two sweeps and an SpMV.  With
-// z = Dt rh (z_R = rh_R, z_B = D_B rh_B) and w = T z:
-//   w_R = z_R, and w_B = D_B^-1 (rh_B - E^T v) with v_R = E rh_B,
-// so in the recurrences s = T p stays equal to p on the red rows.  Per
-// iteration, from the state k_init64 left (y, r):
-//   all    p = z + beta p; s = w + beta s (black; red s = p);
-//          xh += alpha p; rh -= alpha s                                   | post 0
-//   red    [wait: black owners' rh_B] v_R = E rh_B; gamma_R = delta_R = rh_R.rh_R | post 1
-//   black  [wait: red owners' v] w_B = D_B^-1 (rh_B - E^T v), z_B = D_B rh_B;
-//          gamma_B = rh_B.z_B, delta_B = (rh_B - E^T v).rh_B
-//   one grid reduction: stop test, beta = gamma / gamma_old,
-//   alpha = gamma / (delta - beta gamma / alpha_old)
-// Pass 0 transforms instead of updating (xh_R = y_R + E y_B, rh_B =
-// D_B^-1 (r_B - E^T r_R), p = s = 0; xh_B = D_B y_B after the red rows have
-// read y_B); after the stop, y = (Dt + Lt^T)^-1 xh: y_B = D_B^-1 xh_B, then
-// y_R = xh_R - E y_B.  The stop test (every 8th pass) sums ||S r||^2 of the
-// true-form residual r = (Dt + Lt) rh: r_R = rh_R, r_B = z_B + E^T rh_R.
-// xh lives in P.y, rh in P.r, s_B in P.q, w_B in P.t, v_R and z_B in P.z.
-__global__ void __launch_bounds__(kPBlock, 1) k_persistent_ic0(PersistArgs P) {
-    __shared__ double rbuf[3][kPBlock];
-    // gamma, alpha, beta, ||S r||^2, 1/gamma, 1/(gamma alpha), stop threshold
-    __shared__ double sc[7];
-    __shared__ long long s_max_iter;
-    __shared__ int s_stop;        // 1 stop, 2 breakdown
-    __shared__ int s_dep[4];      // [lo, hi] owners for black rows, then for red rows
-    CgState* st = P.st;
-    if (st->done) return;                      // uniform: set before the launch
-    const int n = (int)P.n, nR = (int)P.nR, nB = n - nR;
-    const double* __restrict__ A = P.a;
-    const int32_t* __restrict__ C = P.col;
-    const double* __restrict__ dinv = P.dinv;
-    const double* __restrict__ dpiv = P.dpiv;
-    double* __restrict__ y = P.y;
-    double* __restrict__ r = P.r;
-    double* __restrict__ p = P.p;
-    double* __restrict__ s = P.q;
-    double* __restrict__ w = P.t;
-    double* __restrict__ z = P.z;
-    GridSync* gs = P.gs;
-    const int Rr = (int)rows_per_block(nR), Rb = (int)rows_per_block(nB);
-    const int rlo = (int)blockIdx.x * Rr < nR ? (int)blockIdx.x * Rr : nR;
-    const int rhi = rlo + Rr < nR ? rlo + Rr : nR;
-    const int blo = nR + ((int)blockIdx.x * Rb < nB ? (int)blockIdx.x * Rb : nB);
-    const int bhi = blo + Rb < n ? blo + Rb : n;
-    Epoch ep;
-    ep.target = P.stall ? 1ull : 0ull;
-    {
-        int lo_, hi_;
-        column_blocks(C, n, blo, bhi, 0, Rr, &lo_, &hi_);
-        if (threadIdx.x == 0) {
-            s_dep[0] = lo_;
-            s_dep[1] = hi_;
-        }
-        column_blocks(C, n, rlo, rhi, nR, Rb, &lo_, &hi_);
-        if (threadIdx.x == 0) {
-            s_dep[2] = lo_;
-            s_dep[3] = hi_;
-        }
-        __syncthreads();          // every thread reads s_dep below
-    }
-    if (threadIdx.x == 0) {
-        sc[0] = 0.0;
-        sc[1] = 0.0;
-        sc[2] = 0.0;
-        sc[3] = st->rnorm2;
-        sc[4] = 0.0;
-        sc[5] = 0.0;
-        sc[6] = st->thresh2;
-        s_max_iter = st->max_iter;
-        s_stop = 0;
-    }
-    bool ok;
-    bool halo;
-    {
-        const bool wide = s_dep[1] - s_dep[0] + 1 > kMaxDeps || s_dep[3] - s_dep[2] + 1 > kMaxDeps;
-        double wv[1] = {wide ? 1.0 : 0.0};
-        double none[1];
-        int any = 0;
-        ok = grid_allreduce<1, 1>(rbuf, wv, none, any, P.partials, gs, ep,
-                                  [](const double (&t)[1], double* o, int& f) {
-                                      o[0] = 0.0;
-                                      f = t[0] > 0.0 ? 1 : 0;
-                                  });
-        halo = any == 0;
-    }
-    auto post = [&](int slot, int ps) {
-        if (halo) halo_post(gs, (unsigned long long)(ps + 1), slot);
-    };
-    // wait for phase `slot` of this pass at the owners of the black rows'
-    // columns (which = 0) or of the red rows' columns (which = 1)
-    auto wait = [&](int slot, int ps, int which) -> bool {
-        if (!halo) return grid_barrier(gs, ep);
-        return halo_wait(gs, s_dep[2 * which], s_dep[2 * which + 1],
-                         (unsigned long long)(ps + 1), slot);
-    };
-    int pass = 0;              // passes 1, 2, ... each begin with an update: iterations = pass
-    for (; ok; ++pass) {
-        const bool upd = pass > 0;
-        const bool check = upd && (pass % 8) == 0;
-        const double alpha = sc[1], beta = sc[2];
-        double sums[3] = {0.0, 0.0, 0.0};
-        if (upd) {
-            // red: z = w = rh (old), so s = p: p = rh + beta p, xh += alpha p,
-            // rh -= alpha p
-            {
-                double re[2], pe[2], ye[2];
-                CPS_B_LOOP(rlo, rhi, 2, (re[u] = r[e], pe[u] = p[e], ye[u] = y[e]), {
-                    const double pn = fma(beta, pe[u], re[u]);
-                    p[e] = pn;
-                    y[e] = fma(alpha, pn, ye[u]);
-                    r[e] = fma(-alpha, pn, re[u]);
-                })
-            }
-            // black: p = z + beta p, s = w + beta s, xh += alpha p,
-            // rh -= alpha s
-            double pe[2], se[2], we[2], ze[2], re[2], ye[2];
-            CPS_B_LOOP(blo, bhi, 2,
-                (pe[u] = p[e], se[u] = s[e], we[u] = w[e], ze[u] = z[e], re[u] = r[e],
-                 ye[u] = y[e]),
-                {
-                    const double pn = fma(beta, pe[u], ze[u]);
-                    const double sn = fma(beta, se[u], we[u]);
-                    p[e] = pn;
-                    s[e] = sn;
-                    y[e] = fma(alpha, pn, ye[u]);
-                    r[e] = fma(-alpha, sn, re[u]);
-                })
-        } else {
-            // xh_R = y_R + E y_B (y_B still the untransformed iterate)
-            for (int e = rlo + (int)threadIdx.x; e < rhi; e += kPBlock) {
-                double v = fma(A[e], y[C[e]], y[e]);
-                v = fma(A[n + e], y[C[n + e]], v);
-                v = fma(A[2 * n + e], y[C[2 * n + e]], v);
-                y[e] = v;
-                p[e] = 0.0;
-            }
-            // rh_B = D_B^-1 (r_B - E^T r_R) (r_R is never written here)
-            for (int e = blo + (int)threadIdx.x; e < bhi; e += kPBlock) {
-                double v = fma(-A[e], r[C[e]], r[e]);
-                v = fma(-A[n + e], r[C[n + e]], v);
-                v = fma(-A[2 * n + e], r[C[2 * n + e]], v);
-                r[e] = v * dinv[e];
-                p[e] = 0.0;
-                s[e] = 0.0;
-            }
-        }
-        post(0, pass);
-        // the red phase's first trip reads this block's rows up to the
-        // gathers: fetch them into L1 while waiting on the neighbours
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const int e = rlo + (int)threadIdx.x + u * kPBlock;
-            if (e < rhi) {
-                prefetch_l1(r + e);
-                prefetch_l1(A + e);
-                prefetch_l1(A + n + e);
-                prefetch_l1(A + 2 * n + e);
-                prefetch_l1(C + e);
-                prefetch_l1(C + n + e);
-                prefetch_l1(C + 2 * n + e);
-            }
-        }
-        if (!(ok = wait(0, pass, 1))) break;
-        // red: v_R = E rh_B; gamma_R = delta_R = rh_R.rh_R
-        {
-            double re[2], a0[2], a1[2], a2[2];
-            int c0[2], c1[2], c2[2];
-            CPS_B_LOOP(rlo, rhi, 2,
-                (re[u] = r[e], a0[u] = A[e], a1[u] = A[n + e], a2[u] = A[2 * n + e],
-                 c0[u] = C[e], c1[u] = C[n + e], c2[u] = C[2 * n + e]),
-                {
-                    double v = a0[u] * r[c0[u]];
-                    v = fma(a1[u], r[c1[u]], v);
-                    v = fma(a2[u], r[c2[u]], v);
-                    z[e] = v;
-                    sums[0] = fma(re[u], re[u], sums[0]);
-                    if (check) {
-                        const double tt = P.s[e] * re[u];
-                        sums[2] = fma(tt, tt, sums[2]);
-                    }
-                })
-        }
-        sums[1] = sums[0];
-        post(1, pass);
-        // likewise the black phase's first trip
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const int e = blo + (int)threadIdx.x + u * kPBlock;
-            if (e < bhi) {
-                prefetch_l1(r + e);
-                prefetch_l1(A + e);
-                prefetch_l1(A + n + e);
-                prefetch_l1(A + 2 * n + e);
-                prefetch_l1(C + e);
-                prefetch_l1(C + n + e);
-                prefetch_l1(C + 2 * n + e);
-                prefetch_l1(dpiv + e);
-                prefetch_l1(dinv + e);
-            }
-        }
-        if (!(ok = wait(1, pass, 0))) break;
-        // black: w_B = D_B^-1 (rh_B - E^T v), z_B = D_B rh_B; gamma_B, delta_B
-        {
-            double re[2], a0[2], a1[2], a2[2];
-            int c0[2], c1[2], c2[2];
-            CPS_B_LOOP(blo, bhi, 2,
-                (re[u] = r[e], a0[u] = A[e], a1[u] = A[n + e], a2[u] = A[2 * n + e],
-                 c0[u] = C[e], c1[u] = C[n + e], c2[u] = C[2 * n + e]),
-                {
-                    double t = fma(-a0[u], z[c0[u]], re[u]);
-                    t = fma(-a1[u], z[c1[u]], t);
-                    t = fma(-a2[u], z[c2[u]], t);
-                    const double d = dpiv[e];
-                    const double ze = d * re[u];
-                    w[e] = t * dinv[e];
-                    z[e] = ze;
-                    if (!upd) y[e] = d * y[e];        // xh_B = D_B y_B
-                    sums[0] = fma(re[u], ze, sums[0]);
-                    sums[1] = fma(t, re[u], sums[1]);
-                    if (check) {
-                        double rb = fma(a0[u], r[c0[u]], ze);
-                        rb = fma(a1[u], r[c1[u]], rb);
-                        rb = fma(a2[u], r[c2[u]], rb);
-                        const double tt = P.s[e] * rb;
-                        sums[2] = fma(tt, tt, sums[2]);
-                    }
-                })
-        }
-        // the next update's first trips read only this block's own rows,
-        // final now: fetch them into L1 during the reduction
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const int er = rlo + (int)threadIdx.x + u * kPBlock;
-            if (er < rhi) {
-                prefetch_l1(r + er);
-                prefetch_l1(p + er);
-                prefetch_l1(y + er);
-            }
-        }
-        auto step = [&](const double* t, bool chk, int& f) {
-            const double g = t[0], d = t[1];
-            bool halt = !(g > 0.0) || (upd && pass >= s_max_iter);   // exact, budget
-            if (chk) {
-                sc[3] = t[2];
-                if (t[2] <= sc[6]) halt = true;
-            }
-            f = halt ? 1 : 0;
-            if (!halt) {
-                const double den = fma(-(g * g), sc[5], d);
-                if (!(den > 0.0) || !isfinite(den)) {
-                    // pass 0: z.Tz <= 0, not SPD; later the recurrence's
-                    // difference lost its digits at the FP64 floor: stop,
-                    // and let the true residual decide
-                    f = upd ? 1 : 2;
-                } else {
-                    const double ig = 1.0 / g;
-                    sc[1] = g / den;
-                    sc[2] = g * sc[4];
-                    sc[4] = ig;
-                    sc[5] = den * ig * ig;
-                }
-            }
-            sc[0] = g;
-        };
-        double none[1];
-        int flag = 0;
-        if (check) {
-            double v3[3] = {sums[0], sums[1], sums[2]};
-            ok = grid_allreduce<3, 1>(rbuf, v3, none, flag, P.partials, gs, ep,
-                                      [&](const double (&t)[3], double* o, int& f) {
-                                          o[0] = 0.0;
-                                          step(t, true, f);
-                                      });
-        } else {
-            double v2[2] = {sums[0], sums[1]};
-            ok = grid_allreduce<2, 1>(rbuf, v2, none, flag, P.partials, gs, ep,
-                                      [&](const double (&t)[2], double* o, int& f) {
-                                          o[0] = 0.0;
-                                          step(t, false, f);
-                                      });
-        }
-        if (!ok) break;
-        if (flag) {
-            if (threadIdx.x == 0) s_stop = flag;
-            break;
-        }
-    }
-    if (ok) {
-        // y = (Dt + Lt^T)^-1 xh: y_B = D_B^-1 xh_B, then y_R = xh_R - E y_B
-        for (int e = blo + (int)threadIdx.x; e < bhi; e += kPBlock) y[e] *= dinv[e];
-        post(2, 0);
-        ok = wait(2, 0, 1);
-        if (ok) {
-            for (int e = rlo + (int)threadIdx.x; e < rhi; e += kPBlock) {
-                double v = fma(-A[e], y[C[e]], y[e]);
-                v = fma(-A[n + e], y[C[n + e]], v);
-                v = fma(-A[2 * n + e], y[C[2 * n + e]], v);
-                y[e] = v;
-            }
-        }
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        st->iter = pass;
-        st->rho = sc[0];
-        st->alpha = sc[1];
-        st->beta = sc[2];
-        st->rnorm2 = sc[3];
-        st->status = ok ? (s_stop == 2 ? CPS_ERR_NOT_SPD : CPS_OK) : CPS_ERR_TIMEOUT;
-        st->done = 2;
-    }
-}
-
 // Reduced system (two colours, colour order): CG on S = I - E^T E over the
 // black rows [nR, n) from the state k_black_init left.  Block b owns red rows
 // [b Rr, (b+1) Rr) and black rows nR + [b Rb, (b+1) Rb).
@@ -1161,219 +759,14 @@ __global__ void __launch_bounds__(kPBlock, 1) k_persistent_reduced(PersistArgs P
     }
 }
 
-// The reduced (black-cell Schur complement) CG with the single-reduction
-// (Chronopoulos-Gear) recurrences, from the state k_black_init left (y_B,
-// r_B, ||b||^2, ||S r||^2): s_B = Schur p_B and w_B = Schur r_B are carried,
-// so that both inner products of an iteration come from one Schur product:
-//   [wait for the halo] t_R = E r_B | post, [wait] w_B = r_B - E^T t_R,
-//   gamma = r.r, delta = w.r (every 8th: ||S r||^2) | one grid reduction:
-//   stop test; first pass alpha = gamma/delta, beta = 0; later beta =
-//   gamma/gamma_old, alpha = gamma/(delta - beta gamma/alpha_old) |
-//   p = r + beta p; s = w + beta s; y += alpha p; r -= alpha s | post
-// Two neighbour waits and one grid reduction per iteration (the textbook
-// reduced loop, k_persistent_reduced, has two reductions), at 9 FP64 FMAs a
-// black row plus 3 a red row.  s lives in q, w in z; p and s start at zero.
-__global__ void __launch_bounds__(kPBlock, 1) k_persistent_reduced1(PersistArgs P) {
-    __shared__ double rbuf[3][kPBlock];
-    // gamma, alpha, beta, ||S r||^2, 1/gamma, 1/(gamma alpha), stop threshold
-    __shared__ double sc[7];
-    __shared__ long long s_max_iter;
-    __shared__ int s_stop;
-    CgState* st = P.st;
-    if (st->done) return;                      // uniform: set before the launch
-    const int64_t n = P.n, nR = P.nR, nB = n - nR;
-    const double* __restrict__ A = P.a;
-    const int32_t* __restrict__ C = P.col;
-    double* __restrict__ p = P.p;
-    double* __restrict__ sv = P.q;
-    double* __restrict__ w = P.z;
-    double* __restrict__ r = P.r;
-    double* __restrict__ y = P.y;
-    double* __restrict__ t = P.t;
-    GridSync* gs = P.gs;
-    const int Rr = (int)rows_per_block(nR), Rb = (int)rows_per_block(nB);
-    const int rlo = (int)blockIdx.x * Rr < nR ? (int)blockIdx.x * Rr : (int)nR;
-    const int rhi = rlo + Rr < nR ? rlo + Rr : (int)nR;
-    const int blo = (int)nR + ((int)blockIdx.x * Rb < nB ? (int)blockIdx.x * Rb : (int)nB);
-    const int bhi = blo + Rb < n ? blo + Rb : (int)n;
-    if (threadIdx.x == 0) {
-        sc[0] = st->rho;
-        sc[1] = 0.0;
-        sc[2] = 0.0;
-        sc[3] = st->rnorm2;
-        sc[4] = 0.0;
-        sc[5] = 0.0;
-        sc[6] = st->thresh2;
-        s_max_iter = st->max_iter;
-        s_stop = 0;
-    }
-    bool ok = true;
-    Epoch ep;
-    ep.target = P.stall ? 1ull : 0ull;
-    // the red phase reads r at black rows, the black phase t at red rows
-    // (slot 0: r updated, slot 1: t computed), as in k_persistent_reduced
-    int dplo, dphi, dtlo, dthi;
-    column_blocks(C, n, rlo, rhi, nR, Rb, &dplo, &dphi);
-    column_blocks(C, n, blo, bhi, 0, Rr, &dtlo, &dthi);
-    bool halo;
-    {
-        const bool wide = dphi - dplo + 1 > kMaxDeps || dthi - dtlo + 1 > kMaxDeps;
-        double wv[1] = {wide ? 1.0 : 0.0};
-        double none[1];
-        int any = 0;
-        ok = grid_allreduce<1, 1>(rbuf, wv, none, any, P.partials, gs, ep,
-                                  [](const double (&tt)[1], double* o, int& f) {
-                                      o[0] = 0.0;
-                                      f = tt[0] > 0.0 ? 1 : 0;
-                                  });
-        halo = any == 0;
-    }
-    // the recurrences start from p = s = 0 (own rows only)
-    for (int64_t e = blo + threadIdx.x; e < bhi; e += kPBlock) {
-        p[e] = 0.0;
-        sv[e] = 0.0;
-    }
-    long long it = 0;
-    while (ok) {
-        if (halo && it > 0) {
-            ok = halo_wait(gs, dplo, dphi, (unsigned long long)it, 0);
-            if (!ok) break;
-        }
-        {
-            double a0[kU], a1[kU], a2[kU];
-            int32_t c0[kU], c1[kU], c2[kU];
-            CPS_B_LOOP(rlo, rhi, kU,
-                (a0[u] = A[e], a1[u] = A[n + e], a2[u] = A[2 * n + e], c0[u] = C[e],
-                 c1[u] = C[n + e], c2[u] = C[2 * n + e]),
-                {
-                    double acc = 0.0;
-                    if (c0[u] != (int32_t)e) acc = fma(a0[u], r[c0[u]], acc);
-                    if (c1[u] != (int32_t)e) acc = fma(a1[u], r[c1[u]], acc);
-                    if (c2[u] != (int32_t)e) acc = fma(a2[u], r[c2[u]], acc);
-                    t[e] = acc;
-                })
-        }
-        if (halo) {
-            halo_post(gs, (unsigned long long)(it + 1), 1);
-            ok = halo_wait(gs, dtlo, dthi, (unsigned long long)(it + 1), 1);
-        } else {
-            ok = grid_barrier(gs, ep);
-        }
-        if (!ok) break;
-        const bool check = ((it + 1) % 8) == 0;
-        double sums[3] = {0.0, 0.0, 0.0};
-        {
-            double re[kUGS], a0[kUGS], a1[kUGS], a2[kUGS];
-            int32_t c0[kUGS], c1[kUGS], c2[kUGS];
-            CPS_B_LOOP(blo, bhi, kUGS,
-                (re[u] = r[e], a0[u] = A[e], a1[u] = A[n + e], a2[u] = A[2 * n + e],
-                 c0[u] = C[e], c1[u] = C[n + e], c2[u] = C[2 * n + e]),
-                {
-                    double v = re[u];
-                    if (c0[u] != (int32_t)e) v = fma(-a0[u], t[c0[u]], v);
-                    if (c1[u] != (int32_t)e) v = fma(-a1[u], t[c1[u]], v);
-                    if (c2[u] != (int32_t)e) v = fma(-a2[u], t[c2[u]], v);
-                    w[e] = v;
-                    sums[0] = fma(re[u], re[u], sums[0]);
-                    sums[1] = fma(v, re[u], sums[1]);
-                    if (check) {
-                        const double tt = P.s[e] * re[u];
-                        sums[2] = fma(tt, tt, sums[2]);
-                    }
-                })
-        }
-        // thread 0, from the totals: the stop test and the step scalars (1/gamma
-        // and 1/(gamma alpha) carried, one divide on the critical path)
-        const long long it0 = it;
-        auto post = [&](const double* tt, bool chk, int& f) {
-            const double g = tt[0], d = tt[1];
-            bool halt = !(g > 0.0) || it0 >= s_max_iter;       // exact solution, budget
-            if (chk) {
-                sc[3] = tt[2];
-                if (tt[2] <= sc[6]) halt = true;
-            }
-            f = halt ? 1 : 0;
-            if (!halt) {
-                const double den = it0 == 0 ? d : fma(-(g * g), sc[5], d);
-                if (!(den > 0.0) || !isfinite(den)) {
-                    // on the run's first pass p.Sp <= 0: not SPD; later, the
-                    // recurrence's difference lost its digits at the FP64
-                    // floor: stop, and let the true residual decide
-                    f = it0 > 0 ? 1 : 2;
-                } else {
-                    const double ig = 1.0 / g;
-                    sc[1] = g / den;
-                    sc[2] = it0 == 0 ? 0.0 : g * sc[4];
-                    sc[4] = ig;
-                    sc[5] = den * ig * ig;
-                }
-            }
-            sc[0] = g;
-        };
-        double none[1];
-        int flag = 0;
-        if (check) {
-            double v3[3] = {sums[0], sums[1], sums[2]};
-            ok = grid_allreduce<3, 1>(rbuf, v3, none, flag, P.partials, gs, ep,
-                                      [&](const double (&tt)[3], double* o, int& f) {
-                                          o[0] = 0.0;
-                                          post(tt, true, f);
-                                      });
-        } else {
-            double v2[2] = {sums[0], sums[1]};
-            ok = grid_allreduce<2, 1>(rbuf, v2, none, flag, P.partials, gs, ep,
-                                      [&](const double (&tt)[2], double* o, int& f) {
-                                          o[0] = 0.0;
-                                          post(tt, false, f);
-                                      });
-        }
-        if (!ok) break;
-        if (flag) {
-            if (threadIdx.x == 0) s_stop = flag;
-            break;
-        }
-        {
-            const double alpha = sc[1], beta = sc[2];
-            double pe[kUG], se[kUG], we[kUG], re[kUG], ye[kUG];
-            CPS_B_LOOP(blo, bhi, kUG,
-                (pe[u] = p[e], se[u] = sv[e], we[u] = w[e], re[u] = r[e], ye[u] = y[e]),
-                {
-                    const double pn = fma(beta, pe[u], re[u]);
-                    const double sn = fma(beta, se[u], we[u]);
-                    p[e] = pn;
-                    sv[e] = sn;
-                    y[e] = fma(alpha, pn, ye[u]);
-                    r[e] = fma(-alpha, sn, re[u]);
-                })
-        }
-        ++it;
-        if (halo) {
-            halo_post(gs, (unsigned long long)it, 0);
-        } else {
-            ok = grid_barrier(gs, ep);
-        }
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        st->iter = it;
-        st->rho = sc[0];
-        st->rnorm2 = sc[3];
-        st->status = ok ? (s_stop == 2 ? CPS_ERR_NOT_SPD : CPS_OK) : CPS_ERR_TIMEOUT;
-        st->done = 2;
-    }
-}
-
 }  // namespace
 
 // The persistent kernel of a solve kind: 0 textbook Jacobi, 1 the reduced
-// system, 2 single-reduction Jacobi, 3 single-reduction IC(0) in a
-// two-colour order, 4 the reduced system with the single-reduction
-// recurrences.
+// system, 2 single-reduction Jacobi.
 static void (*persistent_kernel(int kind))(PersistArgs) {
     switch (kind) {
         case 1: return k_persistent_reduced;
         case 2: return k_persistent_gear;
-        case 3: return k_persistent_ic0;
-        case 4: return k_persistent_reduced1;
         default: return k_persistent_cg;
     }
 }
@@ -1393,10 +786,7 @@ int persistent_max_grid(cps_sys s, int reduced) {
 
 // Launches the persistent solve (reduced = 0: Jacobi on all rows; 1: the
 // reduced system; 2: single-reduction Jacobi on all rows, after k_init64 and
-// k_gear_start, with s = A p in q and w = A r in t; 3: single-reduction IC(0)
-// in the two-colour order after k_init64, s in q, w in t, z and the inverse
-// pivots in z, dinv; 4: the reduced system with the single-reduction
-// recurrences after k_black_init, s in q, w in z, the red scratch in t)
+// k_gear_start, with s = A p in q and w = A r in t)
 // after the caller's init kernel; state in s->st.  With
 // win_bytes > 0 the launch carries a persisting L2 access-policy window over
 // [win_base, win_base + win_bytes) (the caller holds the set-aside).  grid:
@@ -1404,7 +794,7 @@ int persistent_max_grid(cps_sys s, int reduced) {
 int persistent_solve(cps_sys s, int reduced, const double* a, const int32_t* col,
                      const double* sc, double* y, double* r, double* p, double* q, double* t,
                      int64_t n, int64_t nR, const void* win_base, size_t win_bytes, int grid,
-                     cudaStream_t stream, double* z, const double* dinv, const double* dpiv) {
+                     cudaStream_t stream) {
     if (!s->gsync) {
         cudaError_t e = cudaMalloc((void**)&s->gsync, sizeof(GridSync));
         if (e != cudaSuccess) {
@@ -1432,8 +822,7 @@ int persistent_solve(cps_sys s, int reduced, const double* a, const int32_t* col
     const int stall = s->inject == CPS_TEST_STALL_BARRIER ? 1 : 0;
     s->inject = 0;
     PersistArgs P{a, col, sc, y, r, p, q, t, n, nR, s->partials,
-                  reinterpret_cast<GridSync*>(s->gsync), s->st, stall, s->diag_min, z, dinv,
-                  dpiv};
+                  reinterpret_cast<GridSync*>(s->gsync), s->st, stall, s->diag_min};
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(G, 1, 1);
     cfg.blockDim = dim3(kPBlock, 1, 1);

@@ -19,7 +19,6 @@
 #include "cps_internal.cuh"
 
 #include <cstring>
-#include <vector>
 
 namespace cps {
 namespace {
@@ -328,20 +327,33 @@ __global__ void k_to_float(const double* __restrict__ v, int64_t m, float* __res
 
 }  // namespace
 
+static int alloc_order(cps_sys s) {
+    for (int32_t** p : {&s->perm, &s->iperm}) {
+        if (*p) continue;
+        cudaError_t e = cudaMalloc((void**)p, 4 * (size_t)s->nt);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            *p = nullptr;
+            cps::set_error(s->ctx, std::string("set_precond: cudaMalloc: ") + cudaGetErrorString(e));
+            return CPS_ERR_NOMEM;
+        }
+    }
+    return CPS_OK;
+}
+
 static int alloc_ic0(cps_sys s) {
-    if (s->pa) return CPS_OK;
     const int64_t n = s->nt;
     struct {
         void** p;
         size_t bytes;
-    } req[] = {{(void**)&s->perm, 4 * (size_t)n},       {(void**)&s->iperm, 4 * (size_t)n},
-               {(void**)&s->pa, 24 * (size_t)n},        {(void**)&s->pcol, 12 * (size_t)n},
+    } req[] = {{(void**)&s->pa, 24 * (size_t)n},        {(void**)&s->pcol, 12 * (size_t)n},
                {(void**)&s->pl, 24 * (size_t)n},        {(void**)&s->pdinv, 8 * (size_t)n},
                {(void**)&s->pdiag, 8 * (size_t)n},
                {(void**)&s->ps, 8 * (size_t)n},         {(void**)&s->pa32, 12 * (size_t)n},
                {(void**)&s->pl32, 12 * (size_t)n},      {(void**)&s->pdinv32, 4 * (size_t)n},
                {(void**)&s->ps32, 4 * (size_t)n}};
     for (auto& r : req) {
+        if (*r.p) continue;
         cudaError_t e = cudaMalloc(r.p, r.bytes);
         if (e != cudaSuccess) {
             cps::set_error(s->ctx, std::string("set_precond: cudaMalloc: ") + cudaGetErrorString(e));
@@ -351,7 +363,9 @@ static int alloc_ic0(cps_sys s) {
     return CPS_OK;
 }
 
-static int colour_cells(cps_sys s, int32_t* colour, cudaStream_t stream, int* ncol_out) {
+// Colours of the cells; with two_only, *ncol_out = -1 where two do not suffice.
+static int colour_cells(cps_sys s, int32_t* colour, bool two_only, cudaStream_t stream,
+                        int* ncol_out) {
     const int64_t n = s->nt;
     const int g = grid_for(s->ctx, n);
     constexpr int kRounds = 16;
@@ -370,7 +384,9 @@ static int colour_cells(cps_sys s, int32_t* colour, cudaStream_t stream, int* nc
     cudaMemcpyAsync(h, flags, sizeof(int) * 3, cudaMemcpyDeviceToHost, stream);
     if (cudaStreamSynchronize(stream) != cudaSuccess) rc = CPS_ERR_CUDA;
     const bool two = rc == CPS_OK && h[0] == 0 && h[1] == 0 && h[2] == 0;
-    if (rc == CPS_OK && !two) {
+    if (rc == CPS_OK && !two && two_only) {
+        *ncol_out = -1;
+    } else if (rc == CPS_OK && !two) {
         // Jones-Plassmann: at most (max degree + 1) = 4 colours.
         cudaMemsetAsync(colour, 0xFF, sizeof(int32_t) * n, stream);
         for (int64_t round = 0; round <= n; round += kRounds) {
@@ -385,7 +401,7 @@ static int colour_cells(cps_sys s, int32_t* colour, cudaStream_t stream, int* nc
             if (h[4 + kRounds - 1] == 0) break;
         }
     }
-    if (rc == CPS_OK) {
+    if (rc == CPS_OK && (two || !two_only)) {
         k_colour_max<<<g, kBlock, 0, stream>>>(colour, n, flags + 3);
         cudaMemcpyAsync(h + 3, flags + 3, sizeof(int), cudaMemcpyDeviceToHost, stream);
         if (cudaStreamSynchronize(stream) != cudaSuccess) rc = CPS_ERR_CUDA;
@@ -397,41 +413,24 @@ static int colour_cells(cps_sys s, int32_t* colour, cudaStream_t stream, int* nc
     return rc;
 }
 
-int precond_impl(cps_sys s, int precond, cudaStream_t stream) {
-    if (precond == CPS_PC_JACOBI) {
-        s->precond = precond;
-        return CPS_OK;
-    }
-    if (precond != CPS_PC_IC0 && precond != CPS_PC_REDUCED) {
-        cps::set_error(s->ctx, "set_precond: unknown preconditioner");
-        return CPS_ERR_ARG;
-    }
-    if (s->ncolours > 0) {   // ordered and factored already (the matrix is fixed)
-        if (precond == CPS_PC_REDUCED && s->ncolours != 2) {
-            cps::set_error(s->ctx, "set_precond: the cell graph is not two-colourable");
-            return CPS_ERR_ARG;
-        }
-        s->precond = precond;
-        return CPS_OK;
-    }
-    int rc = alloc_ic0(s);
+// Orders the cells colour by colour: perm, iperm, colour_start, ncolours (-1
+// with two_only where two colours do not suffice).
+static int order_cells(cps_sys s, bool two_only, cudaStream_t stream) {
+    if (s->ncolours > 0 || (two_only && s->ncolours < 0)) return CPS_OK;
+    int rc = alloc_order(s);
     if (rc) return rc;
     const int64_t n = s->nt;
-    const int g = grid_for(s->ctx, n);
     int32_t* colour = nullptr;
     int* counts = nullptr;
     long long* offsets = nullptr;
-    int* err = nullptr;
     CPS_CUDA_TRY(s->ctx, cudaMallocAsync((void**)&colour, sizeof(int32_t) * n, stream));
-    CPS_CUDA_TRY(s->ctx, cudaMallocAsync((void**)&err, sizeof(int), stream));
-    CPS_CUDA_TRY(s->ctx, cudaMemsetAsync(err, 0, sizeof(int), stream));
     int ncol = 0;
-    rc = colour_cells(s, colour, stream, &ncol);
-    if (rc == CPS_OK && (ncol < 1 || ncol > kMaxColours)) {
+    rc = colour_cells(s, colour, two_only, stream, &ncol);
+    if (rc == CPS_OK && (ncol == 0 || ncol > kMaxColours)) {
         cps::set_error(s->ctx, "set_precond: too many colours");
         rc = CPS_ERR_ARG;
     }
-    if (rc == CPS_OK) {
+    if (rc == CPS_OK && ncol > 0) {
         const int64_t nblk = (n + kBlock - 1) / kBlock;
         const int64_t m = (int64_t)ncol * nblk;
         cudaError_t ce = cudaMallocAsync((void**)&counts, sizeof(int) * m, stream);
@@ -443,47 +442,82 @@ int precond_impl(cps_sys s, int precond, cudaStream_t stream) {
             k_scan<<<1, 1024, 0, stream>>>(counts, m, offsets);
             k_colour_scatter<<<(unsigned)nblk, kBlock, 0, stream>>>(colour, n, ncol, nblk, offsets,
                                                                   s->perm, s->iperm);
-            std::vector<long long> starts(ncol);
+            long long starts[kMaxColours];
             for (int c = 0; c < ncol; ++c)
                 cudaMemcpyAsync(&starts[c], offsets + (int64_t)c * nblk, sizeof(long long),
                                 cudaMemcpyDeviceToHost, stream);
-            k_permute_matrix<<<g, kBlock, 0, stream>>>(s->a, s->col, s->s, s->perm, s->iperm, n,
-                                                       s->pa, s->pcol, s->ps, s->pa32, s->ps32);
             if (cudaStreamSynchronize(stream) != cudaSuccess || cudaGetLastError() != cudaSuccess) {
                 rc = CPS_ERR_CUDA;
             } else {
                 for (int c = 0; c < ncol; ++c) s->colour_start[c] = starts[c];
                 s->colour_start[ncol] = n;
-                for (int c = 0; c < ncol; ++c)
-                    k_ic0_factor<<<g, kBlock, 0, stream>>>(s->pa, s->pcol, n, s->colour_start[c],
-                                                           s->colour_start[c + 1], s->pl, s->pdinv,
-                                                           s->pdiag, err);
-                k_ic0_upper<<<g, kBlock, 0, stream>>>(s->pcol, n, s->pl, s->pdinv, s->pl32,
-                                                      s->pdinv32);
-                k_to_float<<<grid_for(s->ctx, 3 * n), kBlock, 0, stream>>>(s->pl, 3 * n, s->pl32);
-                int herr = 0;
-                cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, stream);
-                if (cudaStreamSynchronize(stream) != cudaSuccess || cudaGetLastError() != cudaSuccess)
-                    rc = CPS_ERR_CUDA;
-                else if (herr) {
-                    cps::set_error(s->ctx, "set_precond: IC(0) pivot <= 0");
-                    rc = herr;
-                }
             }
         }
     }
     if (counts) cudaFreeAsync(counts, stream);
     if (offsets) cudaFreeAsync(offsets, stream);
     cudaFreeAsync(colour, stream);
+    if (rc == CPS_OK) s->ncolours = ncol;
+    return rc;
+}
+
+// The two-colour order of the cells for the two-cyclic solves; *ok false where
+// the graph has none.
+int two_colour_order(cps_sys s, cudaStream_t stream, bool* ok) {
+    const int rc = order_cells(s, true, stream);
+    *ok = rc == CPS_OK && s->ncolours == 2;
+    return rc;
+}
+
+// Permutes the matrix into the colour order and factors it.
+static int factor_ic0(cps_sys s, cudaStream_t stream) {
+    int rc = alloc_ic0(s);
+    if (rc) return rc;
+    const int64_t n = s->nt;
+    const int g = grid_for(s->ctx, n);
+    int* err = nullptr;
+    CPS_CUDA_TRY(s->ctx, cudaMallocAsync((void**)&err, sizeof(int), stream));
+    cudaMemsetAsync(err, 0, sizeof(int), stream);
+    k_permute_matrix<<<g, kBlock, 0, stream>>>(s->a, s->col, s->s, s->perm, s->iperm, n, s->pa,
+                                               s->pcol, s->ps, s->pa32, s->ps32);
+    for (int c = 0; c < s->ncolours; ++c)
+        k_ic0_factor<<<g, kBlock, 0, stream>>>(s->pa, s->pcol, n, s->colour_start[c],
+                                               s->colour_start[c + 1], s->pl, s->pdinv, s->pdiag,
+                                               err);
+    k_ic0_upper<<<g, kBlock, 0, stream>>>(s->pcol, n, s->pl, s->pdinv, s->pl32, s->pdinv32);
+    k_to_float<<<grid_for(s->ctx, 3 * n), kBlock, 0, stream>>>(s->pl, 3 * n, s->pl32);
+    int herr = 0;
+    cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, stream);
     cudaFreeAsync(err, stream);
-    cudaStreamSynchronize(stream);
-    if (rc != CPS_OK) {
-        if (s->ctx->last_error.empty()) cps::set_error(s->ctx, "set_precond: IC(0) set-up failed");
-        return rc;
+    if (cudaStreamSynchronize(stream) != cudaSuccess || cudaGetLastError() != cudaSuccess)
+        return CPS_ERR_CUDA;
+    if (herr) {
+        cps::set_error(s->ctx, "set_precond: IC(0) pivot <= 0");
+        return herr;
     }
-    s->ncolours = ncol;
-    if (precond == CPS_PC_REDUCED && ncol != 2) {
-        s->precond = CPS_PC_JACOBI;
+    s->factored = true;
+    return CPS_OK;
+}
+
+int precond_impl(cps_sys s, int precond, cudaStream_t stream) {
+    if (precond == CPS_PC_JACOBI) {
+        s->precond = precond;
+        return CPS_OK;
+    }
+    if (precond != CPS_PC_IC0 && precond != CPS_PC_REDUCED) {
+        cps::set_error(s->ctx, "set_precond: unknown preconditioner");
+        return CPS_ERR_ARG;
+    }
+    if (!s->factored) {          // the matrix is fixed: ordered and factored once
+        int rc = order_cells(s, false, stream);
+        if (rc == CPS_OK) rc = factor_ic0(s, stream);
+        if (rc != CPS_OK) {
+            if (s->ctx->last_error.empty()) cps::set_error(s->ctx, "set_precond: IC(0) set-up failed");
+            return rc;
+        }
+        if (precond == CPS_PC_REDUCED && s->ncolours != 2) s->precond = CPS_PC_JACOBI;
+    }
+    if (precond == CPS_PC_REDUCED && s->ncolours != 2) {
         cps::set_error(s->ctx, "set_precond: the cell graph is not two-colourable");
         return CPS_ERR_ARG;
     }

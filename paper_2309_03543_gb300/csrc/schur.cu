@@ -1,0 +1,795 @@
+// Two-cyclic solves: on a two-coloured cell graph (red rows R, black rows B;
+// no two neighbours share a colour) the scaled matrix is Ahat =
+// [[I, E], [E^T, I]], and the black cells' Schur complement S = I - E^T E is
+// formed explicitly, one row per black cell: a diagonal and at most six
+// neighbours (two behind each of its three red cells).
+//
+//   - CPS_PC_REDUCED: CG on S.
+//   - FP64 Jacobi: started with a zero red residual (y_R = bhat_R - E y_B),
+//     every second Jacobi-PCG iteration of the full system leaves the red
+//     residual zero again, and two of them are one CG iteration on S (J. K.
+//     Reid, SIAM J. Numer. Anal. 9, 1972: systems with Property A).  So the
+//     Jacobi solve runs on S too, counting two iterations per step.
+//   - IC(0) in the two-colour order: from a zero red residual, PCG with M =
+//     (D + L) D^-1 (D + L^T), D = diag(I, diag S), keeps it zero, and is CG on
+//     S with the preconditioner diag(S): on D_B^-1/2 S D_B^-1/2 (unit
+//     diagonal), the rows scaled here when that preconditioner is selected.
+//
+// Why explicit rows.  Applied as t = E r, w = r - E^T t, the product needs
+// two neighbour waits an iteration, 36 B of matrix per red and per black row
+// and a round trip of t: 88 B and 6 FP64 FMAs per black row.  A row of S is 80
+// B and 7 FMAs and needs one wait.  The vectors halve against the full
+// system's.
+#include "cps_internal.cuh"
+#include "exact_sum.cuh"
+#include "grid_sync.cuh"
+
+#include <cmath>
+#include <cstddef>
+
+namespace cps {
+namespace {
+
+constexpr int kSlots = 6;
+
+// Row k of S (black cell perm[nR + k]) from the red rows' entries only, so
+// that S is symmetric to the last bit: red row c with entries v_i at black
+// cells i gives S_ij -= v_i v_j.
+__global__ void k_schur_rows(const double* __restrict__ a, const int32_t* __restrict__ col,
+                             const double* __restrict__ s, const int32_t* __restrict__ perm,
+                             const int32_t* __restrict__ iperm, int64_t nt, int64_t nR, int nB,
+                             int64_t ld, double* __restrict__ v, int32_t* __restrict__ c6,
+                             double* __restrict__ d, double* __restrict__ wt) {
+    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < nB;
+         k += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t e = perm[nR + k];
+        double diag = 1.0, val[kSlots];
+        int32_t idx[kSlots];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const int32_t c = col[j * nt + e];
+            double own = 0.0, o[3];
+            int32_t oc[3];
+#pragma unroll
+            for (int m = 0; m < 3; ++m) {
+                oc[m] = col[m * nt + c];
+                o[m] = a[m * nt + c];
+            }
+            bool seen = c == e;                   // unused slot: nothing behind it
+#pragma unroll
+            for (int m = 0; m < 3; ++m)
+                if (!seen && oc[m] == e) {
+                    own = o[m];
+                    oc[m] = -1;
+                    seen = true;
+                }
+            if (c == e) own = 0.0;
+            diag = fma(-own, own, diag);
+            int f = 2 * j;
+            val[f] = val[f + 1] = 0.0;
+            idx[f] = idx[f + 1] = (int32_t)k;
+#pragma unroll
+            for (int m = 0; m < 3; ++m) {
+                if (c == e || oc[m] < 0 || oc[m] == c) continue;
+                if (f < 2 * j + 2) {
+                    // both slots are static registers: select by value
+                    if (f == 2 * j) {
+                        val[2 * j] = -(own * o[m]);
+                        idx[2 * j] = (int32_t)(iperm[oc[m]] - nR);
+                    } else {
+                        val[2 * j + 1] = -(own * o[m]);
+                        idx[2 * j + 1] = (int32_t)(iperm[oc[m]] - nR);
+                    }
+                    ++f;
+                }
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < kSlots; ++j) {
+            v[j * ld + k] = val[j];
+            c6[j * ld + k] = idx[j];
+        }
+        d[k] = diag;
+        wt[k] = s[e];
+    }
+}
+
+// Rows of D^-1/2 S D^-1/2 (D = diag S) in place; dsc = D^-1/2, and the weight
+// of the stop test becomes s D^1/2 (the true residual of a black row).
+__global__ void k_schur_scale(double* __restrict__ v, const int32_t* __restrict__ c6,
+                              const double* __restrict__ d, int nB, int64_t ld,
+                              double* __restrict__ dsc, double* __restrict__ wt) {
+    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < nB;
+         k += (int64_t)gridDim.x * blockDim.x) {
+        const double sq = sqrt(d[k]);
+#pragma unroll
+        for (int j = 0; j < kSlots; ++j) {
+            const double w = v[j * ld + k];
+            if (w != 0.0) v[j * ld + k] = w / (sq * sqrt(d[c6[j * ld + k]]));
+        }
+        dsc[k] = 1.0 / sq;
+        wt[k] *= sq;
+    }
+}
+
+// Red cells (mesh order): y_R = b / s - E (S x)_B.
+__global__ void __launch_bounds__(kBlock) k_tc_red(const double* __restrict__ b,
+                                                   const double* __restrict__ x,
+                                                   const double* __restrict__ s,
+                                                   const double* __restrict__ a,
+                                                   const int32_t* __restrict__ col,
+                                                   const int32_t* __restrict__ perm, int64_t nt,
+                                                   int64_t nR, double* __restrict__ y) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nR;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t e = perm[i];
+        double acc = b[e] / s[e];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const int32_t c = col[j * nt + e];
+            if (c != e) acc = fma(-a[j * nt + e], s[c] * x[c], acc);
+        }
+        y[e] = acc;
+    }
+}
+
+// Black rows: y_B = S x, r = bhat - y_B - E^T y_R (scaled by dsc where the
+// rows are), and the run's state: rho = r.r, ||b||^2 over all cells, ||S r||^2.
+__global__ void __launch_bounds__(kBlock) k_tc_init(
+    const double* __restrict__ b, const double* __restrict__ x, const double* __restrict__ s,
+    const double* __restrict__ a, const int32_t* __restrict__ col,
+    const int32_t* __restrict__ perm, const double* __restrict__ dsc,
+    const double* __restrict__ y, int64_t nt, int64_t nR, double* __restrict__ yb,
+    double* __restrict__ r, double rtol, long long budget, double* partials, CgState* st) {
+    double rr = 0.0, bb = 0.0, nn = 0.0;
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nt;
+         e += (int64_t)gridDim.x * blockDim.x) {
+        const double be = b[e];
+        bb = fma(be, be, bb);
+    }
+    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < nt - nR;
+         k += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t e = perm[nR + k];
+        const double se = s[e];
+        const double ye = se * x[e];
+        double ay = ye;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const int32_t c = col[j * nt + e];
+            if (c != e) ay = fma(a[j * nt + e], y[c], ay);
+        }
+        double re = b[e] / se - ay;
+        const double t = se * re;
+        nn = fma(t, t, nn);
+        if (dsc) {
+            const double q = dsc[k];
+            yb[k] = ye / q;
+            re *= q;
+        } else {
+            yb[k] = ye;
+        }
+        r[k] = re;
+        rr = fma(re, re, rr);
+    }
+    double t[3] = {rr, bb, nn};
+    if (grid_sum<3>(t, partials, &st->arrive[2]) && threadIdx.x == 0) {
+        st->rho = t[0];
+        st->bnorm2 = t[1];
+        st->thresh2 = rtol * rtol * t[1];
+        st->rnorm2 = t[2];
+        st->alpha = 0.0;
+        st->beta = 0.0;
+        st->gamma = 0.0;
+        st->iter = 0;
+        st->max_iter = budget;
+        st->status = CPS_OK;
+        st->done = (t[1] == 0.0 || t[2] <= st->thresh2 || budget <= 0) ? 2 : 0;
+    }
+}
+
+// y of the whole system (mesh order) from the black solution:
+// y_R = b / s - E y_B.
+__global__ void __launch_bounds__(kBlock) k_tc_back(const double* __restrict__ b,
+                                                    const double* __restrict__ yb,
+                                                    const double* __restrict__ dsc,
+                                                    const double* __restrict__ s,
+                                                    const double* __restrict__ a,
+                                                    const int32_t* __restrict__ col,
+                                                    const int32_t* __restrict__ iperm, int64_t nt,
+                                                    int64_t nR, double* __restrict__ y) {
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nt;
+         e += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t k = (int64_t)iperm[e] - nR;
+        if (k >= 0) {
+            y[e] = dsc ? yb[k] * dsc[k] : yb[k];
+            continue;
+        }
+        double acc = b[e] / s[e];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const int32_t c = col[j * nt + e];
+            if (c == (int32_t)e) continue;
+            const int64_t kc = (int64_t)iperm[c] - nR;
+            acc = fma(-a[j * nt + e], dsc ? yb[kc] * dsc[kc] : yb[kc], acc);
+        }
+        y[e] = acc;
+    }
+}
+
+// ------------------------------------------------------ the persistent loop
+
+constexpr int kGridMax = 160;        // blocks (one per SM): a lane polls at most five slots
+constexpr int kPollPer = kGridMax / 32;
+constexpr int kSchurDeps = 32;       // owners a block's halo may span (one per lane)
+constexpr int kQuant = 2;             // quantities of one reduction at most
+constexpr int kSlotStride = 16;       // words of a slot: a 128-byte line per block
+constexpr size_t kSlotWords = 4 * (size_t)kGridMax * kSlotStride;   // [quantities][buffer][block]
+
+struct SchurArgs {
+    const double* v;
+    const int32_t* c;
+    const double* d;
+    const double* wt;
+    double* r;
+    double* w;
+    double* p;
+    double* s;
+    double* y;
+    int n;
+    int64_t ld;
+    unsigned long long* pb;     // kSlotWords tagged block totals, zero at launch
+    GridSync* gs;
+    CgState* st;
+    int stall;                  // test hook: every reduction waits for a value that never comes
+    double dmin;                // smallest diagonal of A (stop-test gate), 0 for none
+};
+
+__device__ __forceinline__ unsigned long long ld_relaxed(const unsigned long long* p) {
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ void st_relaxed(unsigned long long* p, unsigned long long v) {
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+
+// T 2^(E - 1075 + h) as a double, |T| < 2^61, rounded half up, in integer
+// arithmetic (NaN if the set held an infinity or NaN, infinity on overflow,
+// zero below the normal range): every warp converts its sum, and the FP64 pipe
+// takes one warp instruction in 17 cycles.
+__device__ __forceinline__ double fixed_bits(long long T, int E, int h) {
+    unsigned long long m = T < 0 ? 0ull - (unsigned long long)T : (unsigned long long)T;
+    int e = E + h;                                  // exponent of a 53-bit m
+    const int sh = 11 - __clzll((long long)m);      // m to 53 bits: right by sh (left if < 0)
+    e += sh;
+    if (sh > 0) {
+        m = (m + (1ull << (sh - 1))) >> sh;
+        if (m >> 53) {
+            m >>= 1;
+            ++e;
+        }
+    } else {
+        m <<= -sh & 63;
+    }
+    unsigned long long bits = ((unsigned long long)e << 52) | (m & 0xFFFFFFFFFFFFFull);
+    if (e >= 2047) bits = 0x7FF0000000000000ull;
+    if (T == 0 || e <= 0) bits = 0;
+    if (T < 0) bits |= 1ull << 63;
+    if (E >= 2047) bits = 0x7FF8000000000000ull;
+    return __longlong_as_double((long long)bits);
+}
+
+// Grid-wide sum of v[0..NV) over blocks of T threads: exact integer sums per
+// warp, per block and over the grid, each rounded to a double (trees of FP64
+// adds, 116 cycles a step and one warp instruction in 17 cycles, measured 0.8
+// to 1.3 us slower an iteration).  Each block stores its NV totals into its slot of one of two buffers, the last
+// mantissa bit replaced by the buffer's use count modulo 2.  Warp k of every
+// block polls the G slots of quantity k until all of them carry this use's bit,
+// and adds them: a total and its arrival travel in one word, so the reduction
+// costs one store and one load across the chip instead of a store, a counter
+// and a load.  A slot is a 128-byte line of its own: with 152 blocks polling,
+// an all-to-all of dense words takes 10000 cycles, of 32-byte sectors 5000, of
+// lines 2100 (a counter and a read of the totals 2850; one block summing and
+// writing the result back 2800; through clusters of 8 3400).  The two buffers
+// alternate, so a slot is rewritten only after every block has passed the
+// reduction in between, and every slot is written and polled at every use of
+// its buffer: reductions of one and of two quantities have buffers and counts
+// (ep) of their own.  Every block gets bit-identical totals.  Thread 0 then
+// runs post(totals), the others go on at the barrier that follows the call.
+// False (in s_fail, for all) if a wait ran out (about one second).
+template <int T, int NV, typename Post>
+__device__ __forceinline__ void tagged_allreduce(const double (&v)[NV], unsigned int& ep,
+                                                 const SchurArgs& P, int& s_fail, Post post) {
+    static_assert(NV >= 1 && NV <= kQuant, "quantities");
+    __shared__ double s_w[kQuant][32];
+    __shared__ double s_tot[kQuant];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int G = (int)gridDim.x;
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+        const int E = __reduce_max_sync(0xffffffffu, align_exp(v[k]));
+        const long long t = warp_sum_fixed<52>(align_fixed(v[k], E, 1));
+        if (lane == 0) s_w[k][warp] = fixed_bits(t, E, 1);
+    }
+    __syncthreads();
+    if (warp < NV) {
+        const unsigned long long tag = 1ull ^ ((ep >> 1) & 1ull);
+        unsigned long long* slots =
+            P.pb + ((NV - 1) * 2 + (size_t)(ep & 1u)) * kGridMax * kSlotStride + warp;
+        const double x = lane < T / 32 ? s_w[warp][lane] : 0.0;
+        const int E = __reduce_max_sync(0xffffffffu, align_exp(x));
+        const long long t = warp_sum_fixed<52>(align_fixed(x, E, 1));
+        if (lane == 0) {
+            const unsigned long long bits =
+                (unsigned long long)__double_as_longlong(fixed_bits(t, E, 1));
+            st_relaxed(slots + blockIdx.x * kSlotStride, (bits & ~1ull) | tag);
+        }
+        unsigned long long got[kPollPer];
+        unsigned int miss = 0;
+#pragma unroll
+        for (int q = 0; q < kPollPer; ++q) {
+            got[q] = 0;
+            if (lane + 32 * q < G) miss |= 1u << q;
+        }
+        const bool never = P.stall != 0 && lane == 0;
+        unsigned long long t0 = 0;
+        bool ok = true;
+        for (long long spins = 0;; ++spins) {
+#pragma unroll
+            for (int q = 0; q < kPollPer; ++q)
+                if (miss & (1u << q)) got[q] = ld_relaxed(slots + (lane + 32 * q) * kSlotStride);
+#pragma unroll
+            for (int q = 0; q < kPollPer; ++q)
+                if ((miss & (1u << q)) && (got[q] & 1ull) == tag && !never) miss &= ~(1u << q);
+            if (__all_sync(0xffffffffu, miss == 0)) break;
+            if ((spins & 255) == 255) {
+                const unsigned long long now = global_ns();
+                if (t0 == 0) t0 = now;
+                const bool out = now - t0 > kWaitNs || spins > kSpinCap ||
+                                 *(volatile int*)&P.gs->timeout != 0;
+                if (__any_sync(0xffffffffu, out)) {
+                    ok = false;
+                    break;
+                }
+            }
+        }
+        if (!ok) {
+            if (lane == 0) {
+                atomicExch(&P.gs->timeout, 1);
+                s_fail = 1;
+            }
+        } else {
+            int em = 1;
+#pragma unroll
+            for (int q = 0; q < kPollPer; ++q)
+                em = max(em, align_exp(__longlong_as_double((long long)got[q])));
+            const int Eg = __reduce_max_sync(0xffffffffu, em);
+            long long acc = 0;       // at most kPollPer values of 2^50 a lane
+#pragma unroll
+            for (int q = 0; q < kPollPer; ++q)
+                acc += align_fixed(__longlong_as_double((long long)got[q]), Eg, 3);
+            const long long tg = warp_sum_fixed<53>(acc);
+            if (lane == 0) s_tot[warp] = fixed_bits(tg, Eg, 3);
+        }
+        if (NV > 1) asm volatile("bar.sync 1, %0;" ::"n"(NV * 32) : "memory");
+        if (threadIdx.x == 0 && !s_fail) post(s_tot);
+    }
+    ++ep;
+}
+
+// Waits (one lane per owner) until the blocks [dlo, dhi] have posted `it`.
+__device__ __forceinline__ bool halo_wait_all(GridSync* gs, int dlo, int dhi,
+                                              unsigned long long it) {
+    __shared__ int s_ok;
+    if (threadIdx.x < 32) {
+        const int q = dlo + (int)threadIdx.x;
+        bool ok = true;
+        if (q <= dhi && q != (int)blockIdx.x) {
+            // (a timeout recorded elsewhere shows at the next reduction)
+            const unsigned long long* f = &gs->flag[q * kFlagStride];
+            unsigned long long t0 = 0;
+            for (long long spins = 1; ld_acquire(f) < it; ++spins) {
+                if ((spins & 255) != 0) continue;
+                const unsigned long long now = global_ns();
+                if (t0 == 0) t0 = now;
+                if (now - t0 > kWaitNs || spins > kSpinCap) {
+                    atomicExch(&gs->timeout, 1);
+                    ok = false;
+                    break;
+                }
+            }
+        }
+        ok = __all_sync(0xffffffffu, ok);
+        if (threadIdx.x == 0) s_ok = ok ? 1 : 0;
+    }
+    __syncthreads();
+    return s_ok != 0;
+}
+
+// CG on the rows of S with the single-reduction (Chronopoulos-Gear)
+// recurrences, from the state k_tc_init left (y_B, r, rho, ||b||^2):
+//   [wait for the neighbours' r] w = S r, gamma = r.r, delta = w.r (every 8th:
+//   ||wt r||^2) | one grid reduction: stop test, beta = gamma / gamma_old,
+//   alpha = gamma / (delta - beta gamma / alpha_old) |
+//   p = r + beta p; s = w + beta s; y += alpha p; r -= alpha s | post
+// 13 FP64 FMAs a row (12 with the unit diagonal).  A thread owns the same rows
+// in both phases, so what only the owner reads stays in its block's shared
+// memory across the iterations: RES vectors of p, s, y, w, r (a copy; the
+// neighbours gather r from global memory), and with MAT the rows themselves.
+// 1/gamma and 1/(gamma alpha) are carried (one thread divides beside the wait
+// for the neighbours), so one divide stays on the path the blocks wait on.
+template <int T, int RES, bool MAT, bool UNIT>
+__global__ void __launch_bounds__(T, 1) k_schur_cg(SchurArgs P) {
+    extern __shared__ double dyn[];
+    // alpha, beta, 1/gamma, 1/(gamma alpha), ||S r||^2, stop threshold, gamma
+    __shared__ double sc[7];
+    __shared__ int s_stop;          // 0 run, 1 stop, 2 breakdown
+    __shared__ int s_fail;          // a wait ran out
+    __shared__ long long s_max_iter;
+    __shared__ int s_lo, s_hi;
+    CgState* st = P.st;
+    if (st->done) return;                      // uniform: set before the launch
+    const int n = P.n;
+    const int64_t ld = P.ld;
+    const int R = (((n + (int)gridDim.x - 1) / (int)gridDim.x) + 31) & ~31;
+    const int lo = min((int)blockIdx.x * R, n);
+    const int cnt = min(lo + R, n) - lo;
+    const int tid = (int)threadIdx.x;
+    double* const rg = P.r + lo;
+    double* const p = RES >= 1 ? dyn : P.p + lo;
+    double* const sv = RES >= 2 ? dyn + R : P.s + lo;
+    double* const y = RES >= 3 ? dyn + 2 * R : P.y + lo;
+    double* const w = RES >= 4 ? dyn + 3 * R : P.w + lo;
+    double* const rl = RES >= 5 ? dyn + 4 * R : rg;
+    // resident rows: values [6][R], diagonal [R], columns [6][R]
+    double* const vm = dyn + RES * R;
+    double* const dm = vm + kSlots * R;
+    int32_t* const cm = reinterpret_cast<int32_t*>(dm + R);
+    const double* const vg = P.v + lo;
+    const double* const dg = P.d + lo;
+    const int32_t* const cg = P.c + lo;
+    GridSync* gs = P.gs;
+
+    if (tid == 0) {
+        s_lo = INT32_MAX;
+        s_hi = -1;
+        sc[2] = sc[3] = 0.0;
+        sc[4] = st->rnorm2;
+        sc[5] = st->thresh2;
+        sc[6] = st->rho;
+        s_stop = 0;
+        s_fail = 0;
+        s_max_iter = st->max_iter;
+    }
+    __syncthreads();
+    {
+        int cmin = INT32_MAX, cmax = -1;
+        for (int i = tid; i < cnt; i += T) {
+#pragma unroll
+            for (int j = 0; j < kSlots; ++j) {
+                const int c = cg[j * ld + i];
+                cmin = min(cmin, c);
+                cmax = max(cmax, c);
+                if (MAT) {
+                    cm[j * R + i] = c;
+                    vm[j * R + i] = vg[j * ld + i];
+                }
+            }
+            if (MAT && !UNIT) dm[i] = dg[i];
+            p[i] = 0.0;
+            sv[i] = 0.0;
+            if (RES >= 3) y[i] = P.y[lo + i];
+            if (RES >= 5) rl[i] = rg[i];
+        }
+        if (cmax >= 0) {
+            atomicMin(&s_lo, cmin / R);
+            atomicMax(&s_hi, cmax / R);
+        }
+    }
+    __syncthreads();
+    const int dlo = s_hi >= 0 ? s_lo : (int)blockIdx.x;
+    const int dhi = s_hi >= 0 ? s_hi : (int)blockIdx.x;
+    unsigned int ep1 = 0, ep2 = 0;  // reductions of one and of two quantities so far
+    unsigned long long bar = 0;     // arrivals of the grid barriers (no local halo)
+    bool halo;
+    {
+        const double wide[1] = {dhi - dlo + 1 > kSchurDeps ? 1.0 : 0.0};
+        tagged_allreduce<T>(wide, ep1, P, s_fail, [&](const double* t) { sc[0] = t[0]; });
+        __syncthreads();
+        halo = sc[0] == 0.0;
+        __syncthreads();
+    }
+    bool ok = s_fail == 0;
+    long long it = 0;
+    while (ok) {
+        double v[kSlots], dd = 1.0;
+        int c[kSlots];
+        auto load = [&](int i) {
+#pragma unroll
+            for (int j = 0; j < kSlots; ++j) {
+                c[j] = MAT ? cm[j * R + i] : cg[j * ld + i];
+                v[j] = MAT ? vm[j * R + i] : vg[j * ld + i];
+            }
+            if (!UNIT) dd = MAT ? dm[i] : dg[i];
+        };
+        // the first trip's rows are on their way while the neighbours finish
+        if (!MAT && tid < cnt) load(tid);
+        if (it > 0) {
+            if (halo) {
+                ok = halo_wait_all(gs, dlo, dhi, (unsigned long long)it);
+            } else {
+                bar += gridDim.x;
+                if (tid == 0) {
+                    red_release_add(&gs->count, 1ull);
+                    if (!wait_geq(&gs->count, bar, gs)) s_fail = 1;
+                }
+                __syncthreads();
+                ok = s_fail == 0;
+            }
+            if (!ok) break;
+        }
+        // the stop test every 8th iteration, and only once it can hold:
+        // ||S r||^2 >= min(diag A) r.r (gamma of the iteration before stands
+        // in for this one's, with a margin of 64)
+        const bool check = (it & 7) == 7 && P.dmin * sc[6] <= 64.0 * sc[5];
+        double sums[2] = {0.0, 0.0}, nn = 0.0;
+        for (int i = tid; i < cnt; i += T) {
+            if (MAT || i != tid) load(i);
+            double g[kSlots];
+#pragma unroll
+            for (int j = 0; j < kSlots; ++j) g[j] = P.r[c[j]];
+            const double re = rl[i];
+            double acc = UNIT ? re : dd * re;
+#pragma unroll
+            for (int j = 0; j < kSlots; ++j) acc = fma(v[j], g[j], acc);
+            w[i] = acc;
+            sums[0] = fma(re, re, sums[0]);
+            sums[1] = fma(acc, re, sums[1]);
+            if (check) {
+                const double t = P.wt[lo + i] * re;
+                nn = fma(t, t, nn);
+            }
+        }
+        const long long it0 = it;
+        if (check) {
+            const double one[1] = {nn};
+            tagged_allreduce<T>(one, ep1, P, s_fail, [&](const double* t) { sc[4] = t[0]; });
+            __syncthreads();
+            ok = s_fail == 0;
+            if (!ok) break;
+        }
+        tagged_allreduce<T>(sums, ep2, P, s_fail, [&](const double* t) {
+            const double g = t[0], dl = t[1];
+            int f = (!(g > 0.0) || it0 >= s_max_iter) ? 1 : 0;     // exact solution, budget
+            if (g != g) f = 2;                                     // NaN input
+            if (check && sc[4] <= sc[5]) f = 1;
+            if (!f) {
+                // from p = s = 0 on the run's first pass: den = delta, beta = 0
+                const double den = it0 == 0 ? dl : fma(-(g * g), sc[3], dl);
+                // on the first pass p.Sp <= 0: not SPD; later, the
+                // recurrence's difference lost its digits at the FP64 floor:
+                // stop, and let the true residual decide
+                if (!(den > 0.0) || !isfinite(den)) f = it0 > 0 ? 1 : 2;
+                sc[0] = g / den;
+                sc[1] = g * sc[2];
+                sc[3] = den;
+            }
+            sc[6] = g;
+            s_stop = f;
+        });
+        __syncthreads();
+        ok = s_fail == 0;
+        if (!ok || s_stop) break;
+        {
+            const double alpha = sc[0], beta = sc[1];
+#pragma unroll 2
+            for (int i = tid; i < cnt; i += T) {
+                const double re = rl[i];
+                const double pn = fma(beta, p[i], re);
+                const double sn = fma(beta, sv[i], w[i]);
+                const double rn = fma(-alpha, sn, re);
+                rg[i] = rn;
+                if (RES >= 5) rl[i] = rn;
+                p[i] = pn;
+                sv[i] = sn;
+                y[i] = fma(alpha, pn, y[i]);
+            }
+        }
+        ++it;
+        if (halo) halo_post(gs, (unsigned long long)it);
+        else __syncthreads();
+        if (tid == 32) {
+            // for the next iteration: off the path that the blocks wait on
+            const double ig = 1.0 / sc[6];
+            sc[2] = ig;
+            sc[3] = sc[3] * ig * ig;
+        }
+    }
+    if (RES >= 3)
+        for (int i = tid; i < cnt; i += T) P.y[lo + i] = y[i];
+    if (blockIdx.x == 0 && tid == 0) {
+        st->iter = it;
+        st->rho = sc[6];
+        st->rnorm2 = sc[4];
+        st->status = ok ? (s_stop == 2 ? CPS_ERR_NOT_SPD : CPS_OK) : CPS_ERR_TIMEOUT;
+        st->done = 2;
+    }
+}
+
+using SchurKernel = void (*)(SchurArgs);
+
+// The kernel whose resident part of R rows fits a block's shared memory, most
+// first, the dynamic bytes it takes and its threads.
+SchurKernel schur_kernel(int64_t R, bool unit, size_t limit, size_t* bytes, int* threads) {
+    struct Form {
+        int threads, res;
+        bool mat;
+        SchurKernel diag, unit;
+    };
+    // Resident rows leave few rows a thread: 512 threads synchronise faster.
+    // Streamed rows want 1024 threads' loads in flight.
+    static const Form forms[] = {
+        {512, 5, true, k_schur_cg<512, 5, true, false>, k_schur_cg<512, 5, true, true>},
+        {1024, 5, false, k_schur_cg<1024, 5, false, false>, k_schur_cg<1024, 5, false, true>},
+        {1024, 4, false, k_schur_cg<1024, 4, false, false>, k_schur_cg<1024, 4, false, true>},
+        {1024, 3, false, k_schur_cg<1024, 3, false, false>, k_schur_cg<1024, 3, false, true>},
+        {1024, 0, false, k_schur_cg<1024, 0, false, false>, k_schur_cg<1024, 0, false, true>}};
+    for (const Form& f : forms) {
+        const SchurKernel k = unit ? f.unit : f.diag;
+        cudaFuncAttributes at;
+        if (cudaFuncGetAttributes(&at, k) != cudaSuccess) return nullptr;
+        const size_t need = (size_t)R * (8 * f.res + (f.mat ? kSlots * 12 + 8 : 0));
+        if (need + at.sharedSizeBytes <= limit) {
+            *bytes = need;
+            *threads = f.threads;
+            return k;
+        }
+    }
+    return nullptr;
+}
+
+}  // namespace
+
+// Frees the Schur rows of a system.
+void free_schur(cps_sys s) {
+    if (s->sch.buf) cudaFree(s->sch.buf);
+    s->sch = SchurData{};
+}
+
+// The rows of S for this system's colour order (two colours), or of
+// D^-1/2 S D^-1/2 (scaled): built on first use and when the form changes.
+int schur_setup(cps_sys s, bool scaled, cudaStream_t stream) {
+    SchurData& h = s->sch;
+    const int64_t nR = s->colour_start[1], nB = s->nt - nR;
+    if (!h.buf) {
+        h.ld = (nB + 31) & ~(int64_t)31;
+        // r, w, p, s, y first: one contiguous range for an L2 window
+        const size_t bytes = (size_t)h.ld * (8 * (5 + kSlots + 3) + 4 * kSlots) +
+                             sizeof(unsigned long long) * kSlotWords;
+        cudaError_t e = cudaMalloc(&h.buf, bytes);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            h.buf = nullptr;
+            cps::set_error(s->ctx, "Schur rows: cudaMalloc failed");
+            return CPS_ERR_NOMEM;
+        }
+        double* q = static_cast<double*>(h.buf);
+        h.r = q;
+        h.w = q + h.ld;
+        h.p = q + 2 * h.ld;
+        h.s = q + 3 * h.ld;
+        h.y = q + 4 * h.ld;
+        h.v = q + 5 * h.ld;
+        h.d = q + (5 + kSlots) * h.ld;
+        h.wt = h.d + h.ld;
+        h.dsc = h.wt + h.ld;
+        h.pb = reinterpret_cast<unsigned long long*>(h.dsc + h.ld);
+        h.c = reinterpret_cast<int32_t*>(h.pb + kSlotWords);
+        h.nB = nB;
+        h.form = 0;
+    }
+    const int want = scaled ? 2 : 1;
+    if (h.form == want || nB == 0) return CPS_OK;
+    const int g = grid_for(s->ctx, nB);
+    k_schur_rows<<<g, kBlock, 0, stream>>>(s->a, s->col, s->s, s->perm, s->iperm, s->nt, nR,
+                                           (int)nB, h.ld, h.v, h.c, h.d, h.wt);
+    if (scaled) k_schur_scale<<<g, kBlock, 0, stream>>>(h.v, h.c, h.d, (int)nB, h.ld, h.dsc, h.wt);
+    CPS_CUDA_TRY(s->ctx, cudaGetLastError());
+    h.form = want;
+    return CPS_OK;
+}
+
+// Blocks of the persistent loop by default: one per SM, at least 256 rows each.
+int schur_grid(cps_sys s) {
+    int G = s->ctx->num_sms < kGridMax ? s->ctx->num_sms : kGridMax;
+    const int64_t most = (s->sch.nB + 255) / 256;
+    if (most < G) G = (int)(most < 1 ? 1 : most);
+    return G;
+}
+
+// A run's start from x (mesh order): y_R, y_B, r and the state in s->st.
+int schur_init(cps_sys s, const double* b, const double* x, double rtol, long long budget,
+               cudaStream_t stream) {
+    const SchurData& h = s->sch;
+    const int64_t nR = s->colour_start[1];
+    const double* dsc = h.form == 2 ? h.dsc : nullptr;
+    k_tc_red<<<s->grid, kBlock, 0, stream>>>(b, x, s->s, s->a, s->col, s->perm, s->nt, nR, s->wy);
+    k_tc_init<<<s->grid, kBlock, 0, stream>>>(b, x, s->s, s->a, s->col, s->perm, dsc, s->wy, s->nt,
+                                              nR, h.y, h.r, rtol, budget, s->partials, s->st);
+    CPS_CUDA_TRY(s->ctx, cudaGetLastError());
+    return CPS_OK;
+}
+
+// y of the whole system from the black solution, into s->wy.
+int schur_back(cps_sys s, const double* b, cudaStream_t stream) {
+    const SchurData& h = s->sch;
+    k_tc_back<<<s->grid, kBlock, 0, stream>>>(b, h.y, h.form == 2 ? h.dsc : nullptr, s->s, s->a,
+                                              s->col, s->iperm, s->nt, s->colour_start[1], s->wy);
+    CPS_CUDA_TRY(s->ctx, cudaGetLastError());
+    return CPS_OK;
+}
+
+// Bytes of the five vectors (the L2 window of the loop).
+size_t schur_window_bytes(cps_sys s) { return sizeof(double) * 5 * (size_t)s->sch.ld; }
+
+// The CG run from schur_init's state as one cooperative launch of `grid`
+// blocks (0: schur_grid), with the five vectors in persisting L2 if window
+// (the caller holds the set-aside).  State in s->st.
+int schur_run(cps_sys s, int grid, bool window, cudaStream_t stream) {
+    SchurData& h = s->sch;
+    if (!s->gsync) {
+        if (cudaMalloc((void**)&s->gsync, sizeof(GridSync)) != cudaSuccess) {
+            cudaGetLastError();
+            cps::set_error(s->ctx, "Schur solve: cudaMalloc failed");
+            return CPS_ERR_NOMEM;
+        }
+    }
+    int G = schur_grid(s);
+    if (grid > 0 && grid < G) G = grid;
+    const int64_t R = (((h.nB + G - 1) / G) + 31) & ~(int64_t)31;
+    size_t smem = 0;
+    int threads = 0;
+    SchurKernel kern = schur_kernel(R, h.form == 2, s->ctx->smem_optin, &smem, &threads);
+    if (!kern) {
+        cudaGetLastError();
+        cps::set_error(s->ctx, "Schur solve: no kernel for this device");
+        return CPS_ERR_CUDA;
+    }
+    CPS_CUDA_TRY(s->ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              (int)smem));
+    CPS_CUDA_TRY(s->ctx, cudaMemsetAsync(s->gsync, 0,
+                                         offsetof(GridSync, flag) +
+                                             sizeof(unsigned long long) * kFlagStride * G,
+                                         stream));
+    CPS_CUDA_TRY(s->ctx, cudaMemsetAsync(h.pb, 0, sizeof(unsigned long long) * kSlotWords, stream));
+    SchurArgs P{h.v, h.c, h.d, h.wt, h.r, h.w, h.p, h.s, h.y, (int)h.nB, h.ld, h.pb,
+                reinterpret_cast<GridSync*>(s->gsync), s->st,
+                s->inject == CPS_TEST_STALL_BARRIER ? 1 : 0, h.form == 2 ? 0.0 : s->diag_min};
+    s->inject = 0;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(G, 1, 1);
+    cfg.blockDim = dim3(threads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    at[1].id = cudaLaunchAttributeAccessPolicyWindow;
+    at[1].val.accessPolicyWindow.base_ptr = h.buf;
+    at[1].val.accessPolicyWindow.num_bytes = schur_window_bytes(s);
+    at[1].val.accessPolicyWindow.hitRatio = 1.0f;
+    at[1].val.accessPolicyWindow.hitProp = cudaAccessPropertyPersisting;
+    at[1].val.accessPolicyWindow.missProp = cudaAccessPropertyStreaming;
+    cfg.attrs = at;
+    cfg.numAttrs = window ? 2 : 1;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, kern, P);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        cps::set_error(s->ctx, std::string("Schur solve launch: ") + cudaGetErrorString(e));
+        return CPS_ERR_CUDA;
+    }
+    return CPS_OK;
+}
+
+}  // namespace cps
