@@ -118,7 +118,7 @@ BYTES_PER_ROW_STEP_SCHUR = 144
 def loop_name(tf: dict) -> str:
     """The FP64 Jacobi loop the tuner chose, with its kernels."""
     if tf.get("two_cyclic"):
-        return ("k_schur_cg (two-cyclic form of Jacobi-PCG: CG on the explicit Schur complement "
+        return ("k_resident_cg (two-cyclic form of Jacobi-PCG: CG on the explicit Schur complement "
                 "of one colour in one cooperative launch, two Jacobi iterations a step)")
     if tf.get("persistent_single_reduction"):
         kname = ("k_persistent_gear (whole Jacobi-PCG solve in one cooperative launch, "

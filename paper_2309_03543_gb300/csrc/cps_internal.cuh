@@ -199,7 +199,6 @@ struct SchurData {
     double* wt = nullptr;     // [ld] weight of the stop test
     double* dsc = nullptr;    // [ld] D^-1/2 (form 2)
     int32_t* c = nullptr;     // [6][ld] columns (= row for an unused slot)
-    unsigned long long* pb = nullptr;   // tagged block totals of the reductions
     int64_t ld = 0, nB = 0;
     int form = 0;             // 0 not built, 1 S, 2 D^-1/2 S D^-1/2
 };
@@ -405,11 +404,13 @@ int precond_impl(cps_sys sys, int precond, cudaStream_t stream);
 int two_colour_order(cps_sys s, cudaStream_t stream, bool* ok);
 void free_schur(cps_sys s);
 int schur_setup(cps_sys s, bool scaled, cudaStream_t stream);
-int schur_grid(cps_sys s);
 int schur_init(cps_sys s, const double* b, const double* x, double rtol, long long budget,
                cudaStream_t stream);
 int schur_back(cps_sys s, const double* b, cudaStream_t stream);
 int schur_run(cps_sys s, int grid, bool window, cudaStream_t stream);
+int ensure_gsync(cps_sys s);
+bool jacobi_resident(cps_sys s);
+int jacobi_run(cps_sys s, int grid, const void* win, size_t win_bytes, cudaStream_t stream);
 size_t schur_window_bytes(cps_sys s);
 int solve_impl(cps_sys sys, const double* b, double* x, double rtol, int64_t max_iter,
                int precision, cps_stats* stats, cudaStream_t stream);

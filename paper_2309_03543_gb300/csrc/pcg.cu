@@ -593,6 +593,19 @@ static void fill_stats(cps_stats* stats, int64_t iters, double rel, int status, 
 
 // ------------------------------------------------------------------ FP64
 
+// The persistent single-reduction Jacobi loop on all cells from the state
+// k_init64 left: with the vectors in shared memory where they fit (schur.cu),
+// else streamed (persistent.cu).
+static int persistent_1red(cps_sys s, const Run<double>& v, int grid, const void* base,
+                           size_t bytes, cudaStream_t stream) {
+    if (jacobi_resident(s)) return jacobi_run(s, grid, base, bytes, stream);
+    k_gear_start<<<s->grid, kBlock, 0, stream>>>(v.a, v.col, v.r, v.p1, v.p0, v.q, s->nt,
+                                                 s->partials, s->st);
+    CPS_CUDA_TRY(s->ctx, cudaGetLastError());
+    return persistent_solve(s, 2, v.a, v.col, v.s, v.y, v.r, v.p0, v.q, v.p1, s->nt, 0, base,
+                            bytes, grid, stream);
+}
+
 // For Jacobi solves, times a short run (64 iterations; 256 on large systems)
 // of each path that applies from x = 0 and keeps the fastest: graph-replayed
 // streaming kernels, the one-launch cluster solve (systems that fit one
@@ -651,16 +664,9 @@ static int choose_fp64_path(cps_sys s, const Run<double>& v, const double* b,
             if (big && l2_window_fits(s, 2)) cands[nc++] = {5, 2, 2, gi, 0};
         }
     }
-    if (!try_cluster) {
-        const int gmax = persistent_max_grid(s, 2);
-        int grids[2] = {gmax, (int)((s->nt + 8191) / 8192)};
-        for (int i = 0; i < 2; ++i) {
-            const int gi = grids[i] < 1 ? 1 : (grids[i] > gmax ? gmax : grids[i]);
-            if (gmax <= 0 || (i == 1 && gi == grids[0])) continue;
-            grids[i] = gi;
-            cands[nc++] = {8, 4, 0, gi, 0};
-            if (big && l2_window_fits(s, 3)) cands[nc++] = {9, 4, 3, gi, 0};
-        }
+    if (!try_cluster || s->nt > 4096) {
+        cands[nc++] = {8, 4, 0, 0, 0};
+        if (big && l2_window_fits(s, 3)) cands[nc++] = {9, 4, 3, 0, 0};
     }
     cudaEvent_t e0, e1;
     CPS_CUDA_TRY(s->ctx, cudaEventCreate(&e0));
@@ -688,13 +694,12 @@ static int choose_fp64_path(cps_sys s, const Run<double>& v, const double* b,
             if (c.path == 2 || c.path == 4) {
                 k_init64<<<s->grid, kBlock, 0, stream>>>(b, s->wx, v.s, v.a, v.col, s->nt, v.y, v.r,
                                                          v.p0, 0.0, probe, 1, s->partials, s->st);
-                if (c.path == 4)
-                    k_gear_start<<<s->grid, kBlock, 0, stream>>>(v.a, v.col, v.r, v.p1, v.p0, v.q,
-                                                                 s->nt, s->partials, s->st);
-                rc = persistent_solve(s, c.path == 4 ? 2 : 0, v.a, v.col, v.s, v.y, v.r, v.p0, v.q,
-                                      c.path == 4 ? v.p1 : nullptr, s->nt,
-                                      0, c.win ? l2_window_base(s, c.win) : nullptr,
-                                      c.win ? l2_window_bytes(s, c.win) : 0, c.grid, stream);
+                const void* base = c.win ? l2_window_base(s, c.win) : nullptr;
+                const size_t bytes = c.win ? l2_window_bytes(s, c.win) : 0;
+                rc = c.path == 4 ? persistent_1red(s, v, c.grid, base, bytes, stream)
+                                 : persistent_solve(s, 0, v.a, v.col, v.s, v.y, v.r, v.p0, v.q,
+                                                    nullptr, s->nt, 0, base, bytes, c.grid,
+                                                    stream);
                 if (rc == CPS_OK) rc = read_state(s, stream, &h);
                 if (rc == CPS_OK && h.status != CPS_OK) rc = CPS_ERR_ARG;   // not usable here
             } else if (c.path == 0 || c.path == 3) {
@@ -1084,17 +1089,13 @@ static int solve_fp64(cps_sys s, const double* b, double* x, double rtol, int64_
                                             budget, ic0 ? 0 : 1, s->partials, s->st);
         ++launches;
         if (persistent) {
-            if (pgear) {
-                k_gear_start<<<g, kBlock, 0, stream>>>(v.a, v.col, v.r, v.p1, v.p0, v.q, n,
-                                                       s->partials, s->st);
-                ++launches;
-            }
             // one launch runs to the stop (it returns at once if init stopped)
-            int rc = persistent_solve(s, pgear ? 2 : 0, v.a, v.col, v.s, v.y, v.r, v.p0, v.q,
-                                      pgear ? v.p1 : nullptr, n, 0,
-                                      window ? l2_window_base(s, window) : nullptr,
-                                      window ? l2_window_bytes(s, window) : 0,
-                                      s->tune[CPS_FP64].pgrid, stream);
+            const void* base = window ? l2_window_base(s, window) : nullptr;
+            const size_t bytes = window ? l2_window_bytes(s, window) : 0;
+            const int pg = s->tune[CPS_FP64].pgrid;
+            int rc = pgear ? persistent_1red(s, v, pg, base, bytes, stream)
+                           : persistent_solve(s, 0, v.a, v.col, v.s, v.y, v.r, v.p0, v.q, nullptr,
+                                              n, 0, base, bytes, pg, stream);
             if (rc) return rc;
             ++launches;
             rc = read_state(s, stream, &h);

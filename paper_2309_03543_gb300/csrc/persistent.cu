@@ -192,7 +192,7 @@ struct PersistArgs {
     GridSync* gs;
     CgState* st;
     int stall;          // test hook: 1 makes every barrier wait for one arrival too many
-    double dmin;        // single-reduction loops: smallest diagonal entry (stop-test gate)
+    double dmin;        // single-reduction loop: smallest diagonal entry (stop-test gate)
 };
 
 // Rows per block for m rows over the grid: a multiple of 32.
@@ -795,14 +795,8 @@ int persistent_solve(cps_sys s, int reduced, const double* a, const int32_t* col
                      const double* sc, double* y, double* r, double* p, double* q, double* t,
                      int64_t n, int64_t nR, const void* win_base, size_t win_bytes, int grid,
                      cudaStream_t stream) {
-    if (!s->gsync) {
-        cudaError_t e = cudaMalloc((void**)&s->gsync, sizeof(GridSync));
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            cps::set_error(s->ctx, "persistent: cudaMalloc failed");
-            return CPS_ERR_NOMEM;
-        }
-    }
+    const int rc = ensure_gsync(s);
+    if (rc) return rc;
     auto kern = persistent_kernel(reduced);
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kPBlock, 0) != cudaSuccess ||

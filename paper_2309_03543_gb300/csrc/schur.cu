@@ -220,7 +220,6 @@ __global__ void __launch_bounds__(kBlock) k_tc_back(const double* __restrict__ b
 
 constexpr int kGridMax = 160;        // blocks (one per SM): a lane polls at most five slots
 constexpr int kPollPer = kGridMax / 32;
-constexpr int kSchurDeps = 32;       // owners a block's halo may span (one per lane)
 constexpr int kQuant = 2;             // quantities of one reduction at most
 constexpr int kSlotStride = 16;       // words of a slot: a 128-byte line per block
 constexpr size_t kSlotWords = 4 * (size_t)kGridMax * kSlotStride;   // [quantities][buffer][block]
@@ -378,16 +377,15 @@ __device__ __forceinline__ void tagged_allreduce(const double (&v)[NV], unsigned
     ++ep;
 }
 
-// Waits (one lane per owner) until the blocks [dlo, dhi] have posted `it`.
-__device__ __forceinline__ bool halo_wait_all(GridSync* gs, int dlo, int dhi,
-                                              unsigned long long it) {
-    __shared__ int s_ok;
+// Waits until every block in the bit set dep has posted `it` (a lane per block
+// and word); a timeout recorded elsewhere shows at the next reduction.
+__device__ __forceinline__ void dep_wait(GridSync* gs, const unsigned int* dep,
+                                         unsigned long long it, int& s_fail) {
     if (threadIdx.x < 32) {
-        const int q = dlo + (int)threadIdx.x;
-        bool ok = true;
-        if (q <= dhi && q != (int)blockIdx.x) {
-            // (a timeout recorded elsewhere shows at the next reduction)
-            const unsigned long long* f = &gs->flag[q * kFlagStride];
+#pragma unroll
+        for (int q = 0; q < kPollPer; ++q) {
+            if (!((dep[q] >> threadIdx.x) & 1u)) continue;
+            const unsigned long long* f = &gs->flag[(32 * q + threadIdx.x) * kFlagStride];
             unsigned long long t0 = 0;
             for (long long spins = 1; ld_acquire(f) < it; ++spins) {
                 if ((spins & 255) != 0) continue;
@@ -395,65 +393,66 @@ __device__ __forceinline__ bool halo_wait_all(GridSync* gs, int dlo, int dhi,
                 if (t0 == 0) t0 = now;
                 if (now - t0 > kWaitNs || spins > kSpinCap) {
                     atomicExch(&gs->timeout, 1);
-                    ok = false;
+                    s_fail = 1;
                     break;
                 }
             }
         }
-        ok = __all_sync(0xffffffffu, ok);
-        if (threadIdx.x == 0) s_ok = ok ? 1 : 0;
     }
     __syncthreads();
-    return s_ok != 0;
 }
 
-// CG on the rows of S with the single-reduction (Chronopoulos-Gear)
-// recurrences, from the state k_tc_init left (y_B, r, rho, ||b||^2):
-//   [wait for the neighbours' r] w = S r, gamma = r.r, delta = w.r (every 8th:
+// CG on rows with a unit or a given diagonal and K neighbours (K = 6: rows of
+// S; K = 3: the scaled matrix itself, FP64 Jacobi on all cells) with the
+// single-reduction (Chronopoulos-Gear) recurrences, from y, r and the state an
+// init kernel left (rho, ||b||^2, thresholds):
+//   [wait for the neighbours' r] w = A r, gamma = r.r, delta = w.r (every 8th:
 //   ||wt r||^2) | one grid reduction: stop test, beta = gamma / gamma_old,
 //   alpha = gamma / (delta - beta gamma / alpha_old) |
 //   p = r + beta p; s = w + beta s; y += alpha p; r -= alpha s | post
-// 13 FP64 FMAs a row (12 with the unit diagonal).  A thread owns the same rows
-// in both phases, so what only the owner reads stays in its block's shared
+// K + 7 FP64 FMAs a row (K + 6 with the unit diagonal).  A thread owns the same
+// rows in both phases, so what only the owner reads stays in its block's shared
 // memory across the iterations: RES vectors of p, s, y, w, r (a copy; the
 // neighbours gather r from global memory), and with MAT the rows themselves.
+// A block waits for the blocks that own its neighbours, whatever the numbering.
 // 1/gamma and 1/(gamma alpha) are carried (one thread divides beside the wait
 // for the neighbours), so one divide stays on the path the blocks wait on.
-template <int T, int RES, bool MAT, bool UNIT>
-__global__ void __launch_bounds__(T, 1) k_schur_cg(SchurArgs P) {
+template <int T, int K, int RES, bool MAT, bool UNIT>
+__global__ void __launch_bounds__(T, 1) k_resident_cg(SchurArgs P) {
     extern __shared__ double dyn[];
     // alpha, beta, 1/gamma, 1/(gamma alpha), ||S r||^2, stop threshold, gamma
     __shared__ double sc[7];
     __shared__ int s_stop;          // 0 run, 1 stop, 2 breakdown
     __shared__ int s_fail;          // a wait ran out
     __shared__ long long s_max_iter;
-    __shared__ int s_lo, s_hi;
+    __shared__ unsigned int s_dep[kPollPer];    // the blocks that own this one's neighbours
     CgState* st = P.st;
     if (st->done) return;                      // uniform: set before the launch
+    constexpr int U = K <= 3 ? 2 : 1;          // rows a trip of the product (loads in flight)
     const int n = P.n;
     const int64_t ld = P.ld;
     const int R = (((n + (int)gridDim.x - 1) / (int)gridDim.x) + 31) & ~31;
-    const int lo = min((int)blockIdx.x * R, n);
-    const int cnt = min(lo + R, n) - lo;
+    const int lo = (int)min((int64_t)blockIdx.x * R, (int64_t)n);
+    const int cnt = (int)min((int64_t)lo + R, (int64_t)n) - lo;
     const int tid = (int)threadIdx.x;
+    const double* const rall = P.r;
     double* const rg = P.r + lo;
     double* const p = RES >= 1 ? dyn : P.p + lo;
     double* const sv = RES >= 2 ? dyn + R : P.s + lo;
     double* const y = RES >= 3 ? dyn + 2 * R : P.y + lo;
     double* const w = RES >= 4 ? dyn + 3 * R : P.w + lo;
     double* const rl = RES >= 5 ? dyn + 4 * R : rg;
-    // resident rows: values [6][R], diagonal [R], columns [6][R]
+    // resident rows: values [K][R], diagonal [R] unless unit, columns [K][R]
     double* const vm = dyn + RES * R;
-    double* const dm = vm + kSlots * R;
-    int32_t* const cm = reinterpret_cast<int32_t*>(dm + R);
+    double* const dm = vm + K * R;
+    int32_t* const cm = reinterpret_cast<int32_t*>(dm + (UNIT ? 0 : R));
     const double* const vg = P.v + lo;
     const double* const dg = P.d + lo;
     const int32_t* const cg = P.c + lo;
     GridSync* gs = P.gs;
 
+    if (tid < kPollPer) s_dep[tid] = 0u;
     if (tid == 0) {
-        s_lo = INT32_MAX;
-        s_hi = -1;
         sc[2] = sc[3] = 0.0;
         sc[4] = st->rnorm2;
         sc[5] = st->thresh2;
@@ -463,70 +462,48 @@ __global__ void __launch_bounds__(T, 1) k_schur_cg(SchurArgs P) {
         s_max_iter = st->max_iter;
     }
     __syncthreads();
-    {
-        int cmin = INT32_MAX, cmax = -1;
-        for (int i = tid; i < cnt; i += T) {
+    for (int i = tid; i < cnt; i += T) {
 #pragma unroll
-            for (int j = 0; j < kSlots; ++j) {
-                const int c = cg[j * ld + i];
-                cmin = min(cmin, c);
-                cmax = max(cmax, c);
-                if (MAT) {
-                    cm[j * R + i] = c;
-                    vm[j * R + i] = vg[j * ld + i];
-                }
+        for (int j = 0; j < K; ++j) {
+            const int c = cg[j * ld + i];
+            const int q = c / R;
+            if (q != (int)blockIdx.x && !((s_dep[q >> 5] >> (q & 31)) & 1u))
+                atomicOr(&s_dep[q >> 5], 1u << (q & 31));
+            if (MAT) {
+                cm[j * R + i] = c;
+                vm[j * R + i] = vg[j * ld + i];
             }
-            if (MAT && !UNIT) dm[i] = dg[i];
-            p[i] = 0.0;
-            sv[i] = 0.0;
-            if (RES >= 3) y[i] = P.y[lo + i];
-            if (RES >= 5) rl[i] = rg[i];
         }
-        if (cmax >= 0) {
-            atomicMin(&s_lo, cmin / R);
-            atomicMax(&s_hi, cmax / R);
-        }
+        if (MAT && !UNIT) dm[i] = dg[i];
+        p[i] = 0.0;
+        sv[i] = 0.0;
+        if (RES >= 3) y[i] = P.y[lo + i];
+        if (RES >= 5) rl[i] = rg[i];
     }
     __syncthreads();
-    const int dlo = s_hi >= 0 ? s_lo : (int)blockIdx.x;
-    const int dhi = s_hi >= 0 ? s_hi : (int)blockIdx.x;
     unsigned int ep1 = 0, ep2 = 0;  // reductions of one and of two quantities so far
-    unsigned long long bar = 0;     // arrivals of the grid barriers (no local halo)
-    bool halo;
-    {
-        const double wide[1] = {dhi - dlo + 1 > kSchurDeps ? 1.0 : 0.0};
-        tagged_allreduce<T>(wide, ep1, P, s_fail, [&](const double* t) { sc[0] = t[0]; });
-        __syncthreads();
-        halo = sc[0] == 0.0;
-        __syncthreads();
-    }
-    bool ok = s_fail == 0;
+    bool ok = true;
     long long it = 0;
-    while (ok) {
-        double v[kSlots], dd = 1.0;
-        int c[kSlots];
-        auto load = [&](int i) {
+    for (;;) {
+        double v[U][K], dd[U];
+        int c[U][K];
+        auto load = [&](int u, int i) {
 #pragma unroll
-            for (int j = 0; j < kSlots; ++j) {
-                c[j] = MAT ? cm[j * R + i] : cg[j * ld + i];
-                v[j] = MAT ? vm[j * R + i] : vg[j * ld + i];
+            for (int j = 0; j < K; ++j) {
+                c[u][j] = MAT ? cm[j * R + i] : cg[j * ld + i];
+                v[u][j] = MAT ? vm[j * R + i] : vg[j * ld + i];
             }
-            if (!UNIT) dd = MAT ? dm[i] : dg[i];
+            dd[u] = UNIT ? 1.0 : (MAT ? dm[i] : dg[i]);
         };
         // the first trip's rows are on their way while the neighbours finish
-        if (!MAT && tid < cnt) load(tid);
+        if (!MAT) {
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (tid + u * T < cnt) load(u, tid + u * T);
+        }
         if (it > 0) {
-            if (halo) {
-                ok = halo_wait_all(gs, dlo, dhi, (unsigned long long)it);
-            } else {
-                bar += gridDim.x;
-                if (tid == 0) {
-                    red_release_add(&gs->count, 1ull);
-                    if (!wait_geq(&gs->count, bar, gs)) s_fail = 1;
-                }
-                __syncthreads();
-                ok = s_fail == 0;
-            }
+            dep_wait(gs, s_dep, (unsigned long long)it, s_fail);
+            ok = s_fail == 0;
             if (!ok) break;
         }
         // the stop test every 8th iteration, and only once it can hold:
@@ -534,22 +511,35 @@ __global__ void __launch_bounds__(T, 1) k_schur_cg(SchurArgs P) {
         // in for this one's, with a margin of 64)
         const bool check = (it & 7) == 7 && P.dmin * sc[6] <= 64.0 * sc[5];
         double sums[2] = {0.0, 0.0}, nn = 0.0;
-        for (int i = tid; i < cnt; i += T) {
-            if (MAT || i != tid) load(i);
-            double g[kSlots];
+        for (int i0 = tid; i0 < cnt; i0 += U * T) {
+            double g[U][K], re[U];
+            if (MAT || i0 != tid) {
 #pragma unroll
-            for (int j = 0; j < kSlots; ++j) g[j] = P.r[c[j]];
-            const double re = rl[i];
-            double acc = UNIT ? re : dd * re;
-#pragma unroll
-            for (int j = 0; j < kSlots; ++j) acc = fma(v[j], g[j], acc);
-            w[i] = acc;
-            sums[0] = fma(re, re, sums[0]);
-            sums[1] = fma(acc, re, sums[1]);
-            if (check) {
-                const double t = P.wt[lo + i] * re;
-                nn = fma(t, t, nn);
+                for (int u = 0; u < U; ++u)
+                    if (u == 0 || i0 + u * T < cnt) load(u, i0 + u * T);
             }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (u == 0 || i0 + u * T < cnt) {
+#pragma unroll
+                    for (int j = 0; j < K; ++j) g[u][j] = rall[c[u][j]];
+                    re[u] = rl[i0 + u * T];
+                }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (u == 0 || i0 + u * T < cnt) {
+                    const int i = i0 + u * T;
+                    double acc = UNIT ? re[u] : dd[u] * re[u];
+#pragma unroll
+                    for (int j = 0; j < K; ++j) acc = fma(v[u][j], g[u][j], acc);
+                    w[i] = acc;
+                    sums[0] = fma(re[u], re[u], sums[0]);
+                    sums[1] = fma(acc, re[u], sums[1]);
+                    if (check) {
+                        const double t = P.wt[lo + i] * re[u];
+                        nn = fma(t, t, nn);
+                    }
+                }
         }
         const long long it0 = it;
         if (check) {
@@ -567,7 +557,7 @@ __global__ void __launch_bounds__(T, 1) k_schur_cg(SchurArgs P) {
             if (!f) {
                 // from p = s = 0 on the run's first pass: den = delta, beta = 0
                 const double den = it0 == 0 ? dl : fma(-(g * g), sc[3], dl);
-                // on the first pass p.Sp <= 0: not SPD; later, the
+                // on the first pass p.Ap <= 0: not SPD; later, the
                 // recurrence's difference lost its digits at the FP64 floor:
                 // stop, and let the true residual decide
                 if (!(den > 0.0) || !isfinite(den)) f = it0 > 0 ? 1 : 2;
@@ -583,22 +573,35 @@ __global__ void __launch_bounds__(T, 1) k_schur_cg(SchurArgs P) {
         if (!ok || s_stop) break;
         {
             const double alpha = sc[0], beta = sc[1];
-#pragma unroll 2
-            for (int i = tid; i < cnt; i += T) {
-                const double re = rl[i];
-                const double pn = fma(beta, p[i], re);
-                const double sn = fma(beta, sv[i], w[i]);
-                const double rn = fma(-alpha, sn, re);
-                rg[i] = rn;
-                if (RES >= 5) rl[i] = rn;
-                p[i] = pn;
-                sv[i] = sn;
-                y[i] = fma(alpha, pn, y[i]);
+            for (int i0 = tid; i0 < cnt; i0 += 2 * T) {
+                double re[2], pe[2], se[2], we[2], ye[2];
+#pragma unroll
+                for (int u = 0; u < 2; ++u)
+                    if (u == 0 || i0 + u * T < cnt) {
+                        const int i = i0 + u * T;
+                        re[u] = rl[i];
+                        pe[u] = p[i];
+                        se[u] = sv[i];
+                        we[u] = w[i];
+                        ye[u] = y[i];
+                    }
+#pragma unroll
+                for (int u = 0; u < 2; ++u)
+                    if (u == 0 || i0 + u * T < cnt) {
+                        const int i = i0 + u * T;
+                        const double pn = fma(beta, pe[u], re[u]);
+                        const double sn = fma(beta, se[u], we[u]);
+                        const double rn = fma(-alpha, sn, re[u]);
+                        rg[i] = rn;
+                        if (RES >= 5) rl[i] = rn;
+                        p[i] = pn;
+                        sv[i] = sn;
+                        y[i] = fma(alpha, pn, ye[u]);
+                    }
             }
         }
         ++it;
-        if (halo) halo_post(gs, (unsigned long long)it);
-        else __syncthreads();
+        halo_post(gs, (unsigned long long)it);
         if (tid == 32) {
             // for the next iteration: off the path that the blocks wait on
             const double ig = 1.0 / sc[6];
@@ -619,37 +622,120 @@ __global__ void __launch_bounds__(T, 1) k_schur_cg(SchurArgs P) {
 
 using SchurKernel = void (*)(SchurArgs);
 
-// The kernel whose resident part of R rows fits a block's shared memory, most
-// first, the dynamic bytes it takes and its threads.
-SchurKernel schur_kernel(int64_t R, bool unit, size_t limit, size_t* bytes, int* threads) {
-    struct Form {
-        int threads, res;
-        bool mat;
-        SchurKernel diag, unit;
-    };
-    // Resident rows leave few rows a thread: 512 threads synchronise faster.
-    // Streamed rows want 1024 threads' loads in flight.
-    static const Form forms[] = {
-        {512, 5, true, k_schur_cg<512, 5, true, false>, k_schur_cg<512, 5, true, true>},
-        {1024, 5, false, k_schur_cg<1024, 5, false, false>, k_schur_cg<1024, 5, false, true>},
-        {1024, 4, false, k_schur_cg<1024, 4, false, false>, k_schur_cg<1024, 4, false, true>},
-        {1024, 3, false, k_schur_cg<1024, 3, false, false>, k_schur_cg<1024, 3, false, true>},
-        {1024, 0, false, k_schur_cg<1024, 0, false, false>, k_schur_cg<1024, 0, false, true>}};
-    for (const Form& f : forms) {
-        const SchurKernel k = unit ? f.unit : f.diag;
+// The kernel of rows with K neighbours whose resident part of R rows fits a
+// block's shared memory, most first, the dynamic bytes it takes and its threads.
+struct Form {
+    int threads, res;
+    bool mat;
+    SchurKernel kern;
+};
+
+// Resident rows leave few rows a thread: 512 threads synchronise faster (7.9
+// against 8.8 us a step at 90k rows).  Streamed rows want 1024 threads' loads in
+// flight.
+template <int K, bool UNIT>
+const Form* forms(int* count) {
+    // Jacobi on all cells (K = 3) not without resident vectors (jacobi_resident)
+    static const Form f[] = {{512, 5, true, k_resident_cg<512, K, 5, true, UNIT>},
+                             {1024, 5, false, k_resident_cg<1024, K, 5, false, UNIT>},
+                             {1024, 4, false, k_resident_cg<1024, K, 4, false, UNIT>},
+                             {1024, 3, false, k_resident_cg<1024, K, 3, false, UNIT>},
+                             {1024, 0, false,
+                              K == 3 ? nullptr : k_resident_cg<1024, 6, 0, false, UNIT>}};
+    *count = K == 3 ? 4 : 5;
+    return f;
+}
+
+const Form* pick_form(int K, bool unit, int64_t R, size_t limit, size_t* bytes) {
+    int count = 0;
+    const Form* f = K == 3 ? forms<3, true>(&count)
+                           : (unit ? forms<6, true>(&count) : forms<6, false>(&count));
+    for (int i = 0; i < count; ++i) {
         cudaFuncAttributes at;
-        if (cudaFuncGetAttributes(&at, k) != cudaSuccess) return nullptr;
-        const size_t need = (size_t)R * (8 * f.res + (f.mat ? kSlots * 12 + 8 : 0));
-        if (need + at.sharedSizeBytes <= limit) {
-            *bytes = need;
-            *threads = f.threads;
-            return k;
+        if (cudaFuncGetAttributes(&at, f[i].kern) != cudaSuccess) return nullptr;
+        const size_t row = 8 * f[i].res + (f[i].mat ? K * 12 + (unit ? 0 : 8) : 0);
+        if ((size_t)R * row + at.sharedSizeBytes <= limit) {
+            *bytes = (size_t)R * row;
+            return &f[i];
         }
     }
     return nullptr;
 }
 
+// One cooperative launch of the loop over G blocks on the rows in P (its gs,
+// st, stall and pb set here), with a persisting L2 window if win_bytes > 0.
+int launch_resident(cps_sys s, SchurArgs P, int K, bool unit, int G, const void* win,
+                    size_t win_bytes, cudaStream_t stream) {
+    const int rc = ensure_gsync(s);
+    if (rc) return rc;
+    const int64_t R = ((((int64_t)P.n + G - 1) / G) + 31) & ~(int64_t)31;
+    size_t smem = 0;
+    const Form* f = pick_form(K, unit, R, s->ctx->smem_optin, &smem);
+    if (!f) {
+        cudaGetLastError();
+        cps::set_error(s->ctx, "persistent: no kernel for this device");
+        return CPS_ERR_CUDA;
+    }
+    CPS_CUDA_TRY(s->ctx, cudaFuncSetAttribute(f->kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              (int)smem));
+    P.gs = reinterpret_cast<GridSync*>(s->gsync);
+    P.pb = reinterpret_cast<unsigned long long*>(P.gs + 1);
+    P.st = s->st;
+    P.stall = s->inject == CPS_TEST_STALL_BARRIER ? 1 : 0;
+    s->inject = 0;
+    // counter, timeout, the G flags in use and the slots start at zero
+    CPS_CUDA_TRY(s->ctx, cudaMemsetAsync(s->gsync, 0,
+                                         offsetof(GridSync, flag) +
+                                             sizeof(unsigned long long) * kFlagStride * G,
+                                         stream));
+    CPS_CUDA_TRY(s->ctx, cudaMemsetAsync(P.pb, 0, sizeof(unsigned long long) * kSlotWords, stream));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(G, 1, 1);
+    cfg.blockDim = dim3(f->threads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    at[1].id = cudaLaunchAttributeAccessPolicyWindow;
+    at[1].val.accessPolicyWindow.base_ptr = const_cast<void*>(win);
+    at[1].val.accessPolicyWindow.num_bytes = win_bytes;
+    at[1].val.accessPolicyWindow.hitRatio = 1.0f;
+    at[1].val.accessPolicyWindow.hitProp = cudaAccessPropertyPersisting;
+    at[1].val.accessPolicyWindow.missProp = cudaAccessPropertyStreaming;
+    cfg.attrs = at;
+    cfg.numAttrs = win_bytes > 0 ? 2 : 1;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, f->kern, P);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        cps::set_error(s->ctx, std::string("persistent launch: ") + cudaGetErrorString(e));
+        return CPS_ERR_CUDA;
+    }
+    return CPS_OK;
+}
+
+// Blocks for n rows: one per SM, at least 256 rows each.
+int resident_grid(cps_sys s, int64_t n) {
+    int G = s->ctx->num_sms < kGridMax ? s->ctx->num_sms : kGridMax;
+    const int64_t most = (n + 255) / 256;
+    if (most < G) G = (int)(most < 1 ? 1 : most);
+    return G;
+}
+
 }  // namespace
+
+// Synchronisation state of a system's persistent launches: the flags, and the
+// slots of the tagged reductions behind them.
+int ensure_gsync(cps_sys s) {
+    if (!s->gsync && cudaMalloc((void**)&s->gsync, sizeof(GridSync) + sizeof(unsigned long long) *
+                                                       kSlotWords) != cudaSuccess) {
+        cudaGetLastError();
+        s->gsync = nullptr;
+        cps::set_error(s->ctx, "persistent: cudaMalloc failed");
+        return CPS_ERR_NOMEM;
+    }
+    return CPS_OK;
+}
 
 // Frees the Schur rows of a system.
 void free_schur(cps_sys s) {
@@ -665,8 +751,7 @@ int schur_setup(cps_sys s, bool scaled, cudaStream_t stream) {
     if (!h.buf) {
         h.ld = (nB + 31) & ~(int64_t)31;
         // r, w, p, s, y first: one contiguous range for an L2 window
-        const size_t bytes = (size_t)h.ld * (8 * (5 + kSlots + 3) + 4 * kSlots) +
-                             sizeof(unsigned long long) * kSlotWords;
+        const size_t bytes = (size_t)h.ld * (8 * (5 + kSlots + 3) + 4 * kSlots);
         cudaError_t e = cudaMalloc(&h.buf, bytes);
         if (e != cudaSuccess) {
             cudaGetLastError();
@@ -684,8 +769,7 @@ int schur_setup(cps_sys s, bool scaled, cudaStream_t stream) {
         h.d = q + (5 + kSlots) * h.ld;
         h.wt = h.d + h.ld;
         h.dsc = h.wt + h.ld;
-        h.pb = reinterpret_cast<unsigned long long*>(h.dsc + h.ld);
-        h.c = reinterpret_cast<int32_t*>(h.pb + kSlotWords);
+        h.c = reinterpret_cast<int32_t*>(h.dsc + h.ld);
         h.nB = nB;
         h.form = 0;
     }
@@ -698,14 +782,6 @@ int schur_setup(cps_sys s, bool scaled, cudaStream_t stream) {
     CPS_CUDA_TRY(s->ctx, cudaGetLastError());
     h.form = want;
     return CPS_OK;
-}
-
-// Blocks of the persistent loop by default: one per SM, at least 256 rows each.
-int schur_grid(cps_sys s) {
-    int G = s->ctx->num_sms < kGridMax ? s->ctx->num_sms : kGridMax;
-    const int64_t most = (s->sch.nB + 255) / 256;
-    if (most < G) G = (int)(most < 1 ? 1 : most);
-    return G;
 }
 
 // A run's start from x (mesh order): y_R, y_B, r and the state in s->st.
@@ -734,62 +810,61 @@ int schur_back(cps_sys s, const double* b, cudaStream_t stream) {
 size_t schur_window_bytes(cps_sys s) { return sizeof(double) * 5 * (size_t)s->sch.ld; }
 
 // The CG run from schur_init's state as one cooperative launch of `grid`
-// blocks (0: schur_grid), with the five vectors in persisting L2 if window
+// blocks (0: one per SM), with the five vectors in persisting L2 if window
 // (the caller holds the set-aside).  State in s->st.
 int schur_run(cps_sys s, int grid, bool window, cudaStream_t stream) {
     SchurData& h = s->sch;
-    if (!s->gsync) {
-        if (cudaMalloc((void**)&s->gsync, sizeof(GridSync)) != cudaSuccess) {
-            cudaGetLastError();
-            cps::set_error(s->ctx, "Schur solve: cudaMalloc failed");
-            return CPS_ERR_NOMEM;
-        }
-    }
-    int G = schur_grid(s);
+    int G = resident_grid(s, h.nB);
     if (grid > 0 && grid < G) G = grid;
-    const int64_t R = (((h.nB + G - 1) / G) + 31) & ~(int64_t)31;
+    SchurArgs P{};
+    P.v = h.v;
+    P.c = h.c;
+    P.d = h.d;
+    P.wt = h.wt;
+    P.r = h.r;
+    P.w = h.w;
+    P.p = h.p;
+    P.s = h.s;
+    P.y = h.y;
+    P.n = (int)h.nB;
+    P.ld = h.ld;
+    P.dmin = h.form == 2 ? 0.0 : s->diag_min;
+    return launch_resident(s, P, kSlots, h.form == 2, G, h.buf,
+                           window ? schur_window_bytes(s) : 0, stream);
+}
+
+// Whether jacobi_run takes this system: p, s and y of a block's rows have to fit
+// its shared memory (up to 1.44M cells on 152 SMs).  With fewer resident the L1
+// that is left does not hold the gathers: at 2.09M cells p and s resident took
+// 48.1 us an iteration, k_persistent_gear (nothing resident, the L1 whole) 42.5;
+// at 0.98M 21.8 against 23.1, at 0.4M 11.6 against 13.8, at 33k 5.7 against 7.8.
+bool jacobi_resident(cps_sys s) {
+    const int G = resident_grid(s, s->nt);
     size_t smem = 0;
-    int threads = 0;
-    SchurKernel kern = schur_kernel(R, h.form == 2, s->ctx->smem_optin, &smem, &threads);
-    if (!kern) {
-        cudaGetLastError();
-        cps::set_error(s->ctx, "Schur solve: no kernel for this device");
-        return CPS_ERR_CUDA;
-    }
-    CPS_CUDA_TRY(s->ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)smem));
-    CPS_CUDA_TRY(s->ctx, cudaMemsetAsync(s->gsync, 0,
-                                         offsetof(GridSync, flag) +
-                                             sizeof(unsigned long long) * kFlagStride * G,
-                                         stream));
-    CPS_CUDA_TRY(s->ctx, cudaMemsetAsync(h.pb, 0, sizeof(unsigned long long) * kSlotWords, stream));
-    SchurArgs P{h.v, h.c, h.d, h.wt, h.r, h.w, h.p, h.s, h.y, (int)h.nB, h.ld, h.pb,
-                reinterpret_cast<GridSync*>(s->gsync), s->st,
-                s->inject == CPS_TEST_STALL_BARRIER ? 1 : 0, h.form == 2 ? 0.0 : s->diag_min};
-    s->inject = 0;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(G, 1, 1);
-    cfg.blockDim = dim3(threads, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = stream;
-    cudaLaunchAttribute at[2];
-    at[0].id = cudaLaunchAttributeCooperative;
-    at[0].val.cooperative = 1;
-    at[1].id = cudaLaunchAttributeAccessPolicyWindow;
-    at[1].val.accessPolicyWindow.base_ptr = h.buf;
-    at[1].val.accessPolicyWindow.num_bytes = schur_window_bytes(s);
-    at[1].val.accessPolicyWindow.hitRatio = 1.0f;
-    at[1].val.accessPolicyWindow.hitProp = cudaAccessPropertyPersisting;
-    at[1].val.accessPolicyWindow.missProp = cudaAccessPropertyStreaming;
-    cfg.attrs = at;
-    cfg.numAttrs = window ? 2 : 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, kern, P);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        cps::set_error(s->ctx, std::string("Schur solve launch: ") + cudaGetErrorString(e));
-        return CPS_ERR_CUDA;
-    }
-    return CPS_OK;
+    return pick_form(3, true, ((((s->nt + G - 1) / G) + 31) & ~(int64_t)31), s->ctx->smem_optin,
+                     &smem) != nullptr;
+}
+
+// FP64 Jacobi on all cells from the state k_init64 left (y, r), the same loop on
+// the scaled matrix's own rows (s = A p in q, w = A r in p1), with r, p, q, y, p1
+// in persisting L2 over win_bytes from win.
+int jacobi_run(cps_sys s, int grid, const void* win, size_t win_bytes, cudaStream_t stream) {
+    int G = resident_grid(s, s->nt);
+    if (grid > 0 && grid < G) G = grid;
+    SchurArgs P{};
+    P.v = s->a;
+    P.c = s->col;
+    P.d = s->diag;
+    P.wt = s->s;
+    P.r = s->wr;
+    P.w = s->wp1;
+    P.p = s->wp0;
+    P.s = s->wq;
+    P.y = s->wy;
+    P.n = (int)s->nt;
+    P.ld = s->nt;
+    P.dmin = s->diag_min;
+    return launch_resident(s, P, 3, true, G, win, win_bytes, stream);
 }
 
 }  // namespace cps
