@@ -778,7 +778,7 @@ def sequence_summary(n: int, rtol: float, iters: int = 200) -> dict:
         x.zero_()
         t, st = timed(lambda: s.solve(rhs[0], x=x, rtol=rtol, max_iter=iters, precision=prec,
                                       check=False)[1], stream)
-        if prec == cps.FP64:
+        if prec == cps.FP64 or s.tuning(cps.FP64).get("two_cyclic"):
             bpc = method_bytes(name.split("_")[0], s.tuning(cps.FP64))
         gbs = bpc * nt * st.iters / t / 1e9
         out[name] = {"iters": st.iters, "us_per_iter": 1e6 * t / max(st.iters, 1),
@@ -850,8 +850,9 @@ def run_sequence(args):
             rel.append(st.rel_res)
             status.append(st.status)
             per.append(dt_)
-        if prec == cps.FP64:
-            bpc = method_bytes(name, s.tuning(cps.FP64))
+        tf = s.tuning(cps.FP64)
+        if prec == cps.FP64 or tf.get("two_cyclic"):
+            bpc = method_bytes("jacobi" if name == "mixed" else name, tf)
         # reduced system: iterations run over the black half of the cells
         units = nt // 2 if pc == cps.PC_REDUCED else nt
         gbs = bpc * nt * it_tot / t_tot / 1e9
@@ -1337,7 +1338,8 @@ def main():
     roof = roofline(tuning["fp64"], nt, jf["iters"], jf["time_to_rtol_s"], peak, peak_kind,
                     args.n)
     jm = variants["jacobi_mixed"]
-    jm["inner_gbs"] = BYTES_PER_CELL_ITER_MIXED * nt * jm["iters"] / jm["time_to_rtol_s"] / 1e9
+    if not tuning["fp64"].get("two_cyclic"):       # else the FP64 loop ran
+        jm["inner_gbs"] = BYTES_PER_CELL_ITER_MIXED * nt * jm["iters"] / jm["time_to_rtol_s"] / 1e9
 
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,

@@ -71,7 +71,7 @@ extern "C" {
                                exactly, CG on the other colour's Schur complement */
 
 #define CPS_FP64 0          /* all storage and arithmetic in binary64 */
-#define CPS_MIXED 1         /* binary32 matrix/vectors inside FP64 refinement */
+#define CPS_MIXED 1         /* binary32 matrix/vectors inside FP64 refinement allowed */
 
 typedef struct cps_ctx_s* cps_ctx;
 typedef struct cps_sys_s* cps_sys;
@@ -169,7 +169,9 @@ int cps_export_matrix(cps_sys sys, double* diag, int32_t* col, double* val, void
  *   max_iter    bound on PCG iterations (summed over refinements)
  *   precision   CPS_FP64 or CPS_MIXED (binary32 matrix, vectors and SpMV in
  *               the inner PCG; binary64 dot products, alpha/beta, and the
- *               outer residual b - A x and update of x)
+ *               outer residual b - A x and update of x; under CPS_PATH_AUTO a
+ *               CP2 system whose cell graph has two colours takes the FP64
+ *               two-cyclic loop instead, which is faster: see CPS_PATH_AUTO)
  *   stats       host pointer, may be NULL
  * b = 0 gives x = 0.  Errors: CPS_ERR_ARG, _NOT_SPD, _NOT_CONVERGED (x holds
  * the last iterate; CPS_MIXED: the iterate with the least true residual, with
@@ -397,7 +399,7 @@ int cps_cp2_kernel_times(cps_sys sys, float* ms);
  * FP64 IC(0) in a two-colour order runs on the streaming kernels for every
  * other pin, and CPS_PATH_AUTO times both ways on the first such solve; with
  * more colours it always streams.
- * Mixed precision always streams. */
+ * Mixed precision streams, but for CPS_PATH_AUTO's two-cyclic form. */
 #define CPS_PATH_AUTO 0
 #define CPS_PATH_STREAM 1
 #define CPS_PATH_CLUSTER 2
