@@ -655,6 +655,11 @@ const Form* pick_form(int K, bool unit, int64_t R, size_t limit, size_t* bytes) 
         if (cudaFuncGetAttributes(&at, f[i].kern) != cudaSuccess) return nullptr;
         const size_t row = 8 * f[i].res + (f[i].mat ? K * 12 + (unit ? 0 : 8) : 0);
         if ((size_t)R * row + at.sharedSizeBytes <= limit) {
+            // the same bound whatever the rows: solves on other host threads
+            // may launch this kernel with other sizes meanwhile
+            if (cudaFuncSetAttribute(f[i].kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)(limit - at.sharedSizeBytes)) != cudaSuccess)
+                return nullptr;
             *bytes = (size_t)R * row;
             return &f[i];
         }
@@ -676,8 +681,6 @@ int launch_resident(cps_sys s, SchurArgs P, int K, bool unit, int G, const void*
         cps::set_error(s->ctx, "persistent: no kernel for this device");
         return CPS_ERR_CUDA;
     }
-    CPS_CUDA_TRY(s->ctx, cudaFuncSetAttribute(f->kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)smem));
     P.gs = reinterpret_cast<GridSync*>(s->gsync);
     P.pb = reinterpret_cast<unsigned long long*>(P.gs + 1);
     P.st = s->st;
