@@ -349,7 +349,7 @@ void free_sys(cps_sys s) {
     free_cp1(s);
     free_schur(s);
     // s->col lives inside s->a's allocation (one range for the L2 window)
-    void* bufs[] = {s->s,     s->diag,  s->a,     s->a32,     s->s32,      s->gfac,
+    void* bufs[] = {s->off, s->s,     s->diag,  s->a,     s->a32,     s->s32,      s->gfac,
                     s->dxi,   s->slot_kind, s->perm, s->iperm, s->pa,  s->pcol,     s->pl,
                     s->pdinv, s->pdiag, s->ps, s->pa32, s->pl32, s->pdinv32, s->ps32,   s->wvec,
                     s->partials, s->st, s->gsync};
@@ -435,6 +435,7 @@ int assemble_impl(cps_ctx ctx, const double* xy, int64_t nv, const int32_t* tri,
         s->wx = w + 7 * vs;
         s->wbest = w + 8 * vs;
     }
+    TRY_ALLOC(s->off, 3 * nt);
     TRY_ALLOC(s->partials, (kNumPartials + 16) * kMaxGrid);
     TRY_ALLOC(s->st, 2);
     if (field_loc == CPS_PER_CELL && kind == CPS_KIND_CP2) {
@@ -459,7 +460,7 @@ int assemble_impl(cps_ctx ctx, const double* xy, int64_t nv, const int32_t* tri,
         cap <<= 1;   // load factor <= 1/4 of the 3 nt side slots (<= 1/2 of sides)
         unsigned long long* keys = nullptr;
         int32_t *id0 = nullptr, *id1 = nullptr, *nbr = nullptr;
-        double *area = nullptr, *ccx = nullptr, *ccy = nullptr, *xi = nullptr, *off = nullptr;
+        double *area = nullptr, *ccx = nullptr, *ccy = nullptr, *xi = nullptr;
         int* err = nullptr;
         unsigned long long* counters = nullptr;  // [0] interior slot count, [1] dmin bits
         int* iso = nullptr;
@@ -476,7 +477,6 @@ int assemble_impl(cps_ctx ctx, const double* xy, int64_t nv, const int32_t* tri,
         if (ce == cudaSuccess) ce = A((void**)&ccx, sizeof(double) * nt);
         if (ce == cudaSuccess) ce = A((void**)&ccy, sizeof(double) * nt);
         if (ce == cudaSuccess) ce = A((void**)&xi, sizeof(double) * 3 * nf);
-        if (ce == cudaSuccess) ce = A((void**)&off, sizeof(double) * 3 * nt);
         if (ce == cudaSuccess) ce = A((void**)&err, sizeof(int) * 2);
         if (ce == cudaSuccess) ce = A((void**)&counters, sizeof(unsigned long long) * 2);
         if (ce == cudaSuccess) {
@@ -507,12 +507,12 @@ int assemble_impl(cps_ctx ctx, const double* xy, int64_t nv, const int32_t* tri,
             TransArgs ta;
             ta.xy = xy; ta.tri = tri; ta.nbr = nbr; ta.ccx = ccx; ta.ccy = ccy; ta.area = area;
             ta.xi = xi; ta.eps = eps; ta.kinv = kinv; ta.slot_kind = s->slot_kind;
-            ta.diag = s->diag; ta.off = off; ta.col = s->col; ta.gfac = s->gfac;
+            ta.diag = s->diag; ta.off = s->off; ta.col = s->col; ta.gfac = s->gfac;
             ta.n_interior = counters; ta.nt = nt; ta.kind = kind; ta.field_loc = field_loc;
             ta.nu = nu; ta.dt = dt; ta.err = err; ta.logk = logk;
             k_transmissibility<<<g1, kBlock, 0, stream>>>(ta);
             k_sqrt_diag<<<g1, kBlock, 0, stream>>>(s->diag, nt, s->s, s->s32, counters + 1, err);
-            k_scale_offdiag<<<g3, kBlock, 0, stream>>>(off, s->col, s->s, nt, s->a, s->a32);
+            k_scale_offdiag<<<g3, kBlock, 0, stream>>>(s->off, s->col, s->s, nt, s->a, s->a32);
             if (s->dxi) k_dxi_dtheta<<<g1, kBlock, 0, stream>>>(eps, kinv, nt, nu, dt, logk, s->dxi, iso);
             s->assembly_launches = 8 + (nb > 0 ? 1 : 0) + (s->dxi ? 1 : 0);
             ce = cudaGetLastError();
@@ -521,7 +521,7 @@ int assemble_impl(cps_ctx ctx, const double* xy, int64_t nv, const int32_t* tri,
             if (ce == cudaSuccess)
                 ce = cudaMemcpyAsync(h_cnt, counters, sizeof(h_cnt), cudaMemcpyDeviceToHost, stream);
         }
-        void* scratch[] = {keys, id0, id1, nbr, area, ccx, ccy, xi, off, err, counters};
+        void* scratch[] = {keys, id0, id1, nbr, area, ccx, ccy, xi, err, counters};
         for (void* p : scratch)
             if (p) cudaFreeAsync(p, stream);
         cudaError_t se = cudaStreamSynchronize(stream);

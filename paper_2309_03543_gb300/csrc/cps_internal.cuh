@@ -313,6 +313,7 @@ struct cps_sys_s {
     double* diag = nullptr;     // [nt] unscaled diagonal (export / info)
     double* a = nullptr;        // [3*nt] scaled off-diagonals (allocation also holds col)
     int32_t* col = nullptr;     // [3*nt] column (= row for an unused slot)
+    double* off = nullptr;      // [3*nt] unscaled off-diagonals (matvec, export)
     size_t mat_bytes = 0;       // bytes of the a + col allocation
     float* a32 = nullptr;       // [3*nt] binary32 copy of a (mixed precision)
     float* s32 = nullptr;       // [nt]

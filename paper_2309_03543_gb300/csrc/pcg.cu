@@ -1597,7 +1597,7 @@ int matvec_impl(cps_sys s, const double* x, double* y, cudaStream_t stream) {
         cps::set_error(s->ctx, "matvec: null pointer");
         return CPS_ERR_ARG;
     }
-    k_matvec64<<<s->grid, kBlock, 0, stream>>>(x, s->s, s->a, s->col, s->nt, y);
+    k_matvec64<<<s->grid, kBlock, 0, stream>>>(x, s->diag, s->off, s->col, s->nt, y);
     CPS_CUDA_TRY(s->ctx, cudaGetLastError());
     return CPS_OK;
 }
@@ -1611,9 +1611,8 @@ int export_impl(cps_sys s, double* diag, int32_t* col, double* val, cudaStream_t
                                          cudaMemcpyDeviceToDevice, stream));
     CPS_CUDA_TRY(s->ctx, cudaMemcpyAsync(col, s->col, sizeof(int32_t) * 3 * s->nt,
                                          cudaMemcpyDeviceToDevice, stream));
-    k_unscale_offdiag<<<grid_for(s->ctx, 3 * s->nt), kBlock, 0, stream>>>(s->a, s->col, s->s,
-                                                                          s->nt, val);
-    CPS_CUDA_TRY(s->ctx, cudaGetLastError());
+    CPS_CUDA_TRY(s->ctx, cudaMemcpyAsync(val, s->off, sizeof(double) * 3 * s->nt,
+                                         cudaMemcpyDeviceToDevice, stream));
     return CPS_OK;
 }
 

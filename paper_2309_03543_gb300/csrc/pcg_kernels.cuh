@@ -521,30 +521,26 @@ __global__ void __launch_bounds__(kBlock) k_correct(double* __restrict__ x,
     CPS_GRID_STRIDE(e, n) { x[e] += (double)d[e] / s[e]; }
 }
 
-// y = A x = S (Ahat (S x)) in FP64.
+// y = A x on the unscaled matrix.  Bound by HBM: 60 B a row against 4 FP64
+// operations (from the scaled values it took 8 and was bound by FP64 issue: 147
+// us at 8.4M cells).  Two rows a trip, all loads before any use.
 __global__ void __launch_bounds__(kBlock) k_matvec64(const double* __restrict__ x,
-                                                     const double* __restrict__ s,
-                                                     const double* __restrict__ a,
+                                                     const double* __restrict__ diag,
+                                                     const double* __restrict__ off,
                                                      const int32_t* __restrict__ col, int64_t n,
                                                      double* __restrict__ y) {
-    CPS_GRID_STRIDE(e, n) {
-        const double se = s[e];
-        double v = se * x[e];
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            const int32_t c = col[j * n + e];
-            v = fma(a[j * n + e], s[c] * x[c], v);
-        }
-        y[e] = se * v;
-    }
-}
-
-__global__ void k_unscale_offdiag(const double* __restrict__ a, const int32_t* __restrict__ col,
-                                  const double* __restrict__ s, int64_t n, double* __restrict__ v) {
-    CPS_GRID_STRIDE(k, 3 * n) {
-        const int64_t e = k % n;
-        v[k] = a[k] * (s[e] * s[col[k]]);
-    }
+    constexpr int U = 2;
+    double xe[U], d[U], a0[U], a1[U], a2[U];
+    int32_t c0[U], c1[U], c2[U];
+    CPS_UNROLLED_LOOP(n, U,
+        (xe[u] = x[e], d[u] = diag[e], a0[u] = off[e], a1[u] = off[n + e], a2[u] = off[2 * n + e],
+         c0[u] = col[e], c1[u] = col[n + e], c2[u] = col[2 * n + e]),
+        {
+            double v = d[u] * xe[u];
+            v = fma(a0[u], x[c0[u]], v);
+            v = fma(a1[u], x[c1[u]], v);
+            y[e] = fma(a2[u], x[c2[u]], v);
+        })
 }
 
 // Gather/scatter between the mesh order and the solver's (colour) order.
