@@ -192,8 +192,12 @@ struct TransArgs {
     int* err;
 };
 
+// Side coefficients and the matrix of a cell: bound by FP64 issue (a root and
+// four divisions a side, some 250 operations a cell).  The interior sides are
+// counted per warp: an atomic per cell on one word held the kernel up.
 __global__ void k_transmissibility(TransArgs A) {
     const int64_t nt = A.nt;
+    unsigned int count = 0;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nt;
          e += (int64_t)gridDim.x * blockDim.x) {
         const int32_t v[3] = {A.tri[3 * e], A.tri[3 * e + 1], A.tri[3 * e + 2]};
@@ -257,7 +261,7 @@ __global__ void k_transmissibility(TransArgs A) {
                     coef = A.nu;
                 }
                 T = l * coef / d;
-                g = ep >= 0 ? l / (2.0 * d) : l / d;
+                if (A.gfac) g = ep >= 0 ? l / (2.0 * d) : l / d;
                 if (ep >= 0) {
                     c = ep;
                     sk = 1;
@@ -273,14 +277,17 @@ __global__ void k_transmissibility(TransArgs A) {
             if (A.gfac) A.gfac[slot] = g;
         }
         A.diag[e] = diag;
-        if (interior) atomicAdd(A.n_interior, (unsigned long long)interior);
+        count += interior;
     }
+    count = __reduce_add_sync(0xffffffffu, count);
+    if ((threadIdx.x & 31) == 0 && count)
+        atomicAdd(A.n_interior, (unsigned long long)count);
 }
 
 // s = sqrt(diag); also the smallest diagonal (as an ordered 64-bit pattern).
 __global__ void k_sqrt_diag(const double* __restrict__ diag, int64_t nt, double* __restrict__ s,
                             float* __restrict__ s32, unsigned long long* dmin, int* err) {
-    unsigned long long local = ~0ULL;
+    unsigned long long local = ~0ULL;       // combined per warp: one atomic each
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nt;
          e += (int64_t)gridDim.x * blockDim.x) {
         const double d = diag[e];
@@ -297,7 +304,11 @@ __global__ void k_sqrt_diag(const double* __restrict__ diag, int64_t nt, double*
         const unsigned long long bits = (unsigned long long)__double_as_longlong(d);
         local = bits < local ? bits : local;
     }
-    atomicMin(dmin, local);
+    const unsigned int all = 0xffffffffu;
+    const unsigned int hi = __reduce_min_sync(all, (unsigned int)(local >> 32));
+    const unsigned int lo = __reduce_min_sync(
+        all, (unsigned int)(local >> 32) == hi ? (unsigned int)local : ~0u);
+    if ((threadIdx.x & 31) == 0) atomicMin(dmin, ((unsigned long long)hi << 32) | lo);
 }
 
 __global__ void k_scale_offdiag(const double* __restrict__ off, const int32_t* __restrict__ col,
