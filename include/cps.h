@@ -193,7 +193,10 @@ int cps_solve(cps_sys sys, const double* b, double* x, double rtol, int64_t max_
  * block takes whole systems from a device work queue (largest first) and
  * solves each with block-level reductions only; a team's blocks join the
  * queue when their system is done, and every system stops as soon as it
- * converges.  The iteration is the single-reduction (Chronopoulos-Gear) form
+ * converges.  An ensemble of CP2 systems whose cell graphs all have two colours
+ * runs, in either precision, FP64 CG on their Schur complements (two Jacobi
+ * iterations a step, counted as two; see CPS_PATH_AUTO).  Else the iteration
+ * is the single-reduction (Chronopoulos-Gear) form
  * of Jacobi CG, restarted from the true residual up to 8 times.  A team
  * wait that runs out (about one second) gives CPS_ERR_TIMEOUT.  With
  * cps_set_batch_path(ctx, CPS_BATCH_GRAPH) instead one launch per phase for

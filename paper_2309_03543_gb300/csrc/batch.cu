@@ -357,7 +357,8 @@ struct TeamPlan {
 // teams[t].sys (rows split in multiples of 32).  Then every block takes whole
 // systems in the order `order` (largest estimated work first) from the
 // counter *next until none is left.  FP64 or mixed precision.
-template <bool MIXED>
+// FORM: 0 FP64 and 1 mixed Jacobi on all cells, 2 every system on its Schur rows.
+template <int FORM>
 __global__ void __launch_bounds__(kBB, 2) kb_one_launch(const BatchDesc* __restrict__ dd,
                                                         const int* __restrict__ order, int nqueue,
                                                         int* next,
@@ -366,30 +367,42 @@ __global__ void __launch_bounds__(kBB, 2) kb_one_launch(const BatchDesc* __restr
                                                         long long max_iter) {
     __shared__ int s_k;
     __shared__ TeamCtx s_tc;
-    for (int t = 0; t < nteams; ++t) {
-        const TeamPlan tp = teams[t];
-        const int rank = (int)blockIdx.x - tp.first;
-        if (rank < 0 || rank >= tp.k) continue;
-        const BatchDesc& d = dd[tp.sys];
-        const int64_t rows = ((d.n + tp.k - 1) / tp.k + 31) / 32 * 32;
-        const int64_t lo = min(d.n, (int64_t)rank * rows);
-        const int64_t hi = min(d.n, lo + rows);
-        if (threadIdx.x == 0)
-            s_tc = TeamCtx{sync + t, (unsigned long long)sync[t].stall, rank, tp.k, 0u};
-        __syncthreads();
-        if (MIXED) kbp_solve_mixed(d, lo, hi, &s_tc, rtol, max_iter);
-        else kbp_solve(d, lo, hi, &s_tc, rtol, max_iter);
-        break;
-    }
+    // first this block's team, if it is in one, then systems from the queue
+    bool queue = false;
     for (;;) {
-        __syncthreads();
-        if (threadIdx.x == 0) s_k = atomicAdd(next, 1);
-        __syncthreads();
-        const int k = s_k;
-        if (k >= nqueue) return;
-        const BatchDesc& d = dd[order[k]];
-        if (MIXED) kbp_solve_mixed(d, 0, d.n, nullptr, rtol, max_iter);
-        else kbp_solve(d, 0, d.n, nullptr, rtol, max_iter);
+        const BatchDesc* d = nullptr;
+        TeamCtx* tc = nullptr;
+        int rank = 0, k = 1;
+        if (!queue) {
+            queue = true;
+            for (int t = 0; t < nteams && !d; ++t) {
+                const TeamPlan tp = teams[t];
+                rank = (int)blockIdx.x - tp.first;
+                if (rank < 0 || rank >= tp.k) continue;
+                d = dd + tp.sys;
+                k = tp.k;
+                tc = &s_tc;
+                if (threadIdx.x == 0)
+                    s_tc = TeamCtx{sync + t, (unsigned long long)sync[t].stall, rank, k, 0u};
+            }
+            __syncthreads();
+            if (!d) continue;
+        } else {
+            __syncthreads();
+            if (threadIdx.x == 0) s_k = atomicAdd(next, 1);
+            __syncthreads();
+            if (s_k >= nqueue) return;
+            d = dd + order[s_k];
+        }
+        if (FORM == 2) {
+            kbp_solve_tc(*d, rank, k, tc, rtol, max_iter);
+        } else {
+            const int64_t rows = k == 1 ? d->n : ((d->n + k - 1) / k + 31) / 32 * 32;
+            const int64_t lo = min(d->n, (int64_t)rank * rows);
+            const int64_t hi = min(d->n, lo + rows);
+            if (FORM == 1) kbp_solve_mixed(*d, lo, hi, tc, rtol, max_iter);
+            else kbp_solve(*d, lo, hi, tc, rtol, max_iter);
+        }
     }
 }
 
@@ -562,7 +575,31 @@ static int solve_batch_one_launch(const cps_sys* systems, int nsys, const double
         d.st = s->st;
         d.n = s->nt;
     }
-    const void* kernel = mixed ? (const void*)kb_one_launch<true> : (const void*)kb_one_launch<false>;
+    // An ensemble of two-coloured CP2 systems runs on their Schur rows, in either
+    // precision (see schur.cu and mixed_two_cyclic); any other on all cells.
+    bool tc = true;
+    for (int i = 0; i < nsys && tc; ++i) {
+        cps_sys s = systems[i];
+        int rc = CPS_OK;
+        if (s->kind != CPS_KIND_CP2) tc = false;
+        else rc = two_colour_order(s, stream, &tc);
+        if (rc == CPS_OK && tc) rc = schur_setup(s, false, stream);
+        if (rc == CPS_ERR_NOMEM) {              // no room for the rows
+            cudaGetLastError();
+            tc = false;
+        } else if (rc) {
+            return rc;
+        }
+        if (!tc) break;
+        hd[i].perm = s->perm;
+        hd[i].iperm = s->iperm;
+        hd[i].nR = s->colour_start[1];
+        hd[i].sch = s->sch;
+    }
+    if (tc) mixed = false;
+    const void* kernel = tc      ? (const void*)kb_one_launch<2>
+                         : mixed ? (const void*)kb_one_launch<1>
+                                 : (const void*)kb_one_launch<0>;
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kBB, 0) !=
             cudaSuccess || per_sm < 1) {
@@ -720,7 +757,6 @@ int solve_batch_impl(const cps_sys* systems, int nsys, const double* const* b,
         d.st = s->st;
         d.n = s->nt;
         d.ntiles = (int32_t)((s->nt + kTileRows - 1) / kTileRows);
-        d.pad = 0;
         if (d.ntiles > 4 * kMaxGrid) {
             cps::set_error(ctx, "solve_batch: a system is too large for the batched path");
             return CPS_ERR_ARG;

@@ -33,6 +33,10 @@ struct BatchDesc {
     int64_t n;
     int32_t ntiles;
     int32_t pad;
+    const int32_t* perm;          // Schur rows: colour order, inverse, first black position
+    const int32_t* iperm;
+    int64_t nR;
+    SchurData sch;
 };
 
 // ---- The ensemble in one launch.  The systems are independent, so they need
@@ -420,6 +424,252 @@ __device__ __forceinline__ bool kbp_solve(const BatchDesc& d, int64_t lo, int64_
         st->bnorm2 = sc.bnorm2;
         st->thresh2 = sc.thresh2;
         st->status = ok ? sc.status : CPS_ERR_TIMEOUT;
+        st->done = 2;
+    }
+    __syncthreads();
+    return ok;
+}
+
+// One system on its explicit Schur rows (see schur.cu: two Jacobi iterations
+// are one CG iteration on S, half of the rows), by this block (tc null) or this
+// member's share (rank of k) of the red cells, of the black rows and of the
+// cells of either colour.  The recurrences, restarts, results and the return
+// value are kbp_solve's, iterations counted two a step; per step one pass over
+// the rows of S (80 B and 9 FP64 FMAs a row) and one over the vectors.
+__device__ __forceinline__ bool kbp_solve_tc(const BatchDesc& d, int rank, int k, TeamCtx* tc,
+                                             double rtol, long long max_iter) {
+    __shared__ SolveScalars sc;
+    const int64_t n = d.n, ld = d.sch.ld;
+    const int nR = (int)d.nR, nB = (int)(n - d.nR);
+    const int rr_ = ((nR + k - 1) / k + 31) & ~31, rb_ = ((nB + k - 1) / k + 31) & ~31;
+    const int rlo = (int)min((int64_t)nR, (int64_t)rank * rr_), rhi = min(nR, rlo + rr_);
+    const int lo = (int)min((int64_t)nB, (int64_t)rank * rb_), hi = min(nB, lo + rb_);
+    const double* __restrict__ A = d.a;
+    const int32_t* __restrict__ C = d.col;
+    const double* __restrict__ S = d.s;
+    const double* __restrict__ V = d.sch.v;
+    const int32_t* __restrict__ Q = d.sch.c;
+    const double* __restrict__ D = d.sch.d;
+    const int32_t* __restrict__ perm = d.perm;
+    double* __restrict__ yb = d.sch.y;
+    double* __restrict__ r = d.sch.r;
+    double* __restrict__ p = d.sch.p;
+    double* __restrict__ sv = d.sch.s;
+    double* __restrict__ w = d.sch.w;
+    double* __restrict__ y = d.y;
+    bool ok = true;               // false once a team wait ran out
+    auto sum1 = [&](double (&v)[1]) {
+        if (tc) ok = team_sum<1>(v, *tc) && ok;
+        else block_sum_exact<1, kBB>(v);
+    };
+    auto sum3 = [&](double (&v)[3]) {
+        if (tc) ok = team_sum<3>(v, *tc) && ok;
+        else block_sum_exact<3, kBB>(v);
+    };
+    auto barrier = [&]() {
+        if (tc) ok = team_barrier(*tc) && ok;
+        else __syncthreads();
+    };
+    if (threadIdx.x == 0) {
+        sc.total = 0;
+        sc.it = 0;
+        sc.status = CPS_OK;
+        sc.bnorm2 = sc.rnorm2 = sc.thresh2 = 0.0;
+    }
+    for (int round = 0; round < 8; ++round) {
+        // y_R = b / s - E (S x)_B, then r_B = bhat - (S x)_B - E^T y_R
+        double v3[3] = {0.0, 0.0, 0.0};
+        for (int i = rlo + (int)threadIdx.x; i < rhi; i += kBB) {
+            const int32_t e = perm[i];
+            const double be = d.b[e];
+            double acc = be / S[e];
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                const int32_t c = C[j * n + e];
+                if (c != e) acc = fma(-A[j * n + e], S[c] * d.x[c], acc);
+            }
+            y[e] = acc;
+            v3[1] = fma(be, be, v3[1]);
+        }
+        barrier();
+        if (!ok) break;
+        for (int i = lo + (int)threadIdx.x; i < hi; i += kBB) {
+            const int32_t e = perm[nR + i];
+            const double se = S[e];
+            const double ye = se * d.x[e];
+            double ay = ye;
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                const int32_t c = C[j * n + e];
+                if (c != e) ay = fma(A[j * n + e], y[c], ay);
+            }
+            const double be = d.b[e];
+            const double re = be / se - ay;
+            yb[i] = ye;
+            r[i] = re;
+            p[i] = 0.0;
+            sv[i] = 0.0;
+            v3[0] = fma(re, re, v3[0]);
+            v3[1] = fma(be, be, v3[1]);
+            const double t = se * re;
+            v3[2] = fma(t, t, v3[2]);
+        }
+        sum3(v3);                 // also the barrier before r is read elsewhere
+        if (!ok) break;
+        if (threadIdx.x == 0) {
+            sc.bnorm2 = v3[1];
+            sc.thresh2 = rtol * rtol * v3[1];
+            sc.rnorm2 = v3[2];
+            sc.budget = max_iter - sc.total;
+            sc.it = 0;
+            sc.ig = sc.c = 0.0;
+            sc.flag = v3[1] == 0.0 ? 3
+                      : (v3[2] > sc.thresh2 && sc.budget > 0 && v3[0] > 0.0) ? 0 : 1;
+        }
+        __syncthreads();
+        if (sc.flag == 3) {           // b = 0: x = 0
+            for (int i = rlo + (int)threadIdx.x; i < rhi; i += kBB) d.x[perm[i]] = 0.0;
+            for (int i = lo + (int)threadIdx.x; i < hi; i += kBB) d.x[perm[nR + i]] = 0.0;
+            if (threadIdx.x == 0) sc.rnorm2 = 0.0;
+            break;
+        }
+        while (sc.flag == 0) {
+            const bool check = (sc.it & 7) == 7;
+            double g3[3] = {0.0, 0.0, 0.0};
+            for (int i = lo + (int)threadIdx.x; i < hi; i += kBB) {
+                const int f = i + kBB;
+                if (f < hi) {
+#pragma unroll
+                    for (int j = 0; j < 6; ++j) {
+                        pf_l1(V + j * ld + f);
+                        pf_l1(Q + j * ld + f);
+                    }
+                    pf_l1(D + f);
+                    pf_l1(r + f);
+                }
+                double v[6], g[6];
+                int32_t c[6];
+#pragma unroll
+                for (int j = 0; j < 6; ++j) {
+                    c[j] = Q[j * ld + i];
+                    v[j] = V[j * ld + i];
+                }
+                const double re = r[i], dd = D[i];
+#pragma unroll
+                for (int j = 0; j < 6; ++j) g[j] = r[c[j]];
+                double acc = dd * re;
+#pragma unroll
+                for (int j = 0; j < 6; ++j) acc = fma(v[j], g[j], acc);
+                w[i] = acc;
+                g3[0] = fma(re, re, g3[0]);
+                g3[1] = fma(acc, re, g3[1]);
+                if (check) {
+                    const double t = d.sch.wt[i] * re;
+                    g3[2] = fma(t, t, g3[2]);
+                }
+            }
+            sum3(g3);
+            if (!ok) break;
+            if (threadIdx.x == 0) {
+                const double g = g3[0], dl = g3[1];
+                bool halt = !(g > 0.0) || 2 * sc.it >= sc.budget;
+                if (check) {
+                    sc.rnorm2 = g3[2];
+                    if (g3[2] <= sc.thresh2) halt = true;
+                }
+                int f = halt ? 1 : 0;
+                if (!halt) {
+                    const double den = sc.it == 0 ? dl : fma(-(g * g), sc.c, dl);
+                    if (!(den > 0.0) || !isfinite(den)) {
+                        // on a round's first pass p.Sp <= 0: not SPD; later the
+                        // recurrence lost its digits at the FP64 floor: stop,
+                        // and let the true residual decide
+                        f = sc.it > 0 ? 1 : 2;
+                        if (f == 2) sc.status = CPS_ERR_NOT_SPD;
+                    } else {
+                        const double ig = 1.0 / g;
+                        sc.alpha = g / den;
+                        sc.beta = g * sc.ig;
+                        sc.ig = ig;
+                        sc.c = den * ig * ig;
+                    }
+                }
+                sc.gamma = g;
+                sc.flag = f;
+            }
+            __syncthreads();
+            if (sc.flag) break;
+            {
+                const double alpha = sc.alpha, beta = sc.beta;
+                double pe[2], se[2], we[2], re[2], ye[2];
+                CPS_BLK_LOOP(lo, hi, 2,
+                    (pf_l1(p + f), pf_l1(sv + f), pf_l1(w + f), pf_l1(r + f), pf_l1(yb + f)),
+                    (pe[u] = p[e], se[u] = sv[e], we[u] = w[e], re[u] = r[e], ye[u] = yb[e]),
+                    {
+                        const double pn = fma(beta, pe[u], re[u]);
+                        const double sn = fma(beta, se[u], we[u]);
+                        p[e] = pn;
+                        sv[e] = sn;
+                        yb[e] = fma(alpha, pn, ye[u]);
+                        r[e] = fma(-alpha, sn, re[u]);
+                    })
+            }
+            barrier();            // also orders thread 0's next writes of sc behind the reads
+            if (!ok) break;
+            if (threadIdx.x == 0) ++sc.it;
+            __syncthreads();
+        }
+        if (!ok) break;
+        // y of the whole system (black cells as they are, red recovered), then
+        // x = y / s and the true residual ||b - A x||^2 (every exit above
+        // follows a team-wide sum)
+        for (int i = lo + (int)threadIdx.x; i < hi; i += kBB) y[perm[nR + i]] = yb[i];
+        for (int i = rlo + (int)threadIdx.x; i < rhi; i += kBB) {
+            const int32_t e = perm[i];
+            double acc = d.b[e] / S[e];
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                const int32_t c = C[j * n + e];
+                if (c != e) acc = fma(-A[j * n + e], yb[d.iperm[c] - nR], acc);
+            }
+            y[e] = acc;
+        }
+        barrier();
+        if (!ok) break;
+        double nn[1] = {0.0};
+        auto finish = [&](int32_t e) {
+            const double se = S[e];
+            const double ye = y[e];
+            double ay = ye;
+#pragma unroll
+            for (int j = 0; j < 3; ++j) ay = fma(A[j * n + e], y[C[j * n + e]], ay);
+            const double res = d.b[e] - se * ay;
+            d.x[e] = ye / se;
+            nn[0] = fma(res, res, nn[0]);
+        };
+        for (int i = rlo + (int)threadIdx.x; i < rhi; i += kBB) finish(perm[i]);
+        for (int i = lo + (int)threadIdx.x; i < hi; i += kBB) finish(perm[nR + i]);
+        sum1(nn);
+        if (!ok) break;
+        if (threadIdx.x == 0) {
+            const long long left = max_iter - sc.total, made = 2 * sc.it;
+            sc.total += made < left ? made : left;
+            sc.it = 0;
+            sc.rnorm2 = nn[0];
+            sc.flag = (sc.status != CPS_OK || nn[0] <= sc.thresh2 || sc.total >= max_iter) ? 1 : 0;
+        }
+        __syncthreads();
+        if (sc.flag) break;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && rank == 0) {
+        CgState* st = d.st;
+        st->iter = sc.total + 2 * sc.it;
+        st->rnorm2 = sc.rnorm2;
+        st->bnorm2 = sc.bnorm2;
+        st->thresh2 = sc.thresh2;
+        st->status = ok ? sc.status : CPS_ERR_TIMEOUT;
+        st->updates = 1;
         st->done = 2;
     }
     __syncthreads();
