@@ -395,7 +395,7 @@ __global__ void __launch_bounds__(kBB, 2) kb_one_launch(const BatchDesc* __restr
             d = dd + order[s_k];
         }
         if (FORM == 2) {
-            kbp_solve_tc(*d, rank, k, tc, rtol, max_iter);
+            kbp_solve_tc(*d, rank, k, tc, rtol, max_iter, 7);
         } else {
             const int64_t rows = k == 1 ? d->n : ((d->n + k - 1) / k + 31) / 32 * 32;
             const int64_t lo = min(d->n, (int64_t)rank * rows);

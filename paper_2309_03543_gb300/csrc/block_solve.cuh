@@ -435,9 +435,10 @@ __device__ __forceinline__ bool kbp_solve(const BatchDesc& d, int64_t lo, int64_
 // member's share (rank of k) of the red cells, of the black rows and of the
 // cells of either colour.  The recurrences, restarts, results and the return
 // value are kbp_solve's, iterations counted two a step; per step one pass over
-// the rows of S (80 B and 9 FP64 FMAs a row) and one over the vectors.
+// the rows of S (80 B and 9 FP64 FMAs a row) and one over the vectors.  The
+// stop test runs on the steps whose low bits are all set in mask.
 __device__ __forceinline__ bool kbp_solve_tc(const BatchDesc& d, int rank, int k, TeamCtx* tc,
-                                             double rtol, long long max_iter) {
+                                             double rtol, long long max_iter, int mask) {
     __shared__ SolveScalars sc;
     const int64_t n = d.n, ld = d.sch.ld;
     const int nR = (int)d.nR, nB = (int)(n - d.nR);
@@ -534,7 +535,7 @@ __device__ __forceinline__ bool kbp_solve_tc(const BatchDesc& d, int rank, int k
             break;
         }
         while (sc.flag == 0) {
-            const bool check = (sc.it & 7) == 7;
+            const bool check = ((int)sc.it & mask) == mask;
             double g3[3] = {0.0, 0.0, 0.0};
             for (int i = lo + (int)threadIdx.x; i < hi; i += kBB) {
                 const int f = i + kBB;

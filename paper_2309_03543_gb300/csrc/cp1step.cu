@@ -184,7 +184,10 @@ struct Cp1DevArgs {
     int64_t nt;
 };
 
-template <bool MIXED>
+// FORM: 0 FP64 and 1 mixed Jacobi on all cells, 2 both systems on their Schur
+// rows.  The mass term makes a solve about eight Jacobi iterations, four steps
+// on S: a stop test every step, not every eighth.
+template <int FORM>
 __global__ void __launch_bounds__(kBB, 2) k_cp1_step(Cp1DevArgs P) {
     __shared__ TeamCtx s_tc;
     __shared__ int s_stop;
@@ -219,8 +222,10 @@ __global__ void __launch_bounds__(kBB, 2) k_cp1_step(Cp1DevArgs P) {
         if (!ok) break;
         // the two solves, each by the whole grid, warm-started from du
         for (int k = 0; k < 2 && ok; ++k)
-            ok = (MIXED ? kbp_solve_mixed(P.sys[k], lo, hi, &s_tc, P.rtol, P.max_iter)
-                        : kbp_solve(P.sys[k], lo, hi, &s_tc, P.rtol, P.max_iter)) && ok;
+            ok = (FORM == 2   ? kbp_solve_tc(P.sys[k], (int)blockIdx.x, G, &s_tc, P.rtol,
+                                             P.max_iter, 0)
+                  : FORM == 1 ? kbp_solve_mixed(P.sys[k], lo, hi, &s_tc, P.rtol, P.max_iter)
+                              : kbp_solve(P.sys[k], lo, hi, &s_tc, P.rtol, P.max_iter)) && ok;
         if (!ok) break;
         // every block: the change sums of its rows (du final everywhere after
         // the team sum that ends each solve), one exact team sum; the solves'
@@ -381,7 +386,23 @@ static int cp1_step_one_launch(cps_sys sx, cps_sys sy, double* du, double toll,
                                cps_cp1_stats* stats, cudaStream_t stream) {
     Cp1Data* c = sx->cp1;
     const int64_t nt = sx->nt;
-    const void* kernel = mixed ? (const void*)k_cp1_step<true> : (const void*)k_cp1_step<false>;
+    // on the Schur rows where the cell graph has two colours (one for both systems)
+    bool tc = true;
+    cps_sys sys[2] = {sx, sy};
+    for (cps_sys s : sys) {
+        int rc = two_colour_order(s, stream, &tc);
+        if (rc == CPS_OK && tc) rc = schur_setup(s, false, stream);
+        if (rc == CPS_ERR_NOMEM) {              // no room for the rows
+            cudaGetLastError();
+            tc = false;
+        } else if (rc) {
+            return rc;
+        }
+        if (!tc) break;
+    }
+    const void* kernel = tc      ? (const void*)k_cp1_step<2>
+                         : mixed ? (const void*)k_cp1_step<1>
+                                 : (const void*)k_cp1_step<0>;
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kBB, 0) != cudaSuccess ||
         per_sm < 1) {
@@ -395,7 +416,6 @@ static int cp1_step_one_launch(cps_sys sx, cps_sys sy, double* du, double toll,
     hs.stall = sx->inject == CPS_TEST_STALL_BARRIER ? 1 : 0;   // test hook, one-shot
     sx->inject = 0;
     BatchDesc hd[2];
-    cps_sys sys[2] = {sx, sy};
     for (int k = 0; k < 2; ++k) {
         cps_sys s = sys[k];
         BatchDesc& d = hd[k];
@@ -416,6 +436,12 @@ static int cp1_step_one_launch(cps_sys sx, cps_sys sy, double* du, double toll,
         d.partials = s->partials;
         d.st = s->st;
         d.n = nt;
+        if (tc) {
+            d.perm = s->perm;
+            d.iperm = s->iperm;
+            d.nR = s->colour_start[1];
+            d.sch = s->sch;
+        }
     }
     Cp1DevArgs a{};
     a.lap = c->lap;
