@@ -8,6 +8,7 @@
 #include "exact_sum.cuh"
 
 #include <cstdint>
+#include <type_traits>
 
 namespace cps {
 namespace {
@@ -209,7 +210,7 @@ struct SolveScalars {
 
 // w = Ahat r on rows [lo, hi) with gamma = r.r, delta = w.r and, if check,
 // ||S r||^2 into v[0..3).
-#define CPS_BLK_SPMV_W(lo, hi, check, v)                                               \
+#define CPS_BLK_SPMV_W_(lo, hi, check, v)                                              \
     {                                                                                  \
         double re[2], a0[2], a1[2], a2[2];                                             \
         int32_t c0[2], c1[2], c2[2];                                                   \
@@ -231,6 +232,12 @@ struct SolveScalars {
                 }                                                                      \
             })                                                                         \
     }
+
+// (a loop of its own for the passes that test: predicated FP64 instructions take
+// their turns on the pipe)
+#define CPS_BLK_SPMV_W(lo, hi, check, v)                                               \
+    if (check) CPS_BLK_SPMV_W_(lo, hi, true, v)                                        \
+    else CPS_BLK_SPMV_W_(lo, hi, false, v)
 
 // One system, rows [lo, hi) solved by this block: the whole system (tc null)
 // or this member's slice of a team's system (tc in shared memory).  FP64
@@ -537,38 +544,43 @@ __device__ __forceinline__ bool kbp_solve_tc(const BatchDesc& d, int rank, int k
         while (sc.flag == 0) {
             const bool check = ((int)sc.it & mask) == mask;
             double g3[3] = {0.0, 0.0, 0.0};
-            for (int i = lo + (int)threadIdx.x; i < hi; i += kBB) {
-                const int f = i + kBB;
-                if (f < hi) {
-#pragma unroll
-                    for (int j = 0; j < 6; ++j) {
-                        pf_l1(V + j * ld + f);
-                        pf_l1(Q + j * ld + f);
+            // (a loop of its own for the passes that test: see k_resident_cg)
+            auto product = [&](auto test) {
+                for (int i = lo + (int)threadIdx.x; i < hi; i += kBB) {
+                    const int f = i + kBB;
+                    if (f < hi) {
+    #pragma unroll
+                        for (int j = 0; j < 6; ++j) {
+                            pf_l1(V + j * ld + f);
+                            pf_l1(Q + j * ld + f);
+                        }
+                        pf_l1(D + f);
+                        pf_l1(r + f);
                     }
-                    pf_l1(D + f);
-                    pf_l1(r + f);
+                    double v[6], g[6];
+                    int32_t c[6];
+    #pragma unroll
+                    for (int j = 0; j < 6; ++j) {
+                        c[j] = Q[j * ld + i];
+                        v[j] = V[j * ld + i];
+                    }
+                    const double re = r[i], dd = D[i];
+    #pragma unroll
+                    for (int j = 0; j < 6; ++j) g[j] = r[c[j]];
+                    double acc = dd * re;
+    #pragma unroll
+                    for (int j = 0; j < 6; ++j) acc = fma(v[j], g[j], acc);
+                    w[i] = acc;
+                    g3[0] = fma(re, re, g3[0]);
+                    g3[1] = fma(acc, re, g3[1]);
+                    if constexpr (decltype(test)::value) {
+                        const double t = d.sch.wt[i] * re;
+                        g3[2] = fma(t, t, g3[2]);
+                    }
                 }
-                double v[6], g[6];
-                int32_t c[6];
-#pragma unroll
-                for (int j = 0; j < 6; ++j) {
-                    c[j] = Q[j * ld + i];
-                    v[j] = V[j * ld + i];
-                }
-                const double re = r[i], dd = D[i];
-#pragma unroll
-                for (int j = 0; j < 6; ++j) g[j] = r[c[j]];
-                double acc = dd * re;
-#pragma unroll
-                for (int j = 0; j < 6; ++j) acc = fma(v[j], g[j], acc);
-                w[i] = acc;
-                g3[0] = fma(re, re, g3[0]);
-                g3[1] = fma(acc, re, g3[1]);
-                if (check) {
-                    const double t = d.sch.wt[i] * re;
-                    g3[2] = fma(t, t, g3[2]);
-                }
-            }
+            };
+            if (check) product(std::true_type{});
+            else product(std::false_type{});
             sum3(g3);
             if (!ok) break;
             if (threadIdx.x == 0) {

@@ -35,6 +35,7 @@
 
 #include <cmath>
 #include <cstddef>
+#include <type_traits>
 
 namespace cps {
 namespace {
@@ -334,15 +335,19 @@ __global__ void __launch_bounds__(kPBlock, 1) k_persistent_cg(PersistArgs P) {
         double rr[2] = {0.0, 0.0};
         {
             double qe[kUV], re0[kUV];
-            CPS_B_LOOP(lo, hi, kUV, (qe[u] = q[e], re0[u] = r[e]), {
-                const double re = fma(-alpha, qe[u], re0[u]);
-                r[e] = re;
-                rr[0] = fma(re, re, rr[0]);
-                if (check) {
-                    const double tt = P.s[e] * re;
-                    rr[1] = fma(tt, tt, rr[1]);
-                }
-            })
+            auto update = [&](auto test) {
+                CPS_B_LOOP(lo, hi, kUV, (qe[u] = q[e], re0[u] = r[e]), {
+                    const double re = fma(-alpha, qe[u], re0[u]);
+                    r[e] = re;
+                    rr[0] = fma(re, re, rr[0]);
+                    if constexpr (decltype(test)::value) {
+                        const double tt = P.s[e] * re;
+                        rr[1] = fma(tt, tt, rr[1]);
+                    }
+                })
+            };
+            if (check) update(std::true_type{});
+            else update(std::false_type{});
         }
         double sb[1];
         int stop = 0;
@@ -708,15 +713,19 @@ __global__ void __launch_bounds__(kPBlock, 1) k_persistent_reduced(PersistArgs P
         double rr[2] = {0.0, 0.0};
         {
             double qe[kUV], re0[kUV];
-            CPS_B_LOOP(blo, bhi, kUV, (qe[u] = q[e], re0[u] = r[e]), {
-                const double re = fma(-alpha, qe[u], re0[u]);
-                r[e] = re;
-                rr[0] = fma(re, re, rr[0]);
-                if (check) {
-                    const double tt = P.s[e] * re;
-                    rr[1] = fma(tt, tt, rr[1]);
-                }
-            })
+            auto update = [&](auto test) {
+                CPS_B_LOOP(blo, bhi, kUV, (qe[u] = q[e], re0[u] = r[e]), {
+                    const double re = fma(-alpha, qe[u], re0[u]);
+                    r[e] = re;
+                    rr[0] = fma(re, re, rr[0]);
+                    if constexpr (decltype(test)::value) {
+                        const double tt = P.s[e] * re;
+                        rr[1] = fma(tt, tt, rr[1]);
+                    }
+                })
+            };
+            if (check) update(std::true_type{});
+            else update(std::false_type{});
         }
         double sb[1];
         int stop = 0;
