@@ -343,27 +343,48 @@ __global__ void k_dxi_dtheta(const double* __restrict__ eps, const double* __res
 
 }  // namespace
 
-template <typename T>
-static int dev_alloc(cps_ctx ctx, T** p, size_t n) {
-    cudaError_t e = cudaMalloc((void**)p, sizeof(T) * (n > 0 ? n : 1));
-    if (e != cudaSuccess) {
-        cps::set_error(ctx, std::string("cudaMalloc: ") + cudaGetErrorString(e));
-        *p = nullptr;
-        return CPS_ERR_NOMEM;
+// The arrays of a new system as slices of one allocation (a call to the
+// driver costs more than most of the assembly's kernels), 256-byte aligned.
+namespace {
+struct Slab {
+    struct Slice {
+        void** p;
+        size_t bytes;
+    };
+    Slice slices[16];
+    int count = 0;
+    size_t total = 0;
+    template <typename T>
+    void add(T** p, size_t n) {
+        const size_t bytes = (sizeof(T) * (n > 0 ? n : 1) + 255) & ~(size_t)255;
+        slices[count++] = {reinterpret_cast<void**>(p), bytes};
+        total += bytes;
     }
-    return CPS_OK;
-}
+    int allocate(cps_ctx ctx, void** base) {
+        cudaError_t e = cudaMalloc(base, total);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            *base = nullptr;
+            cps::set_error(ctx, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+            return CPS_ERR_NOMEM;
+        }
+        char* at = static_cast<char*>(*base);
+        for (int i = 0; i < count; ++i) {
+            *slices[i].p = at;
+            at += slices[i].bytes;
+        }
+        return CPS_OK;
+    }
+};
+}  // namespace
 
 void free_sys(cps_sys s) {
     if (!s) return;
     free_cp2(s);
     free_cp1(s);
     free_schur(s);
-    // s->col lives inside s->a's allocation (one range for the L2 window)
-    void* bufs[] = {s->off, s->s,     s->diag,  s->a,     s->a32,     s->s32,      s->gfac,
-                    s->dxi,   s->slot_kind, s->perm, s->iperm, s->pa,  s->pcol,     s->pl,
-                    s->pdinv, s->pdiag, s->ps, s->pa32, s->pl32, s->pdinv32, s->ps32,   s->wvec,
-                    s->partials, s->st, s->gsync};
+    void* bufs[] = {s->slab, s->perm, s->iperm, s->pa,   s->pcol, s->pl,      s->pdinv,
+                    s->pdiag, s->ps,  s->pa32,  s->pl32, s->pdinv32, s->ps32, s->gsync};
     for (void* b : bufs)
         if (b) cudaFree(b);
     if (s->hst) cudaFreeHost(s->hst);
@@ -411,29 +432,32 @@ int assemble_impl(cps_ctx ctx, const double* xy, int64_t nv, const int32_t* tri,
     s->dt = dt;
     const int64_t nf = field_loc == CPS_PER_VERTEX ? nv : nt;
     int rc = CPS_OK;
-#define TRY_ALLOC(p, n)                        \
-    do {                                       \
-        rc = dev_alloc(ctx, &(p), (size_t)(n)); \
-        if (rc) goto fail_free;                \
-    } while (0)
-    TRY_ALLOC(s->s, nt);
-    TRY_ALLOC(s->diag, nt);
-    // Off-diagonal values and columns in one allocation: a [3 nt] doubles,
-    // then col [3 nt] int32 (256-byte aligned), so that one L2 access-policy
-    // window covers the whole matrix the iteration streams.
     {
+        Slab slab;
+        slab.add(&s->s, nt);
+        slab.add(&s->diag, nt);
+        // Off-diagonal values and columns in one slice: a [3 nt] doubles, then
+        // col [3 nt] int32 (256-byte aligned), so that one L2 access-policy
+        // window covers the whole matrix the iteration streams.
         const size_t a_elems = ((size_t)3 * nt + 31) / 32 * 32;
         const size_t col_elems = ((size_t)3 * nt * sizeof(int32_t) + sizeof(double) - 1) / sizeof(double);
-        TRY_ALLOC(s->a, a_elems + col_elems);
+        slab.add(&s->a, a_elems + col_elems);
+        slab.add(&s->off, 3 * nt);
+        slab.add(&s->a32, 3 * nt);
+        slab.add(&s->s32, nt);
+        slab.add(&s->slot_kind, 3 * nt);
+        const int64_t vs = (nt + 31) / 32 * 32;     // 256-byte aligned vectors
+        slab.add(&s->wvec, 9 * vs);
+        slab.add(&s->partials, (kNumPartials + 16) * kMaxGrid);
+        slab.add(&s->st, 2);
+        if (field_loc == CPS_PER_CELL && kind == CPS_KIND_CP2) {
+            slab.add(&s->gfac, 3 * nt);
+            slab.add(&s->dxi, nt);
+        }
+        rc = slab.allocate(ctx, &s->slab);
+        if (rc) goto fail_free;
         s->col = reinterpret_cast<int32_t*>(s->a + a_elems);
         s->mat_bytes = (a_elems + col_elems) * sizeof(double);
-    }
-    TRY_ALLOC(s->a32, 3 * nt);
-    TRY_ALLOC(s->s32, nt);
-    TRY_ALLOC(s->slot_kind, 3 * nt);
-    {
-        const int64_t vs = (nt + 31) / 32 * 32;     // 256-byte aligned slices
-        TRY_ALLOC(s->wvec, 9 * vs);
         s->vec_stride = vs;
         double* w = s->wvec;
         s->wr = w;
@@ -446,14 +470,6 @@ int assemble_impl(cps_ctx ctx, const double* xy, int64_t nv, const int32_t* tri,
         s->wx = w + 7 * vs;
         s->wbest = w + 8 * vs;
     }
-    TRY_ALLOC(s->off, 3 * nt);
-    TRY_ALLOC(s->partials, (kNumPartials + 16) * kMaxGrid);
-    TRY_ALLOC(s->st, 2);
-    if (field_loc == CPS_PER_CELL && kind == CPS_KIND_CP2) {
-        TRY_ALLOC(s->gfac, 3 * nt);
-        TRY_ALLOC(s->dxi, nt);
-    }
-#undef TRY_ALLOC
     {
         cudaError_t e = cudaMallocHost((void**)&s->hst, 2 * sizeof(CgState));
         if (e != cudaSuccess) { rc = fail(ctx, CPS_ERR_NOMEM, "cudaMallocHost failed"); goto fail_free; }

@@ -307,14 +307,16 @@ struct cps_sys_s {
     cps::Cp1Data* cp1 = nullptr;  // CP1 step data (cps_cp1_setup, on the x system)
     int64_t assembly_launches = 0;
 
+    void* slab = nullptr;       // the allocation that holds the matrix, the adjoint's
+                                // factors, the workspace, partials and state
     // Matrix in symmetrically scaled padded-ELL form: A = S (I + Aoff) S with
     // S = diag(s), s = sqrt(diag(A)); slot-major arrays [3][nt].
     double* s = nullptr;        // [nt]
     double* diag = nullptr;     // [nt] unscaled diagonal (export / info)
-    double* a = nullptr;        // [3*nt] scaled off-diagonals (allocation also holds col)
+    double* a = nullptr;        // [3*nt] scaled off-diagonals (slice also holds col)
     int32_t* col = nullptr;     // [3*nt] column (= row for an unused slot)
     double* off = nullptr;      // [3*nt] unscaled off-diagonals (matvec, export)
-    size_t mat_bytes = 0;       // bytes of the a + col allocation
+    size_t mat_bytes = 0;       // bytes of the a + col slice
     float* a32 = nullptr;       // [3*nt] binary32 copy of a (mixed precision)
     float* s32 = nullptr;       // [nt]
     // Adjoint: per slot dT/dxi_e, per cell dxi/dtheta (CP2, cell fields).
@@ -343,7 +345,7 @@ struct cps_sys_s {
     float* ps32 = nullptr;
 
     // PCG workspace (allocated at assembly so that solves never allocate), one
-    // allocation of 9 vectors of vec_stride doubles in the order r, p0, q, y,
+    // slice of 9 vectors of vec_stride doubles in the order r, p0, q, y,
     // p1, z, b, x, best: r, p0 and q, the vectors every iteration reads and
     // writes, are one contiguous range for an L2 access-policy window.
     double* wvec = nullptr;
