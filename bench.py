@@ -778,8 +778,8 @@ def sequence_summary(n: int, rtol: float, iters: int = 200) -> dict:
         x.zero_()
         t, st = timed(lambda: s.solve(rhs[0], x=x, rtol=rtol, max_iter=iters, precision=prec,
                                       check=False)[1], stream)
-        if prec == cps.FP64 or s.tuning(cps.FP64).get("two_cyclic"):
-            bpc = method_bytes(name.split("_")[0], s.tuning(cps.FP64))
+        # (under the automatic path a FP64 loop serves the mixed solves too)
+        bpc = method_bytes(name.split("_")[0], s.tuning(cps.FP64))
         gbs = bpc * nt * st.iters / t / 1e9
         out[name] = {"iters": st.iters, "us_per_iter": 1e6 * t / max(st.iters, 1),
                      "bytes_per_cell_iter": bpc, "algorithmic_gbs": gbs, "frac": gbs / peak}
@@ -850,9 +850,8 @@ def run_sequence(args):
             rel.append(st.rel_res)
             status.append(st.status)
             per.append(dt_)
-        tf = s.tuning(cps.FP64)
-        if prec == cps.FP64 or tf.get("two_cyclic"):
-            bpc = method_bytes("jacobi" if name == "mixed" else name, tf)
+        # (under the automatic path a FP64 loop serves the mixed solves too)
+        bpc = method_bytes("jacobi" if name == "mixed" else name, s.tuning(cps.FP64))
         # reduced system: iterations run over the black half of the cells
         units = nt // 2 if pc == cps.PC_REDUCED else nt
         gbs = bpc * nt * it_tot / t_tot / 1e9

@@ -170,8 +170,8 @@ int cps_export_matrix(cps_sys sys, double* diag, int32_t* col, double* val, void
  *   precision   CPS_FP64 or CPS_MIXED (binary32 matrix, vectors and SpMV in
  *               the inner PCG; binary64 dot products, alpha/beta, and the
  *               outer residual b - A x and update of x; under CPS_PATH_AUTO a
- *               CP2 system whose cell graph has two colours takes the FP64
- *               two-cyclic loop instead, which is faster: see CPS_PATH_AUTO)
+ *               CP2 system takes the FP64 loop instead where that is faster:
+ *               with Jacobi, and with IC(0) in a two-colour order)
  *   stats       host pointer, may be NULL
  * b = 0 gives x = 0.  Errors: CPS_ERR_ARG, _NOT_SPD, _NOT_CONVERGED (x holds
  * the last iterate; CPS_MIXED: the iterate with the least true residual, with
@@ -193,9 +193,10 @@ int cps_solve(cps_sys sys, const double* b, double* x, double rtol, int64_t max_
  * block takes whole systems from a device work queue (largest first) and
  * solves each with block-level reductions only; a team's blocks join the
  * queue when their system is done, and every system stops as soon as it
- * converges.  An ensemble of CP2 systems whose cell graphs all have two colours
- * runs, in either precision, FP64 CG on their Schur complements (two Jacobi
- * iterations a step, counted as two; see CPS_PATH_AUTO).  Else the iteration
+ * converges.  An ensemble of CP2 systems runs in FP64 in either precision, and
+ * where all its cell graphs have two colours as CG on their Schur complements
+ * (two Jacobi iterations a step, counted as two; see CPS_PATH_AUTO).  Else the
+ * iteration
  * is the single-reduction (Chronopoulos-Gear) form
  * of Jacobi CG, restarted from the true residual up to 8 times.  A team
  * wait that runs out (about one second) gives CPS_ERR_TIMEOUT.  With
@@ -402,7 +403,7 @@ int cps_cp2_kernel_times(cps_sys sys, float* ms);
  * FP64 IC(0) in a two-colour order runs on the streaming kernels for every
  * other pin, and CPS_PATH_AUTO times both ways on the first such solve; with
  * more colours it always streams.
- * Mixed precision streams, but for CPS_PATH_AUTO's two-cyclic form. */
+ * Mixed precision streams, where CPS_PATH_AUTO does not take a FP64 loop for it. */
 #define CPS_PATH_AUTO 0
 #define CPS_PATH_STREAM 1
 #define CPS_PATH_CLUSTER 2

@@ -576,7 +576,7 @@ static int solve_batch_one_launch(const cps_sys* systems, int nsys, const double
         d.n = s->nt;
     }
     // An ensemble of two-coloured CP2 systems runs on their Schur rows, in either
-    // precision (see schur.cu and mixed_two_cyclic); any other on all cells.
+    // precision; any other on all cells.
     bool tc = true;
     for (int i = 0; i < nsys && tc; ++i) {
         cps_sys s = systems[i];
@@ -596,7 +596,11 @@ static int solve_batch_one_launch(const cps_sys* systems, int nsys, const double
         hd[i].nR = s->colour_start[1];
         hd[i].sch = s->sch;
     }
-    if (tc) mixed = false;
+    // FP64 on all cells beats the binary32 refinement there too (ensemble of 256,
+    // 4.0 against 6.6 s): see mixed_takes_fp64
+    bool cp2 = true;
+    for (int i = 0; i < nsys; ++i) cp2 = cp2 && systems[i]->kind == CPS_KIND_CP2;
+    if (tc || cp2) mixed = false;
     const void* kernel = tc      ? (const void*)kb_one_launch<2>
                          : mixed ? (const void*)kb_one_launch<1>
                                  : (const void*)kb_one_launch<0>;

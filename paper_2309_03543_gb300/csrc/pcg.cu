@@ -1416,28 +1416,16 @@ static int solve_reduced(cps_sys s, const double* b, double* x, double rtol, int
 
 // ------------------------------------------------------------------ mixed
 
-// CPS_MIXED on a two-coloured CP2 system under CPS_PATH_AUTO: the FP64 CG on
-// the Schur rows, *done true with the call's status.  The binary32 iteration
-// runs on all cells and needs 1.4 (160k cells) to 2.1 times (2.09M) the FP64
-// count; per Jacobi iteration it takes 20.6 us at 318k cells and 37.6 us at
-// 2.09M, the Schur loop 4.4 and 16.8.  So the more precise loop is the faster
-// one at every size (318k cells to 1e-10: 22.5 against 145 ms).
-static int mixed_two_cyclic(cps_sys s, const double* b, double* x, double rtol, int64_t max_iter,
-                            cps_stats* stats, cudaStream_t stream, bool* done) {
-    *done = false;
-    const bool ic0 = s->precond == CPS_PC_IC0;
-    if (s->tune[CPS_FP64].pinned || s->kind != CPS_KIND_CP2) return CPS_OK;
-    bool two = false;
-    int rc = two_colour_order(s, stream, &two);
-    if (rc == CPS_OK && two) rc = schur_setup(s, ic0, stream);
-    if (rc == CPS_ERR_NOMEM) {              // no room for the rows: the loop on all cells
-        cudaGetLastError();
-        return CPS_OK;
-    }
-    if (rc || !two) return rc;
-    *done = true;
-    rc = solve_two_cyclic(s, b, x, rtol, max_iter, ic0 ? 1 : 2, 0, false, stats, stream);
-    return rc;
+// CPS_MIXED on a CP2 system under CPS_PATH_AUTO, where a FP64 loop is the faster
+// one at every size measured: the binary32 iteration streams all cells in two
+// launches an iteration and needs 1.4 (160k cells) to 2.1 times (2.09M) the FP64
+// count, so it loses to the two-cyclic loop (318k cells to 1e-10: 23 against 144
+// ms) and, on graphs of more colours, to the FP64 Jacobi loops on all cells
+// (318k cells 55 against 138 ms, 2.09M 0.60 against 0.82 s).  With IC(0) that holds for two colours; with more, both
+// precisions stream the same sweeps and binary32 keeps its iteration.
+static bool mixed_takes_fp64(cps_sys s) {
+    if (s->tune[CPS_FP64].pinned || s->kind != CPS_KIND_CP2) return false;
+    return s->precond == CPS_PC_JACOBI || s->ncolours == 2;
 }
 
 static int solve_mixed(cps_sys s, const double* b, double* x, double rtol, int64_t max_iter,
@@ -1450,11 +1438,7 @@ static int solve_mixed(cps_sys s, const double* b, double* x, double rtol, int64
         int rc = autotune<float>(s, CPS_MIXED, v, stream);
         if (rc) return rc;
     }
-    {
-        bool done = false;
-        int rc = mixed_two_cyclic(s, b, x, rtol, max_iter, stats, stream, &done);
-        if (rc || done) return rc;
-    }
+    if (mixed_takes_fp64(s)) return solve_fp64(s, b, x, rtol, max_iter, stats, stream);
     const double* A64 = ic0 ? s->pa : s->a;
     const double* S64 = ic0 ? s->ps : s->s;
     const double* bb = b;
@@ -1587,7 +1571,11 @@ int solve_impl(cps_sys s, const double* b, double* x, double rtol, int64_t max_i
         l2_set_aside(s, 0, stream);   // error paths: give back a set-aside still held
         return rc;
     }
-    if (precision == CPS_MIXED) return solve_mixed(s, b, x, rtol, max_iter, stats, stream);
+    if (precision == CPS_MIXED) {
+        const int rc = solve_mixed(s, b, x, rtol, max_iter, stats, stream);
+        l2_set_aside(s, 0, stream);   // error paths: give back a set-aside still held
+        return rc;
+    }
     cps::set_error(s->ctx, "solve: bad precision");
     return CPS_ERR_ARG;
 }
