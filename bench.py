@@ -1336,9 +1336,6 @@ def main():
     jf = variants["jacobi_fp64"]
     roof = roofline(tuning["fp64"], nt, jf["iters"], jf["time_to_rtol_s"], peak, peak_kind,
                     args.n)
-    jm = variants["jacobi_mixed"]
-    if not tuning["fp64"].get("two_cyclic"):       # else the FP64 loop ran
-        jm["inner_gbs"] = BYTES_PER_CELL_ITER_MIXED * nt * jm["iters"] / jm["time_to_rtol_s"] / 1e9
 
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
