@@ -53,8 +53,9 @@ struct __align__(16) SideSlot {
 // arrays of their own and a second walk that looked the neighbours up, and 2.07
 // with this.
 __global__ void k_pair_sides(const int32_t* __restrict__ tri, int64_t nt, int64_t nv,
-                             SideSlot* table, unsigned long long mask, int32_t* __restrict__ nbr,
+                             SideSlot* table, unsigned int lines, int32_t* __restrict__ nbr,
                              int* err) {
+    const unsigned long long cap = (unsigned long long)lines * kBucket;
     const int64_t n3 = 3 * nt;
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n3;
          t += (int64_t)gridDim.x * blockDim.x) {
@@ -70,11 +71,12 @@ __global__ void k_pair_sides(const int32_t* __restrict__ tri, int64_t nt, int64_
         const unsigned long long hi = (unsigned long long)(va < vb ? vb : va);
         const unsigned long long key = lo * (unsigned long long)nv + hi;
         const unsigned long long hash = mix64(key);
-        const unsigned long long line = (lo * kBucket) & mask, first = hash >> 61;
-        for (unsigned long long probe = 0; probe <= mask + kBucket; ++probe) {
-            const unsigned long long h = probe < kBucket
-                                             ? (line + ((first + probe) & (kBucket - 1))) & mask
-                                             : (hash + (probe - kBucket)) & mask;
+        const unsigned long long line = (unsigned long long)((unsigned int)lo % lines) * kBucket;
+        unsigned long long h = 0;
+        for (unsigned long long probe = 0; probe < cap + kBucket; ++probe) {
+            if (probe < kBucket) h = line + ((hash + probe) & (kBucket - 1));
+            else if (probe == kBucket) h = __umul64hi(hash, cap);
+            else h = h + 1 < cap ? h + 1 : 0;
             SideSlot* q = &table[h];
             // a plain look first: a taken slot stays taken, and atomics queue
             unsigned long long old = *(volatile unsigned long long*)&q->key;
@@ -429,6 +431,7 @@ int assemble_impl(cps_ctx ctx, const double* xy, int64_t nv, const int32_t* tri,
     s->dt = dt;
     const int64_t nf = field_loc == CPS_PER_VERTEX ? nv : nt;
     int rc = CPS_OK;
+    unsigned long long* counters = nullptr;  // interior slot count, dmin bits, error and iso flags
     {
         Slab slab;
         slab.add(&s->s, nt);
@@ -443,6 +446,7 @@ int assemble_impl(cps_ctx ctx, const double* xy, int64_t nv, const int32_t* tri,
         slab.add(&s->a32, 3 * nt);
         slab.add(&s->s32, nt);
         slab.add(&s->slot_kind, 3 * nt);
+        slab.add(&counters, 3);
         const int64_t vs = (nt + 31) / 32 * 32;     // 256-byte aligned vectors
         slab.add(&s->wvec, 9 * vs);
         slab.add(&s->partials, (kNumPartials + 16) * kMaxGrid);
@@ -478,39 +482,40 @@ int assemble_impl(cps_ctx ctx, const double* xy, int64_t nv, const int32_t* tri,
     }
     s->grid = grid_for(ctx, nt);
     {
-        // Scratch of the assembly, stream ordered and released before return.
-        // at most 3/4 of the table is taken (cells without a common side), about
-        // 3/8 on a mesh, with a line for each of its nt / 2 vertices
-        unsigned long long cap = kBucket;
-        while (cap < (unsigned long long)(4 * nt)) cap <<= 1;
-        SideSlot* table = nullptr;
-        int32_t* nbr = nullptr;
-        double *area = nullptr, *ccx = nullptr, *ccy = nullptr, *xi = nullptr;
-        int* err = nullptr;
-        unsigned long long* counters = nullptr;  // [0] interior slot count, [1] dmin bits
-        int* iso = nullptr;
+        // The assembly's scratch lies in slices that are written after it is read
+        // (in stream-ordered allocations of its own: 2.07 against 1.50 ms an assembly
+        // of 2.09M cells, 1.11 against 0.72 of 0.82M).  The side
+        // table: 4 slots a cell, of which at most 3/4 are taken (cells without a
+        // common side), 3/8 on a mesh, with a line for each of its nt / 2 vertices;
+        // 64 B a cell in the 76 of a, col, off, a32 and s32, which lie in a row.
+        // The rest: 7.5 of the solver's nine vectors.
+        const unsigned int lines = (unsigned int)((4 * nt + kBucket - 1) / kBucket);
+        SideSlot* table = reinterpret_cast<SideSlot*>(s->a);
+        const size_t table_bytes = sizeof(SideSlot) * kBucket * (size_t)lines;
+        int32_t* nbr = reinterpret_cast<int32_t*>(s->wvec);
+        double* area = s->wvec + 2 * s->vec_stride;
+        double* ccx = s->wvec + 3 * s->vec_stride;
+        double* ccy = s->wvec + 4 * s->vec_stride;
+        double* xi = s->wvec + 5 * s->vec_stride;
+        double* xi_own = nullptr;                // more nodes than cells
+        int* err = reinterpret_cast<int*>(counters + 2);
+        int* iso = err + 1;
         int h_err = 0;
         unsigned long long h_cnt[2] = {0, 0};
         int h_iso = 1;
-        auto A = [&](void** p, size_t bytes) { return cudaMallocAsync(p, bytes, stream); };
         cudaError_t ce = cudaSuccess;
-        ce = A((void**)&table, sizeof(SideSlot) * cap);
-        if (ce == cudaSuccess) ce = A((void**)&nbr, sizeof(int32_t) * 3 * nt);
-        if (ce == cudaSuccess) ce = A((void**)&area, sizeof(double) * nt);
-        if (ce == cudaSuccess) ce = A((void**)&ccx, sizeof(double) * nt);
-        if (ce == cudaSuccess) ce = A((void**)&ccy, sizeof(double) * nt);
-        if (ce == cudaSuccess) ce = A((void**)&xi, sizeof(double) * 3 * nf);
-        if (ce == cudaSuccess) ce = A((void**)&err, sizeof(int) * 2);
-        if (ce == cudaSuccess) ce = A((void**)&counters, sizeof(unsigned long long) * 2);
+        if (nf > nt) {
+            ce = cudaMallocAsync((void**)&xi_own, sizeof(double) * 3 * nf, stream);
+            xi = xi_own;
+        }
         if (ce == cudaSuccess) {
-            iso = err + 1;
             const int g3 = grid_for(ctx, 3 * nt);
             const int g1 = grid_for(ctx, nt);
             const int gf = grid_for(ctx, nf);
             // the arrival counters of the grid reductions start at zero (memory
             // a freed system gave back need not be)
             cudaMemsetAsync(s->st, 0, sizeof(CgState) * 2, stream);
-            cudaMemsetAsync(table, 0xFF, sizeof(SideSlot) * cap, stream);
+            cudaMemsetAsync(table, 0xFF, table_bytes, stream);
             cudaMemsetAsync(nbr, 0xFF, sizeof(int32_t) * 3 * nt, stream);
             cudaMemsetAsync(err, 0, sizeof(int), stream);
             cudaMemsetAsync(iso, 0x00, sizeof(int), stream);
@@ -519,7 +524,7 @@ int assemble_impl(cps_ctx ctx, const double* xy, int64_t nv, const int32_t* tri,
             cudaMemsetAsync(s->slot_kind, 0, sizeof(int32_t) * 3 * nt, stream);
             const int one = 1;
             cudaMemcpyAsync(iso, &one, sizeof(int), cudaMemcpyHostToDevice, stream);
-            k_pair_sides<<<g3, kBlock, 0, stream>>>(tri, nt, nv, table, cap - 1, nbr, err);
+            k_pair_sides<<<g3, kBlock, 0, stream>>>(tri, nt, nv, table, lines, nbr, err);
             k_cell_geometry<<<g1, kBlock, 0, stream>>>(xy, tri, nt, nv, area, ccx, ccy, err);
             k_xi<<<gf, kBlock, 0, stream>>>(eps, kinv, nf, nu, dt, logk, xi, err);
             if (nb > 0)
@@ -542,9 +547,7 @@ int assemble_impl(cps_ctx ctx, const double* xy, int64_t nv, const int32_t* tri,
             if (ce == cudaSuccess)
                 ce = cudaMemcpyAsync(h_cnt, counters, sizeof(h_cnt), cudaMemcpyDeviceToHost, stream);
         }
-        void* scratch[] = {table, nbr, area, ccx, ccy, xi, err, counters};
-        for (void* p : scratch)
-            if (p) cudaFreeAsync(p, stream);
+        if (xi_own) cudaFreeAsync(xi_own, stream);
         cudaError_t se = cudaStreamSynchronize(stream);
         if (ce == cudaSuccess) ce = se;
         if (ce != cudaSuccess) {
