@@ -184,6 +184,7 @@ struct TransArgs {
     double* gfac;          // may be null
     unsigned long long* n_interior;
     int64_t nt;
+    int64_t nv;
     int kind;
     int field_loc;     // CPS_PER_VERTEX or CPS_PER_CELL (log-permeability maps to cells)
     bool logk;
@@ -200,6 +201,15 @@ __global__ void k_transmissibility(TransArgs A) {
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nt;
          e += (int64_t)gridDim.x * blockDim.x) {
         const int32_t v[3] = {A.tri[3 * e], A.tri[3 * e + 1], A.tri[3 * e + 2]};
+        if (v[0] < 0 || v[0] >= A.nv || v[1] < 0 || v[1] >= A.nv || v[2] < 0 || v[2] >= A.nv) {
+            // refused by k_cell_geometry: nothing is read through these ids
+            A.diag[e] = 1.0;
+            for (int j = 0; j < 3; ++j) {
+                A.off[(int64_t)j * nt + e] = 0.0;
+                A.col[(int64_t)j * nt + e] = (int32_t)e;
+            }
+            continue;
+        }
         const double cex = A.ccx[e], cey = A.ccy[e];
         double diag = 0.0;
         if (A.kind != CPS_KIND_CP2) {
@@ -534,7 +544,7 @@ int assemble_impl(cps_ctx ctx, const double* xy, int64_t nv, const int32_t* tri,
             ta.xy = xy; ta.tri = tri; ta.nbr = nbr; ta.ccx = ccx; ta.ccy = ccy; ta.area = area;
             ta.xi = xi; ta.eps = eps; ta.kinv = kinv; ta.slot_kind = s->slot_kind;
             ta.diag = s->diag; ta.off = s->off; ta.col = s->col; ta.gfac = s->gfac;
-            ta.n_interior = counters; ta.nt = nt; ta.kind = kind; ta.field_loc = field_loc;
+            ta.n_interior = counters; ta.nt = nt; ta.nv = nv; ta.kind = kind; ta.field_loc = field_loc;
             ta.nu = nu; ta.dt = dt; ta.err = err; ta.logk = logk;
             k_transmissibility<<<g1, kBlock, 0, stream>>>(ta);
             k_sqrt_diag<<<g1, kBlock, 0, stream>>>(s->diag, nt, s->s, s->s32, counters + 1, err);

@@ -93,3 +93,17 @@ def test_a_side_of_more_than_two_cells_is_refused(ctx, k):
         ctx.assemble(xy, tri, np.array([0], np.int32), eps, synth.iso_kinv(eps), cps.PER_VERTEX,
                      cps.KIND_CP2, 1.5e-5, 0.225)
     assert err.value.code == cps._cps.ERR_NONMANIFOLD
+
+
+@pytest.mark.parametrize("kind", [cps.KIND_CP2, cps.KIND_CP1_X])
+@pytest.mark.parametrize("where", [(0, 0), (50, 1), (97, 2)])
+def test_vertex_ids_out_of_range_are_refused(ctx, kind, where):
+    m = synth.lattice(8, seed=0)
+    eps = np.ones(m.nv)
+    for bad in (m.nv, 2**31 - 1, -1, -2**31):
+        tri = m.tri.copy()
+        tri[where] = bad
+        with pytest.raises(cps.CpsError) as err:
+            ctx.assemble(m.xy, tri, m.dirichlet, eps, synth.iso_kinv(eps), cps.PER_VERTEX, kind,
+                         1.5e-5, 0.225)
+        assert err.value.code == cps._cps.ERR_ARG
