@@ -43,7 +43,8 @@ struct __align__(16) SideSlot {
     int32_t id0, id1;
 };
 
-// Pairs the two cells of every side and writes the neighbour of each: the
+// Pairs the two cells of every side and writes the side of the neighbour (3 cell
+// + local side) into each one's slot of nbr [3][nt], boundary sides -1: the
 // second cell to arrive at a slot knows both.  A side is looked for in the
 // line of its lower vertex first, so that a numbering with locality walks the
 // table in lines instead of at random, and then from a hashed slot on: a
@@ -88,8 +89,8 @@ __global__ void k_pair_sides(const int32_t* __restrict__ tri, int64_t nt, int64_
                     set_error(err, CPS_ERR_NONMANIFOLD);
                 } else {
                     const int32_t eo = other / 3;
-                    nbr[(int64_t)j * nt + e] = eo;
-                    nbr[(int64_t)(other - 3 * eo) * nt + eo] = (int32_t)e;
+                    nbr[(int64_t)j * nt + e] = other;
+                    nbr[(int64_t)(other - 3 * eo) * nt + eo] = (int32_t)t;
                 }
             }
             break;
@@ -170,7 +171,7 @@ __global__ void k_mark_dirichlet(const int32_t* __restrict__ dirichlet, int64_t 
 struct TransArgs {
     const double* xy;
     const int32_t* tri;
-    const int32_t* nbr;
+    const int32_t* nbr;    // [3][nt] side across, 3 cell + local side, or -1
     const double* ccx;
     const double* ccy;
     const double* area;
@@ -192,116 +193,142 @@ struct TransArgs {
     int* err;
 };
 
-// Side coefficients and the matrix of a cell: bound by FP64 issue (a root and
-// four divisions a side, some 250 operations a cell).  The interior sides are
-// counted per warp: an atomic per cell on one word held the kernel up.
-__global__ void k_transmissibility(TransArgs A) {
+// Side coefficients.  Bound by FP64 issue: a root and four divisions a side. So an
+// interior side is computed once, by the lower of its two cells, and written to both
+// rows (seen from the other cell the same operations run on negated inputs, to the
+// same bits).  A warp takes its turns on the FP64 pipe for one active lane as for
+// 32, so a block first lists the sides its 256 cells have to compute, and then takes
+// them one a thread: 365 us at 2.09M cells, 710 with both cells computing their
+// sides.  A Dirichlet side's coefficient waits in off for k_diagonal.
+__global__ void __launch_bounds__(kBlock) k_transmissibility(TransArgs A) {
+    __shared__ unsigned short s_list[3 * kBlock];     // 3 (cell of the block) + local side
+    __shared__ int s_count;
     const int64_t nt = A.nt;
+    const int tid = (int)threadIdx.x, lane = tid & 31;
     unsigned int count = 0;
+    for (int64_t base = blockIdx.x * (int64_t)kBlock; base < nt;
+         base += (int64_t)gridDim.x * kBlock) {
+        if (tid == 0) s_count = 0;
+        __syncthreads();
+        const int64_t own = base + tid;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            bool mine = false;
+            if (own < nt) {
+                const int64_t slot = (int64_t)j * nt + own;
+                const int32_t sp = A.nbr[slot];
+                const bool dir = A.slot_kind[slot] == 2;
+                const int64_t ia = A.tri[3 * own + (j + 1) % 3], ib = A.tri[3 * own + (j + 2) % 3];
+                // a cell with a vertex out of range is refused elsewhere; its paired sides have
+                // both vertices in range
+                const bool in = ia >= 0 && ia < A.nv && ib >= 0 && ib < A.nv;
+                mine = sp >= 0 ? own <= sp / 3 : dir && in;
+                if (sp < 0 && !mine) {
+                    A.off[slot] = 0.0;
+                    A.col[slot] = (int32_t)own;
+                    A.slot_kind[slot] = 0;
+                    if (A.gfac) A.gfac[slot] = 0.0;
+                }
+            }
+            const unsigned int m = __ballot_sync(0xffffffffu, mine);
+            int at = 0;
+            if (lane == 0 && m) at = atomicAdd(&s_count, __popc(m));
+            at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << lane) - 1));
+            if (mine) s_list[at] = (unsigned short)(3 * tid + j);
+        }
+        __syncthreads();
+        const int n = s_count;
+        for (int i = tid; i < n; i += kBlock) {
+            const int code = s_list[i];
+            const int64_t e = base + code / 3;
+            const int j = code % 3;
+            const int64_t slot = (int64_t)j * nt + e;
+            const int64_t ia = A.tri[3 * e + (j + 1) % 3], ib = A.tri[3 * e + (j + 2) % 3];
+            const double px = A.xy[2 * ia], py = A.xy[2 * ia + 1];
+            const double qx = A.xy[2 * ib], qy = A.xy[2 * ib + 1];
+            const double tx = qx - px, ty = qy - py;
+            const double l = sqrt(tx * tx + ty * ty);
+            const double nx = ty / l, ny = -tx / l;
+            const double cex = A.ccx[e], cey = A.ccy[e];
+            const int32_t sp = A.nbr[slot];
+            const int32_t ep = sp >= 0 ? sp / 3 : -1;
+            const double d = ep >= 0 ? (A.ccx[ep] - cex) * nx + (A.ccy[ep] - cey) * ny
+                                     : (0.5 * (px + qx) - cex) * nx + (0.5 * (py + qy) - cey) * ny;
+            if (!(d > 1e-12 * l)) set_error(A.err, CPS_ERR_NONDELAUNAY);
+            double coef = A.nu;
+            if (A.kind == CPS_KIND_CP2) {
+                double x0, x1, x2;
+                if (A.field_loc == CPS_PER_VERTEX) {
+                    x0 = 0.5 * (A.xi[3 * ia] + A.xi[3 * ib]);
+                    x1 = 0.5 * (A.xi[3 * ia + 1] + A.xi[3 * ib + 1]);
+                    x2 = 0.5 * (A.xi[3 * ia + 2] + A.xi[3 * ib + 2]);
+                } else if (ep >= 0) {
+                    x0 = 0.5 * (A.xi[3 * e] + A.xi[3 * (int64_t)ep]);
+                    x1 = 0.5 * (A.xi[3 * e + 1] + A.xi[3 * (int64_t)ep + 1]);
+                    x2 = 0.5 * (A.xi[3 * e + 2] + A.xi[3 * (int64_t)ep + 2]);
+                } else {
+                    x0 = A.xi[3 * e];
+                    x1 = A.xi[3 * e + 1];
+                    x2 = A.xi[3 * e + 2];
+                }
+                coef = x0 * (nx * nx) + 2.0 * x1 * (nx * ny) + x2 * (ny * ny);
+            }
+            const double T = l * coef / d;
+            const double g = !A.gfac ? 0.0 : (ep >= 0 ? l / (2.0 * d) : l / d);
+            A.off[slot] = -T;
+            A.col[slot] = ep >= 0 ? ep : (int32_t)e;
+            A.slot_kind[slot] = ep >= 0 ? 1 : 2;
+            if (A.gfac) A.gfac[slot] = g;
+            if (ep >= 0) {
+                const int64_t far = (int64_t)(sp - 3 * ep) * nt + ep;
+                A.off[far] = -T;
+                A.col[far] = (int32_t)e;
+                A.slot_kind[far] = 1;
+                if (A.gfac) A.gfac[far] = g;
+                count += 2;
+            }
+        }
+        __syncthreads();
+    }
+    count = __reduce_add_sync(0xffffffffu, count);
+    if (lane == 0 && count) atomicAdd(A.n_interior, (unsigned long long)count);
+}
+
+// Diagonal (mass term and side coefficients) and s = sqrt(diag); also the smallest
+// diagonal (as an ordered 64-bit pattern).
+__global__ void k_diagonal(TransArgs A, double* __restrict__ s, float* __restrict__ s32,
+                           unsigned long long* dmin) {
+    const int64_t nt = A.nt;
+    unsigned long long local = ~0ULL;       // combined per warp: one atomic each
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nt;
          e += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t v[3] = {A.tri[3 * e], A.tri[3 * e + 1], A.tri[3 * e + 2]};
-        if (v[0] < 0 || v[0] >= A.nv || v[1] < 0 || v[1] >= A.nv || v[2] < 0 || v[2] >= A.nv) {
-            // refused by k_cell_geometry: nothing is read through these ids
-            A.diag[e] = 1.0;
-            for (int j = 0; j < 3; ++j) {
-                A.off[(int64_t)j * nt + e] = 0.0;
-                A.col[(int64_t)j * nt + e] = (int32_t)e;
-            }
-            continue;
-        }
-        const double cex = A.ccx[e], cey = A.ccy[e];
-        double diag = 0.0;
+        double d = 0.0;
         if (A.kind != CPS_KIND_CP2) {
             // Mbar_kk A_e, Mbar the mean over the cell's nodes of (I + nu eps Kinv dt)/dt
             const int comp = A.kind == CPS_KIND_CP1_X ? 0 : 2;
             double mkk;
             if (A.field_loc == CPS_PER_VERTEX) {
                 mkk = 0.0;
-                for (int k = 0; k < 3; ++k)
-                    mkk += (1.0 + A.nu * A.eps[v[k]] * A.kinv[3 * (int64_t)v[k] + comp] * A.dt) / A.dt;
+                for (int k = 0; k < 3; ++k) {
+                    const int64_t v = A.tri[3 * e + k];
+                    if (v < 0 || v >= A.nv) continue;         // refused elsewhere
+                    mkk += (1.0 + A.nu * A.eps[v] * A.kinv[3 * v + comp] * A.dt) / A.dt;
+                }
                 mkk /= 3.0;
             } else {
                 mkk = (1.0 + A.nu * A.eps[e] * kinv_at(A.kinv, e, comp, A.logk) * A.dt) / A.dt;
             }
-            diag = mkk * A.area[e];
+            d = __dmul_rn(mkk, A.area[e]);   // rounded before the sides are added
         }
-        unsigned int interior = 0;
+#pragma unroll
         for (int j = 0; j < 3; ++j) {
             const int64_t slot = (int64_t)j * nt + e;
-            const int64_t ia = v[(j + 1) % 3], ib = v[(j + 2) % 3];
-            const double px = A.xy[2 * ia], py = A.xy[2 * ia + 1];
-            const double qx = A.xy[2 * ib], qy = A.xy[2 * ib + 1];
-            const double tx = qx - px, ty = qy - py;
-            const double l = sqrt(tx * tx + ty * ty);
-            const double nx = ty / l, ny = -tx / l;
-            const int32_t ep = A.nbr[slot];
-            const bool dir = A.slot_kind[slot] == 2;
-            double T = 0.0, g = 0.0;
-            int32_t c = (int32_t)e;
-            int sk = 0;
-            if (ep >= 0 || dir) {
-                double d;
-                if (ep >= 0) {
-                    d = (A.ccx[ep] - cex) * nx + (A.ccy[ep] - cey) * ny;
-                } else {
-                    d = (0.5 * (px + qx) - cex) * nx + (0.5 * (py + qy) - cey) * ny;
-                }
-                if (!(d > 1e-12 * l)) set_error(A.err, CPS_ERR_NONDELAUNAY);
-                double coef;
-                if (A.kind == CPS_KIND_CP2) {
-                    double x0, x1, x2;
-                    if (A.field_loc == CPS_PER_VERTEX) {
-                        x0 = 0.5 * (A.xi[3 * ia] + A.xi[3 * ib]);
-                        x1 = 0.5 * (A.xi[3 * ia + 1] + A.xi[3 * ib + 1]);
-                        x2 = 0.5 * (A.xi[3 * ia + 2] + A.xi[3 * ib + 2]);
-                    } else if (ep >= 0) {
-                        x0 = 0.5 * (A.xi[3 * e] + A.xi[3 * (int64_t)ep]);
-                        x1 = 0.5 * (A.xi[3 * e + 1] + A.xi[3 * (int64_t)ep + 1]);
-                        x2 = 0.5 * (A.xi[3 * e + 2] + A.xi[3 * (int64_t)ep + 2]);
-                    } else {
-                        x0 = A.xi[3 * e];
-                        x1 = A.xi[3 * e + 1];
-                        x2 = A.xi[3 * e + 2];
-                    }
-                    const double dn = x0 * (nx * nx) + 2.0 * x1 * (nx * ny) + x2 * (ny * ny);
-                    coef = dn;
-                } else {
-                    coef = A.nu;
-                }
-                T = l * coef / d;
-                if (A.gfac) g = ep >= 0 ? l / (2.0 * d) : l / d;
-                if (ep >= 0) {
-                    c = ep;
-                    sk = 1;
-                    ++interior;
-                } else {
-                    sk = 2;
-                }
-            }
-            diag += T;
-            A.off[slot] = (sk == 1) ? -T : 0.0;
-            A.col[slot] = c;
-            A.slot_kind[slot] = sk;
-            if (A.gfac) A.gfac[slot] = g;
+            d += -A.off[slot];
+            if (A.slot_kind[slot] == 2) A.off[slot] = 0.0;
         }
-        A.diag[e] = diag;
-        count += interior;
-    }
-    count = __reduce_add_sync(0xffffffffu, count);
-    if ((threadIdx.x & 31) == 0 && count)
-        atomicAdd(A.n_interior, (unsigned long long)count);
-}
-
-// s = sqrt(diag); also the smallest diagonal (as an ordered 64-bit pattern).
-__global__ void k_sqrt_diag(const double* __restrict__ diag, int64_t nt, double* __restrict__ s,
-                            float* __restrict__ s32, unsigned long long* dmin, int* err) {
-    unsigned long long local = ~0ULL;       // combined per warp: one atomic each
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nt;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        const double d = diag[e];
+        A.diag[e] = d;
         if (!(d > 0.0) || !isfinite(d)) {
-            set_error(err, CPS_ERR_SINGULAR);
+            set_error(A.err, CPS_ERR_SINGULAR);
             s[e] = 1.0;
             s32[e] = 1.0f;
             local = 0ULL;
@@ -323,14 +350,16 @@ __global__ void k_sqrt_diag(const double* __restrict__ diag, int64_t nt, double*
 __global__ void k_scale_offdiag(const double* __restrict__ off, const int32_t* __restrict__ col,
                                 const double* __restrict__ s, int64_t nt, double* __restrict__ a,
                                 float* __restrict__ a32) {
-    const int64_t n3 = 3 * nt;
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n3;
-         k += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t e = k % nt;
-        const int32_t c = col[k];
-        const double v = off[k] / (s[e] * s[c]);
-        a[k] = v;
-        a32[k] = (float)v;
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nt;
+         e += (int64_t)gridDim.x * blockDim.x) {
+        const double se = s[e];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const int64_t k = (int64_t)j * nt + e;
+            const double v = off[k] / (se * s[col[k]]);
+            a[k] = v;
+            a32[k] = (float)v;
+        }
     }
 }
 
@@ -547,10 +576,10 @@ int assemble_impl(cps_ctx ctx, const double* xy, int64_t nv, const int32_t* tri,
             ta.n_interior = counters; ta.nt = nt; ta.nv = nv; ta.kind = kind; ta.field_loc = field_loc;
             ta.nu = nu; ta.dt = dt; ta.err = err; ta.logk = logk;
             k_transmissibility<<<g1, kBlock, 0, stream>>>(ta);
-            k_sqrt_diag<<<g1, kBlock, 0, stream>>>(s->diag, nt, s->s, s->s32, counters + 1, err);
-            k_scale_offdiag<<<g3, kBlock, 0, stream>>>(s->off, s->col, s->s, nt, s->a, s->a32);
+            k_diagonal<<<g1, kBlock, 0, stream>>>(ta, s->s, s->s32, counters + 1);
+            k_scale_offdiag<<<g1, kBlock, 0, stream>>>(s->off, s->col, s->s, nt, s->a, s->a32);
             if (s->dxi) k_dxi_dtheta<<<g1, kBlock, 0, stream>>>(eps, kinv, nt, nu, dt, logk, s->dxi, iso);
-            s->assembly_launches = 7 + (nb > 0 ? 1 : 0) + (s->dxi ? 1 : 0);
+            s->assembly_launches = 6 + (nb > 0 ? 1 : 0) + (s->dxi ? 1 : 0);
             ce = cudaGetLastError();
             if (ce == cudaSuccess) ce = cudaMemcpyAsync(&h_err, err, sizeof(int), cudaMemcpyDeviceToHost, stream);
             if (ce == cudaSuccess) ce = cudaMemcpyAsync(&h_iso, iso, sizeof(int), cudaMemcpyDeviceToHost, stream);
