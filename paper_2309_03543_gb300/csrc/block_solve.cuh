@@ -539,6 +539,7 @@ __device__ __forceinline__ bool kbp_solve_tc(const BatchDesc& d, int rank, int k
             for (int i = rlo + (int)threadIdx.x; i < rhi; i += kBB) d.x[perm[i]] = 0.0;
             for (int i = lo + (int)threadIdx.x; i < hi; i += kBB) d.x[perm[nR + i]] = 0.0;
             if (threadIdx.x == 0) sc.rnorm2 = 0.0;
+            barrier();            // these cells lie anywhere: no member reads x before all are 0
             break;
         }
         while (sc.flag == 0) {
