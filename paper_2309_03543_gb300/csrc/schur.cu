@@ -219,10 +219,10 @@ __global__ void __launch_bounds__(kBlock) k_tc_back(const double* __restrict__ b
 
 // ------------------------------------------------------ the persistent loop
 
-constexpr int kGridMax = 160;        // blocks (one per SM): a lane polls at most five slots
+constexpr int kGridMax = 160;        // blocks (one per SM): five warps poll their totals
 constexpr int kPollPer = kGridMax / 32;
 constexpr int kQuant = 2;             // quantities of one reduction at most
-constexpr int kSlotStride = 16;       // words of a slot: a 128-byte line per block
+constexpr int kSlotStride = 16;       // words of a slot: a 128-byte line per block, 16 bytes a quantity
 constexpr size_t kSlotWords = 4 * (size_t)kGridMax * kSlotStride;   // [quantities][buffer][block]
 
 struct SchurArgs {
@@ -237,47 +237,62 @@ struct SchurArgs {
     double* y;
     int n;
     int64_t ld;
-    unsigned long long* pb;     // kSlotWords tagged block totals, zero at launch
+    unsigned long long* pb;     // kSlotWords words of block totals, zero at launch
     GridSync* gs;
     CgState* st;
     int stall;                  // test hook: every reduction waits for a value that never comes
     double dmin;                // smallest diagonal of A (stop-test gate), 0 for none
 };
 
-__device__ __forceinline__ unsigned long long ld_relaxed(const unsigned long long* p) {
-    unsigned long long v;
-    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
+// A block's total and the number of its use, one 16-byte access (single-copy
+// atomic: 128-bit scoped loads and stores).
+__device__ __forceinline__ void ld_total(const unsigned long long* p, double& v,
+                                         unsigned long long& use) {
+    unsigned long long bits;
+    asm volatile(
+        "{\n\t.reg .b128 t;\n\tld.relaxed.gpu.global.b128 t, [%2];\n\tmov.b128 {%0, %1}, t;\n\t}"
+        : "=l"(bits), "=l"(use)
+        : "l"(p)
+        : "memory");
+    v = __longlong_as_double((long long)bits);
 }
 
-__device__ __forceinline__ void st_relaxed(unsigned long long* p, unsigned long long v) {
-    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+__device__ __forceinline__ void st_total(unsigned long long* p, double v, unsigned long long use) {
+    asm volatile(
+        "{\n\t.reg .b128 t;\n\tmov.b128 t, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], t;\n\t}"
+        ::"l"(p), "l"((unsigned long long)__double_as_longlong(v)), "l"(use)
+        : "memory");
 }
 
-// T 2^(E - 1075 + h) as a double, |T| < 2^61, rounded half up, in integer
+// T 2^(E - 1075 + h) as a double, |T| <= 2^62, rounded half up, in integer
 // arithmetic (NaN if the set held an infinity or NaN, infinity on overflow,
-// zero below the normal range): every warp converts its sum, and the FP64 pipe
-// takes one warp instruction in 17 cycles.
+// a subnormal below the normal range): the FP64 pipe takes one warp instruction
+// in 17 cycles.
 __device__ __forceinline__ double fixed_bits(long long T, int E, int h) {
     unsigned long long m = T < 0 ? 0ull - (unsigned long long)T : (unsigned long long)T;
-    int e = E + h;                                  // exponent of a 53-bit m
-    const int sh = 11 - __clzll((long long)m);      // m to 53 bits: right by sh (left if < 0)
-    e += sh;
-    if (sh > 0) {
-        m = (m + (1ull << (sh - 1))) >> sh;
-        if (m >> 53) {
-            m >>= 1;
-            ++e;
-        }
-    } else {
-        m <<= -sh & 63;
-    }
-    unsigned long long bits = ((unsigned long long)e << 52) | (m & 0xFFFFFFFFFFFFFull);
-    if (e >= 2047) bits = 0x7FF0000000000000ull;
-    if (T == 0 || e <= 0) bits = 0;
+    const int e = E + h;                            // exponent field of a 53-bit m
+    // m to 53 bits (right by sh, left if < 0), to fewer below the normal range
+    const int sh = max(11 - __clzll((long long)m), 1 - e);
+    m = sh > 0 ? (m + (1ull << (sh - 1))) >> sh : m << (-sh & 63);
+    // bit 52 of m, and a carry into bit 53, count up the field
+    unsigned long long bits = ((unsigned long long)(e + sh - 1) << 52) + m;
+    if (bits > 0x7FF0000000000000ull) bits = 0x7FF0000000000000ull;
+    if (T == 0) bits = 0;
     if (T < 0) bits |= 1ull << 63;
     if (E >= 2047) bits = 0x7FF8000000000000ull;
     return __longlong_as_double((long long)bits);
+}
+
+// v / 2^(E - 1075) for |v| < 2^(E - 1022), rounded half up: at most 2^53 in magnitude,
+// every bit of the values in the largest one's binade.
+__device__ __forceinline__ long long align_whole(double v, int E) {
+    const long long bits = __double_as_longlong(v);
+    const int e = (int)((bits >> 52) & 0x7FF);
+    long long m = bits & 0xFFFFFFFFFFFFFLL;
+    if (e) m |= 1LL << 52;
+    const int sh = E - (e > 0 ? e : 1);
+    if (sh > 0) m = sh > 62 ? 0 : (m + (1LL << (sh - 1))) >> sh;
+    return bits < 0 ? -m : m;
 }
 
 // v > 0 and finite, on the bits (a compare on the FP64 pipe takes its latency).
@@ -287,12 +302,12 @@ __device__ __forceinline__ bool positive_finite(double v) {
 }
 
 // Grid-wide sum of v[0..NV) over blocks of T threads: exact integer sums per
-// warp, per block and over the grid, each rounded to a double (trees of FP64
+// warp and per block, rounded to a double once, and over the grid (trees of FP64
 // adds, 116 cycles a step and one warp instruction in 17 cycles, measured 0.8
-// to 1.3 us slower an iteration).  Each block stores its NV totals into its slot of one of two buffers, the last
-// mantissa bit replaced by the buffer's use count modulo 2.  Warp k of every
-// block polls the G slots of quantity k until all of them carry this use's bit,
-// and adds them: a total and its arrival travel in one word, so the reduction
+// to 1.3 us slower an iteration).  Each block stores its NV totals into its slot of
+// one of two buffers, with the buffer's use count beside each.  A warp of every
+// block polls 32 of the G slots of a quantity until all of them carry this use,
+// and adds them; the first of a quantity's warps adds the warps' sums: a total and its arrival travel in one access, so the reduction
 // costs one store and one load across the chip instead of a store, a counter
 // and a load.  A slot is a 128-byte line of its own: with 152 blocks polling,
 // an all-to-all of dense words takes 10000 cycles, of 32-byte sectors 5000, of
@@ -308,78 +323,90 @@ template <int T, int NV, typename Post>
 __device__ __forceinline__ void tagged_allreduce(const double (&v)[NV], unsigned int& ep,
                                                  const SchurArgs& P, int& s_fail, Post post) {
     static_assert(NV >= 1 && NV <= kQuant, "quantities");
-    __shared__ double s_w[kQuant][32];
-    __shared__ double s_tot[kQuant];
+    __shared__ long long s_w[NV][32];          // sums of the warps, each in units of its own
+    __shared__ int s_e[NV][32];
+    __shared__ long long s_g[NV][kPollPer];    // sums of 32 blocks' totals, likewise
+    __shared__ int s_ge[NV][kPollPer];
+    __shared__ double s_tot[NV];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int G = (int)gridDim.x;
+    const int nq = (G + 31) >> 5;              // warps that poll for a quantity
 #pragma unroll
     for (int k = 0; k < NV; ++k) {
         const int E = __reduce_max_sync(0xffffffffu, align_exp(v[k]));
         const long long t = warp_sum_fixed<52>(align_fixed(v[k], E, 1));
-        if (lane == 0) s_w[k][warp] = fixed_bits(t, E, 1);
+        if (lane == 0) {
+            s_w[k][warp] = t;
+            s_e[k][warp] = E;
+        }
     }
     __syncthreads();
-    if (warp < NV) {
-        const unsigned long long tag = 1ull ^ ((ep >> 1) & 1ull);
+    if (warp < NV * nq) {
+        const int k = NV > 1 && warp >= nq ? 1 : 0;
+        const int q = warp - k * nq;
+        const unsigned long long use = (unsigned long long)(ep >> 1) + 1;
         unsigned long long* slots =
-            P.pb + ((NV - 1) * 2 + (size_t)(ep & 1u)) * kGridMax * kSlotStride + warp;
-        const double x = lane < T / 32 ? s_w[warp][lane] : 0.0;
-        const int E = __reduce_max_sync(0xffffffffu, align_exp(x));
-        const long long t = warp_sum_fixed<52>(align_fixed(x, E, 1));
-        if (lane == 0) {
-            const unsigned long long bits =
-                (unsigned long long)__double_as_longlong(fixed_bits(t, E, 1));
-            st_relaxed(slots + blockIdx.x * kSlotStride, (bits & ~1ull) | tag);
+            P.pb + ((NV - 1) * 2 + (size_t)(ep & 1u)) * kGridMax * kSlotStride + 2 * k;
+        if (q == 0) {
+            const int Ew = lane < T / 32 ? s_e[k][lane] : 1;
+            const int E = __reduce_max_sync(0xffffffffu, Ew);
+            // at most 2^57 a warp, in the largest unit
+            const int sh = E - Ew;
+            long long x = lane < T / 32 ? s_w[k][lane] : 0;
+            if (sh > 0) x = sh > 60 ? 0 : (x + (1LL << (sh - 1))) >> sh;
+            const long long t = warp_sum_fixed<57>(x);
+            if (lane == 0) st_total(slots + blockIdx.x * kSlotStride, fixed_bits(t, E, 1), use);
         }
-        unsigned long long got[kPollPer];
-        unsigned int miss = 0;
-#pragma unroll
-        for (int q = 0; q < kPollPer; ++q) {
-            got[q] = 0;
-            if (lane + 32 * q < G) miss |= 1u << q;
-        }
+        slots += (lane + 32 * q) * kSlotStride;
+        double got = 0.0;
+        bool miss = lane + 32 * q < G;
         const bool never = P.stall != 0 && lane == 0;
         unsigned long long t0 = 0;
-        bool ok = true;
         for (long long spins = 0;; ++spins) {
-#pragma unroll
-            for (int q = 0; q < kPollPer; ++q)
-                if (miss & (1u << q)) got[q] = ld_relaxed(slots + (lane + 32 * q) * kSlotStride);
-#pragma unroll
-            for (int q = 0; q < kPollPer; ++q)
-                if ((miss & (1u << q)) && (got[q] & 1ull) == tag && !never) miss &= ~(1u << q);
-            if (__all_sync(0xffffffffu, miss == 0)) break;
+            if (miss) {
+                unsigned long long seen;
+                ld_total(slots, got, seen);
+                miss = seen != use || never;
+            }
+            if (__all_sync(0xffffffffu, !miss)) break;
             if ((spins & 255) == 255) {
                 const unsigned long long now = global_ns();
                 if (t0 == 0) t0 = now;
                 const bool out = now - t0 > kWaitNs || spins > kSpinCap ||
                                  *(volatile int*)&P.gs->timeout != 0;
                 if (__any_sync(0xffffffffu, out)) {
-                    ok = false;
+                    if (lane == 0) {
+                        atomicExch(&P.gs->timeout, 1);
+                        s_fail = 1;
+                    }
                     break;
                 }
             }
         }
-        if (!ok) {
+        int E = __reduce_max_sync(0xffffffffu, align_exp(got));
+        long long t = warp_sum_fixed<53>(align_whole(got, E));     // at most 2^58
+        if (nq > 1) {
             if (lane == 0) {
-                atomicExch(&P.gs->timeout, 1);
-                s_fail = 1;
+                s_g[k][q] = t;
+                s_ge[k][q] = E;
             }
-        } else {
-            int em = 1;
+            asm volatile("bar.sync 1, %0;" ::"r"(NV * nq * 32) : "memory");
+            if (q == 0) {
+                const int Eq = lane < nq ? s_ge[k][lane] : 1;
+                E = __reduce_max_sync(0xffffffffu, Eq);
+                const int sh = E - Eq;
+                t = lane < nq ? s_g[k][lane] : 0;
+                if (sh > 0) t = sh > 61 ? 0 : (t + (1LL << (sh - 1))) >> sh;
+                static_assert(kPollPer <= 8, "the lanes of the sum");
 #pragma unroll
-            for (int q = 0; q < kPollPer; ++q)
-                em = max(em, align_exp(__longlong_as_double((long long)got[q])));
-            const int Eg = __reduce_max_sync(0xffffffffu, em);
-            long long acc = 0;       // at most kPollPer values of 2^50 a lane
-#pragma unroll
-            for (int q = 0; q < kPollPer; ++q)
-                acc += align_fixed(__longlong_as_double((long long)got[q]), Eg, 3);
-            const long long tg = warp_sum_fixed<53>(acc);
-            if (lane == 0) s_tot[warp] = fixed_bits(tg, Eg, 3);
+                for (int d = 4; d > 0; d >>= 1) t += __shfl_down_sync(0xffffffffu, t, d);
+            }
         }
-        if (NV > 1) asm volatile("bar.sync 1, %0;" ::"n"(NV * 32) : "memory");
-        if (threadIdx.x == 0 && !s_fail) post(s_tot);
+        if (q == 0) {
+            if (lane == 0) s_tot[k] = fixed_bits(t, E, 0);
+            if (NV > 1) asm volatile("bar.sync 2, %0;" ::"n"(NV * 32) : "memory");
+            if (threadIdx.x == 0 && !s_fail) post(s_tot);
+        }
     }
     ++ep;
 }
