@@ -426,8 +426,9 @@ int cps_set_solver_path(cps_sys sys, int path);
  * block are host arrays of 3 entries (SpMV, residual update, direction
  * update; the third is ignored for CPS_MIXED): unroll 1, 2 or 4 rows per
  * thread per trip (also 8 for the two FP64 update kernels), grid 1..4096
- * blocks, block 256 (or, CPS_FP64 only, 1024) threads.  CPS_ERR_ARG for
- * anything else. */
+ * blocks, block 256 (or, CPS_FP64 only, 1024) threads.  Shapes pinned for
+ * CPS_MIXED also keep the system's CPS_MIXED solves in the binary32 iteration
+ * that they are for.  CPS_ERR_ARG for anything else. */
 int cps_set_kernel_shapes(cps_sys sys, int precision, const int32_t* unroll, const int32_t* grid,
                           const int32_t* block);
 

@@ -361,6 +361,7 @@ int cps_set_kernel_shapes(cps_sys sys, int precision, const int32_t* unroll, con
         t.k[k].block = block[k];
     }
     t.done = true;
+    if (precision == CPS_MIXED) t.pinned = true;     // they are binary32's: it runs
     t.kg_set = false;        // the single-reduction update follows the pinned residual update
     cps::drop_graphs(sys, precision);       // captured with the old shapes
     return CPS_OK;
@@ -372,9 +373,10 @@ int cps_get_tuning(cps_sys sys, int precision, int32_t* unroll, int32_t* grid, i
         return CPS_ERR_ARG;
     const cps::Tuning& t = sys->tune[precision];
     for (int k = 0; k < 3; ++k) {
-        unroll[k] = t.done ? t.k[k].unroll : 0;
-        grid[k] = t.done ? t.k[k].grid : 0;
-        if (block) block[k] = t.done ? t.k[k].block : 0;
+        const bool set = t.done || t.k[k].grid > 0;
+        unroll[k] = set ? t.k[k].unroll : 0;
+        grid[k] = set ? t.k[k].grid : 0;
+        if (block) block[k] = set ? t.k[k].block : 0;
     }
     if (flags) {
         flags[0] = (t.path_done && t.path == 1) ? 1 + t.cluster_variant : 0;

@@ -90,7 +90,9 @@ struct Tuning {
     int ic0_path = 0;
     int ic0_win = 0;         // persisting L2 window of the persistent IC(0) loop (0 or 3)
     bool ic0_done = false;
-    bool pinned = false;     // cps_set_solver_path chose the path (not CPS_PATH_AUTO)
+    // CPS_FP64: cps_set_solver_path chose the path (not CPS_PATH_AUTO); CPS_MIXED:
+    // cps_set_kernel_shapes chose the binary32 kernels' shapes
+    bool pinned = false;
     // FP64 Jacobi on a two-coloured graph, two-cyclic form (schur.cu): 0 not
     // timed, 1 taken by CPS_PATH_AUTO, 2 slower than the loop above
     int tc = 0;
