@@ -175,7 +175,8 @@ int cps_export_matrix(cps_sys sys, double* diag, int32_t* col, double* val, void
  *   stats       host pointer, may be NULL
  * b = 0 gives x = 0.  Errors: CPS_ERR_ARG, _NOT_SPD, _NOT_CONVERGED (x holds
  * the last iterate; CPS_MIXED: the iterate with the least true residual, with
- * that residual in stats -- where kappa(A) times the binary32 unit roundoff
+ * that residual in stats, where a FP64 loop ran too (of the start and the ends
+ * of its up to 8 runs) -- where kappa(A) times the binary32 unit roundoff
  * approaches 1 the binary32 corrections stop reducing the FP64 residual, and
  * the solve ends there instead of letting refinement drive it up), _CUDA. */
 int cps_solve(cps_sys sys, const double* b, double* x, double rtol, int64_t max_iter,
@@ -193,18 +194,19 @@ int cps_solve(cps_sys sys, const double* b, double* x, double rtol, int64_t max_
  * block takes whole systems from a device work queue (largest first) and
  * solves each with block-level reductions only; a team's blocks join the
  * queue when their system is done, and every system stops as soon as it
- * converges.  An ensemble of CP2 systems runs in FP64 in either precision, and
- * where all its cell graphs have two colours as CG on their Schur complements
- * (two Jacobi iterations a step, counted as two; see CPS_PATH_AUTO).  Else the
- * iteration
- * is the single-reduction (Chronopoulos-Gear) form
- * of Jacobi CG, restarted from the true residual up to 8 times.  A team
+ * converges.  An ensemble of CP2 systems runs in FP64 in either precision
+ * (CPS_MIXED then returns the iterate with the least true residual all the
+ * same), and where all its cell graphs have two colours as CG on their Schur
+ * complements (two Jacobi iterations a step, counted as two; see
+ * CPS_PATH_AUTO).  Else the iteration is the single-reduction
+ * (Chronopoulos-Gear) form of Jacobi CG, restarted from the true residual up to
+ * 8 times.  A team
  * wait that runs out (about one second) gives CPS_ERR_TIMEOUT.  With
  * cps_set_batch_path(ctx, CPS_BATCH_GRAPH) instead one launch per phase for
  * all systems, a per-system convergence mask, and iteration chunks replayed
  * from a CUDA graph (a system of more than 33,554,432 cells is rejected there
- * with CPS_ERR_ARG -- solve it alone).  CPS_MIXED: by default the same one
- * launch, each system (or team) running the single solve's refinement with
+ * with CPS_ERR_ARG -- solve it alone).  CPS_MIXED with other systems among
+ * them: by default the same one launch, each system (or team) running the single solve's refinement with
  * every decision on the device -- binary32 textbook CG inner iterations with
  * FP64 inner products, an FP64 true residual after each, the best FP64
  * iterate kept (stats.refinements = residual replacements); with

@@ -406,6 +406,16 @@ __global__ void __launch_bounds__(kBB, 2) kb_one_launch(const BatchDesc* __restr
     }
 }
 
+// The callers' starts, for ensembles that return the iterate with the least residual.
+__global__ void __launch_bounds__(kBB) kb_save_start(const BatchDesc* __restrict__ dd, int nsys) {
+    for (int i = 0; i < nsys; ++i) {
+        const BatchDesc& d = dd[i];
+        for (int64_t e = blockIdx.x * (int64_t)kBB + threadIdx.x; e < d.n;
+             e += (int64_t)gridDim.x * kBB)
+            d.start[e] = d.x[e];
+    }
+}
+
 // The systems' states into one array (one copy to the host).
 __global__ void kb_gather_states(const BatchDesc* __restrict__ dd, int nsys, CgState* out) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nsys; i += gridDim.x * blockDim.x)
@@ -570,7 +580,6 @@ static int solve_batch_one_launch(const cps_sys* systems, int nsys, const double
         d.t = s->wp1;
         d.a32 = s->a32;
         d.s32 = s->s32;
-        d.best = s->wbest;
         d.partials = s->partials;
         d.st = s->st;
         d.n = s->nt;
@@ -600,7 +609,13 @@ static int solve_batch_one_launch(const cps_sys* systems, int nsys, const double
     // 4.0 against 6.6 s): see mixed_takes_fp64
     bool cp2 = true;
     for (int i = 0; i < nsys; ++i) cp2 = cp2 && systems[i]->kind == CPS_KIND_CP2;
-    if (tc || cp2) mixed = false;
+    // CPS_MIXED promises the iterate with the least true residual on either route
+    const bool least = mixed && (tc || cp2);
+    for (int i = 0; i < nsys && mixed; ++i) {
+        hd[i].best = systems[i]->wbest;
+        if (least) hd[i].start = systems[i]->wx;
+    }
+    if (least) mixed = false;
     const void* kernel = tc      ? (const void*)kb_one_launch<2>
                          : mixed ? (const void*)kb_one_launch<1>
                                  : (const void*)kb_one_launch<0>;
@@ -661,6 +676,7 @@ static int solve_batch_one_launch(const cps_sys* systems, int nsys, const double
                             stream) != cudaSuccess)
             rc = CPS_ERR_CUDA;
     }
+    if (rc == CPS_OK && least) kb_save_start<<<grid, kBB, 0, stream>>>(dd, nsys);
     if (rc == CPS_OK) {
         // cooperative: every team's blocks are resident together
         int* dnext = dorder + nqueue;
@@ -683,9 +699,22 @@ static int solve_batch_one_launch(const cps_sys* systems, int nsys, const double
     if (rc == CPS_OK) {
         for (int i = 0; i < nsys; ++i) {
             const CgState& h = hst[i];
-            const double rel = h.bnorm2 > 0 ? std::sqrt(h.rnorm2 / h.bnorm2) : 0.0;
+            double rel = h.bnorm2 > 0 ? std::sqrt(h.rnorm2 / h.bnorm2) : 0.0;
             int st = h.status;
             if (st == CPS_OK && h.bnorm2 > 0 && !(rel <= rtol)) st = CPS_ERR_NOT_CONVERGED;
+            if (least && st == CPS_ERR_NOT_CONVERGED) {
+                // the caller's start, if no round ended below it
+                double r2 = INFINITY;
+                int rs = true_residual2(systems[i], b[i], systems[i]->wx, &r2, stream);
+                if (rs == CPS_OK && (r2 < h.rnorm2 || std::isnan(h.rnorm2))) {
+                    if (cudaMemcpyAsync(x[i], systems[i]->wx, sizeof(double) * systems[i]->nt,
+                                        cudaMemcpyDeviceToDevice, stream) != cudaSuccess)
+                        rs = CPS_ERR_CUDA;
+                    rel = std::sqrt(r2 / h.bnorm2);
+                    if (rel <= rtol) st = CPS_OK;
+                }
+                if (rs != CPS_OK) rc = rs;
+            }
             if (st != CPS_OK && first == CPS_OK) first = st;
             if (stats) {
                 stats[i].iters = h.iter;
@@ -710,9 +739,9 @@ static int solve_batch_one_launch(const cps_sys* systems, int nsys, const double
         return rc;
     }
     if (first == CPS_ERR_NOT_CONVERGED)
-        cps::set_error(ctx, mixed ? "solve_batch: a member did not reach rtol in mixed precision "
-                                    "(max_iter, or binary32 refinement stopped reducing its "
-                                    "residual: its x holds the iterate with the least residual)"
+        cps::set_error(ctx, mixed || least ? "solve_batch: a member did not reach rtol in mixed precision "
+                                    "(max_iter, or its residual stopped falling: its x holds the "
+                                    "iterate with the least residual)"
                                   : "solve_batch: max_iter reached");
     if (first == CPS_ERR_NOT_SPD) cps::set_error(ctx, "solve_batch: p.Ap <= 0");
     if (first == CPS_ERR_TIMEOUT)

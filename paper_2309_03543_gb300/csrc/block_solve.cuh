@@ -28,7 +28,8 @@ struct BatchDesc {
     double* t;                    // one-launch solve only: w = Ahat r
     const float* a32;             // one-launch mixed solve: binary32 matrix and S
     const float* s32;
-    double* best;                 // one-launch mixed solve: the best FP64 iterate
+    double* best;                 // the best FP64 iterate (FP64 loops: null unless CPS_MIXED)
+    double* start;                // the caller's x (FP64 loops under CPS_MIXED)
     double* partials;
     CgState* st;
     int64_t n;
@@ -204,9 +205,26 @@ struct SolveScalars {
     double ig;                    // 1 / gamma
     double c;                     // 1 / (gamma alpha)
     long long total, it, budget;
+    double best;                  // least ||b - A x||^2 at the end of a round (d.best)
     int flag;                     // 0 run, 1 stop, 2 breakdown, 3 b = 0
     int status;
+    int keep;                     // this round's x is the least so far
 };
+
+// Thread 0, at a round's end (rnorm2 and flag set; keep: CPS_MIXED, which returns
+// the iterate with the least true residual where rtol is not reached): 1 x becomes
+// the best iterate, 2 the solve's last round ended above it (rnorm2 set to its
+// residual): x is replaced, 0 neither.
+__device__ __forceinline__ int round_ends(SolveScalars& sc, bool keep, bool last) {
+    if (!keep || sc.status != CPS_OK || sc.rnorm2 <= sc.thresh2) return 0;
+    if (sc.rnorm2 <= sc.best) {
+        sc.best = sc.rnorm2;
+        return 1;
+    }
+    if (!(sc.flag || last) || !(sc.best < INFINITY)) return 0;
+    sc.rnorm2 = sc.best;
+    return 2;
+}
 
 // w = Ahat r on rows [lo, hi) with gamma = r.r, delta = w.r and, if check,
 // ||S r||^2 into v[0..3).
@@ -283,6 +301,7 @@ __device__ __forceinline__ bool kbp_solve(const BatchDesc& d, int64_t lo, int64_
         sc.it = 0;
         sc.status = CPS_OK;
         sc.bnorm2 = sc.rnorm2 = sc.thresh2 = 0.0;
+        sc.best = INFINITY;
     }
     for (int round = 0; round < 8; ++round) {
         // y = S x, r = S^-1 b - Ahat y, p = s = 0
@@ -419,8 +438,13 @@ __device__ __forceinline__ bool kbp_solve(const BatchDesc& d, int64_t lo, int64_
             sc.it = 0;
             sc.rnorm2 = nn[0];
             sc.flag = (sc.status != CPS_OK || nn[0] <= sc.thresh2 || sc.total >= max_iter) ? 1 : 0;
+            sc.keep = round_ends(sc, d.best != nullptr, round == 7);
         }
         __syncthreads();
+        if (sc.keep == 1)
+            for (int64_t e = lo + threadIdx.x; e < hi; e += kBB) d.best[e] = d.x[e];
+        if (sc.keep == 2)
+            for (int64_t e = lo + threadIdx.x; e < hi; e += kBB) d.x[e] = d.best[e];
         if (sc.flag) break;
     }
     __syncthreads();
@@ -483,6 +507,7 @@ __device__ __forceinline__ bool kbp_solve_tc(const BatchDesc& d, int rank, int k
         sc.it = 0;
         sc.status = CPS_OK;
         sc.bnorm2 = sc.rnorm2 = sc.thresh2 = 0.0;
+        sc.best = INFINITY;
     }
     for (int round = 0; round < 8; ++round) {
         // y_R = b / s - E (S x)_B, then r_B = bhat - (S x)_B - E^T y_R
@@ -671,8 +696,16 @@ __device__ __forceinline__ bool kbp_solve_tc(const BatchDesc& d, int rank, int k
             sc.it = 0;
             sc.rnorm2 = nn[0];
             sc.flag = (sc.status != CPS_OK || nn[0] <= sc.thresh2 || sc.total >= max_iter) ? 1 : 0;
+            sc.keep = round_ends(sc, d.best != nullptr, round == 7);
         }
         __syncthreads();
+        if (sc.keep) {
+            double* to = sc.keep == 1 ? d.best : d.x;
+            const double* from = sc.keep == 1 ? d.x : d.best;
+            for (int i = rlo + (int)threadIdx.x; i < rhi; i += kBB) to[perm[i]] = from[perm[i]];
+            for (int i = lo + (int)threadIdx.x; i < hi; i += kBB)
+                to[perm[nR + i]] = from[perm[nR + i]];
+        }
         if (sc.flag) break;
     }
     __syncthreads();

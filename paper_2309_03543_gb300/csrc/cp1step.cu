@@ -432,7 +432,7 @@ static int cp1_step_one_launch(cps_sys sx, cps_sys sy, double* du, double toll,
         d.t = s->wp1;
         d.a32 = s->a32;
         d.s32 = s->s32;
-        d.best = s->wbest;
+        d.best = tc || !mixed ? nullptr : s->wbest;
         d.partials = s->partials;
         d.st = s->st;
         d.n = nt;

@@ -417,6 +417,7 @@ int ensure_gsync(cps_sys s);
 bool jacobi_resident(cps_sys s);
 int jacobi_run(cps_sys s, int grid, const void* win, size_t win_bytes, cudaStream_t stream);
 size_t schur_window_bytes(cps_sys s);
+int true_residual2(cps_sys s, const double* b, const double* x, double* r2, cudaStream_t stream);
 int solve_impl(cps_sys sys, const double* b, double* x, double rtol, int64_t max_iter,
                int precision, cps_stats* stats, cudaStream_t stream);
 int solve_batch_impl(const cps_sys* systems, int nsys, const double* const* b,

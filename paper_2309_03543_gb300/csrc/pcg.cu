@@ -831,12 +831,68 @@ static int probe_schur(cps_sys s, const double* b, long long probe, int grid, bo
     return CPS_OK;
 }
 
+// ||b - A x||^2 (mesh order) into *r2; r, p0 and y are scratch.
+int true_residual2(cps_sys s, const double* b, const double* x, double* r2, cudaStream_t stream) {
+    const Run<float> f = make_run<float>(s);
+    k_res64<<<s->grid, kBlock, 0, stream>>>(b, x, s->s, s->a, s->col, s->nt, f.r, f.p0, f.y, 0.0, 0.0,
+                                            0, 1, 1, s->partials, s->st);
+    CPS_CUDA_TRY(s->ctx, cudaGetLastError());
+    CgState h{};
+    const int rc = read_state(s, stream, &h);
+    if (rc == CPS_OK) *r2 = h.rnorm2;
+    return rc;
+}
+
+// The iterate with the least true residual, which CPS_MIXED returns where it
+// does not reach rtol: the caller's start and the end of every run of a FP64
+// solve are the iterates whose true residual is formed.
+struct Least {
+    bool on = false;
+    double best = INFINITY;      // ||b - A x||^2 of the iterate in wbest
+
+    // a run ended at xx with ||b - A xx||^2 = r2, and another one follows
+    int offer(cps_sys s, const double* xx, double r2, cudaStream_t stream) {
+        if (!on || !(r2 < best)) return CPS_OK;
+        best = r2;
+        CPS_CUDA_TRY(s->ctx, cudaMemcpyAsync(s->wbest, xx, sizeof(double) * s->nt,
+                                             cudaMemcpyDeviceToDevice, stream));
+        return CPS_OK;
+    }
+
+    // xx (the last one, h.rnorm2) becomes the least of the runs' ends; *start: the
+    // caller's start x0 (mesh order) is less still, its residual then in h
+    int finish(cps_sys s, const double* b, const double* x0, double* xx, CgState& h, bool* start,
+               cudaStream_t stream) {
+        *start = false;
+        if (!on) return CPS_OK;
+        double r0 = INFINITY;
+        const int rc = true_residual2(s, b, x0, &r0, stream);
+        if (rc) return rc;
+        if (best < h.rnorm2 || std::isnan(h.rnorm2)) {
+            if (best < INFINITY)
+                CPS_CUDA_TRY(s->ctx, cudaMemcpyAsync(xx, s->wbest, sizeof(double) * s->nt,
+                                                     cudaMemcpyDeviceToDevice, stream));
+            h.rnorm2 = best;
+        }
+        if (r0 < h.rnorm2) {
+            *start = true;
+            h.rnorm2 = r0;
+        }
+        return CPS_OK;
+    }
+};
+
 // A whole solve on the explicit Schur rows (schur.cu; the caller has set them
 // up): `per` iterations of the solve's method per CG iteration on S (2 for
 // Jacobi, 1 for IC(0) and the reduced system).
 static int solve_two_cyclic(cps_sys s, const double* b, double* x, double rtol, int64_t max_iter,
                             int per, int grid, bool window, cps_stats* stats,
-                            cudaStream_t stream) {
+                            cudaStream_t stream, bool keep_least = false) {
+    Least least;
+    least.on = keep_least;
+    if (keep_least)
+        CPS_CUDA_TRY(s->ctx, cudaMemcpyAsync(s->wx, x, sizeof(double) * s->nt,
+                                             cudaMemcpyDeviceToDevice, stream));
     const int64_t n = s->nt;
     int64_t total = 0, launches = 0;
     if (window) {
@@ -862,6 +918,18 @@ static int solve_two_cyclic(cps_sys s, const double* b, double* x, double rtol, 
         total += done < left ? done : left;
         status = h.status;
         if (status != CPS_OK || h.rnorm2 <= h.thresh2 || total >= max_iter) break;
+        rc = least.offer(s, x, h.rnorm2, stream);
+        if (rc) return rc;
+    }
+    if (status == CPS_OK && !(h.rnorm2 <= h.thresh2)) {
+        bool start = false;
+        int rc = least.finish(s, b, s->wx, x, h, &start, stream);
+        if (rc) return rc;
+        if (start) {
+            CPS_CUDA_TRY(s->ctx, cudaMemcpyAsync(x, s->wx, sizeof(double) * n,
+                                                 cudaMemcpyDeviceToDevice, stream));
+            CPS_CUDA_TRY(s->ctx, cudaStreamSynchronize(stream));
+        }
     }
     if (window) {
         int rc = l2_set_aside(s, 0, stream);
@@ -1010,8 +1078,10 @@ static int choose_ic0_path(cps_sys s, const Run<double>& v, const double* b, con
     return CPS_OK;
 }
 
+// keep_least: where rtol is not reached, x becomes the iterate with the least true
+// residual (CPS_MIXED).
 static int solve_fp64(cps_sys s, const double* b, double* x, double rtol, int64_t max_iter,
-                      cps_stats* stats, cudaStream_t stream) {
+                      cps_stats* stats, cudaStream_t stream, bool keep_least = false) {
     const int64_t n = s->nt;
     const int g = s->grid;
     const bool ic0 = s->precond == CPS_PC_IC0;
@@ -1031,7 +1101,8 @@ static int solve_fp64(cps_sys s, const double* b, double* x, double rtol, int64_
         bool take = false;
         int rc = choose_two_cyclic(s, b, stream, &take);
         if (rc) return rc;
-        if (take) return solve_two_cyclic(s, b, x, rtol, max_iter, 2, 0, false, stats, stream);
+        if (take)
+            return solve_two_cyclic(s, b, x, rtol, max_iter, 2, 0, false, stats, stream, keep_least);
     }
     const bool cluster = !ic0 && s->tune[CPS_FP64].path == 1;
     const bool persistent = !ic0 && (s->tune[CPS_FP64].path == 2 || s->tune[CPS_FP64].path == 4);
@@ -1060,9 +1131,14 @@ static int solve_fp64(cps_sys s, const double* b, double* x, double rtol, int64_
     if (ic0 && s->ncolours == 2 && s->tune[CPS_FP64].ic0_path == 1 &&
         schur_setup(s, true, stream) == CPS_OK)
         return solve_two_cyclic(s, b, x, rtol, max_iter, 1, 0, s->tune[CPS_FP64].ic0_win != 0,
-                                stats, stream);
+                                stats, stream, keep_least);
     CgState h{};
     int status = CPS_OK;
+    Least least;
+    least.on = keep_least;
+    if (keep_least && !ic0)         // (IC(0) leaves x as it is until the end)
+        CPS_CUDA_TRY(s->ctx, cudaMemcpyAsync(s->wx, x, sizeof(double) * n,
+                                             cudaMemcpyDeviceToDevice, stream));
     // A restart recomputes r = b - A x when the recursively updated residual
     // has met rtol but the true residual has not (rounding drift).
     for (int restart = 0; restart < 8; ++restart) {
@@ -1083,6 +1159,8 @@ static int solve_fp64(cps_sys s, const double* b, double* x, double rtol, int64_
             rc = read_state(s, stream, &h);
             if (rc) return rc;
             if (status != CPS_OK || h.rnorm2 <= h.thresh2 || total >= max_iter) break;
+            rc = least.offer(s, xx, h.rnorm2, stream);
+            if (rc) return rc;
             continue;
         }
         k_init64<<<g, kBlock, 0, stream>>>(bb, xx, v.s, v.a, v.col, n, v.y, v.r, v.p0, rtol,
@@ -1109,6 +1187,8 @@ static int solve_fp64(cps_sys s, const double* b, double* x, double rtol, int64_
             rc = read_state(s, stream, &h);
             if (rc) return rc;
             if (status != CPS_OK || h.rnorm2 <= h.thresh2 || total >= max_iter) break;
+            rc = least.offer(s, xx, h.rnorm2, stream);
+            if (rc) return rc;
             continue;
         }
         if (ic0) {
@@ -1136,11 +1216,22 @@ static int solve_fp64(cps_sys s, const double* b, double* x, double rtol, int64_
         rc = read_state(s, stream, &h);
         if (rc) return rc;
         if (status != CPS_OK || h.rnorm2 <= h.thresh2 || total >= max_iter) break;
+        rc = least.offer(s, xx, h.rnorm2, stream);
+        if (rc) return rc;
     }
-    if (ic0) {
+    bool start = false;
+    if (status == CPS_OK && !(h.rnorm2 <= h.thresh2)) {
+        int rc = least.finish(s, b, ic0 ? x : s->wx, xx, h, &start, stream);
+        if (rc) return rc;
+    }
+    if (ic0 && !start) {
         k_permute_out<<<g, kBlock, 0, stream>>>(s->wx, s->perm, n, x);
         ++launches;
         CPS_CUDA_TRY(s->ctx, cudaGetLastError());
+        CPS_CUDA_TRY(s->ctx, cudaStreamSynchronize(stream));
+    } else if (start && !ic0) {
+        CPS_CUDA_TRY(s->ctx, cudaMemcpyAsync(x, s->wx, sizeof(double) * n,
+                                             cudaMemcpyDeviceToDevice, stream));
         CPS_CUDA_TRY(s->ctx, cudaStreamSynchronize(stream));
     }
     if (window) {
@@ -1442,7 +1533,7 @@ static int solve_mixed(cps_sys s, const double* b, double* x, double rtol, int64
             const Tuning d = default_tuning(s);
             for (int k = 0; k < 3; ++k) t.k[k] = d.k[k];
         }
-        return solve_fp64(s, b, x, rtol, max_iter, stats, stream);
+        return solve_fp64(s, b, x, rtol, max_iter, stats, stream, true);
     }
     const Run<float> v = make_run<float>(s);
     if (!s->tune[CPS_MIXED].done) {

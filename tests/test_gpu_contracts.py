@@ -143,3 +143,63 @@ def test_first_mixed_solve_times_no_kernels_it_does_not_run(ctx):
     _, st = seconds()
     assert st.refinements > 1 and st.rel_res <= 1e-10
     s.free()
+
+
+def _rises(p):
+    """A right-hand side from whose start x = 0 the residual of CG rises several
+    times before it falls."""
+    return torch.ones(p.mesh.nt, dtype=torch.float64, device="cuda")
+
+
+@pytest.mark.parametrize("pc", [cps.PC_JACOBI, cps.PC_IC0])
+@pytest.mark.parametrize("mesh", ["lattice", "defect"])
+@pytest.mark.parametrize("start", ["zero", "better"])
+def test_unconverged_mixed_solve_returns_the_least_residual(ctx, pc, mesh, start):
+    """Eight iterations, after which the residual is above the start's: the start
+    comes back, with its residual, whichever loop ran; from a start better than
+    any iterate of a solve that cannot reach its tolerance, no worse a one."""
+    p = synth.channel_block_problem(40, seed=4) if mesh == "lattice" else synth.defect_problem(20, seed=3)
+    s = _assemble(ctx, p)
+    s.set_precond(pc)
+    b = _rises(p)
+    A = oracle.assemble_problem(p)
+    bn = b.cpu().numpy()
+
+    def rel(x):
+        return np.linalg.norm(bn - A.matvec(x.cpu().numpy())) / np.linalg.norm(bn)
+
+    if start == "zero":
+        x, st = s.solve(b, rtol=1e-13, max_iter=8, precision=cps.MIXED, check=False)
+        assert st.status == cps._cps.ERR_NOT_CONVERGED
+        assert st.rel_res <= 1.0 + 1e-12 and abs(rel(x) - st.rel_res) <= 1e-9
+    else:
+        x0, _ = s.solve(b, rtol=1e-10)
+        _, st0 = s.solve(b, x=x0.clone(), rtol=1e-10)     # its residual, as the solver forms it
+        for k in (2, 4, 40):
+            x, st = s.solve(b, x=x0.clone(), rtol=0.0, max_iter=k, precision=cps.MIXED, check=False)
+            assert st.status == cps._cps.ERR_NOT_CONVERGED
+            assert st.rel_res <= st0.rel_res * (1 + 1e-6) and rel(x) <= 1.05 * st0.rel_res
+    s.free()
+
+
+@pytest.mark.parametrize("mesh", ["lattice", "defect"])
+def test_unconverged_mixed_ensemble_returns_the_least_residual(ctx, mesh):
+    """Members solved by single blocks and by teams, after eight iterations."""
+    sizes = [30000, 600, 9000]
+    if mesh == "lattice":
+        probs = [synth.ensemble_member_problem(nt, seed=70 + i) for i, nt in enumerate(sizes)]
+    else:
+        probs = [synth.defect_problem(n, seed=5 + i) for i, n in enumerate((120, 18, 60))]
+    systems = [_assemble(ctx, p) for p in probs]
+    bs = [_rises(p) for p in probs]
+    xs = [torch.zeros_like(b) for b in bs]
+    st = cps.solve_batch(systems, bs, xs, rtol=1e-10, max_iter=8, precision=cps.MIXED, check=False)
+    for s, b, x, t in zip(systems, bs, xs, st):
+        assert t.status == cps._cps.ERR_NOT_CONVERGED and t.iters <= 8
+        r = float((b - s.matvec(x)).norm() / b.norm())
+        assert t.rel_res <= 1.0 + 1e-12 and abs(r - t.rel_res) <= 1e-9
+    # and in FP64 the last iterate, as before
+    st = cps.solve_batch(systems, bs, xs, rtol=1e-10, max_iter=8, check=False)
+    assert all(t.rel_res > 1.0 for t in st)
+    for s in systems:
+        s.free()
