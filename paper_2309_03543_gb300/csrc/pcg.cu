@@ -606,20 +606,30 @@ static int persistent_1red(cps_sys s, const Run<double>& v, int grid, const void
                             bytes, grid, stream);
 }
 
+// The probes' right-hand side, in wb: 0x3F bytes, a small positive constant.  Not the
+// caller's, whose zero, NaN or infinity would end a run at once and leave a choice,
+// remembered for every system of this size, that nothing was measured for.
+static int probe_rhs(cps_sys s, cudaStream_t stream) {
+    CPS_CUDA_TRY(s->ctx, cudaMemsetAsync(s->wb, 0x3F, sizeof(double) * s->nt, stream));
+    return CPS_OK;
+}
+
 // For Jacobi solves, times a short run (64 iterations; 256 on large systems)
 // of each path that applies from x = 0 and keeps the fastest: graph-replayed
 // streaming kernels, the one-launch cluster solve (systems that fit one
 // cluster's shared memory), streaming with the matrix or with the vectors
 // r, p, q held in persisting L2 (large systems whose window fits the
 // set-aside), and the persistent grid-synchronised launch.
-static int choose_fp64_path(cps_sys s, const Run<double>& v, const double* b,
-                            cudaStream_t stream) {
+static int choose_fp64_path(cps_sys s, const Run<double>& v, cudaStream_t stream) {
     Tuning& t = s->tune[CPS_FP64];
     t.path_done = true;
     t.path = 0;
     t.l2win = 0;
     t.pgrid = 0;
     if (s->precond != CPS_PC_JACOBI) return CPS_OK;
+    const double* b = s->wb;
+    const int brc = probe_rhs(s, stream);
+    if (brc) return brc;
     const bool try_cluster = s->nt <= cluster_max_rows(s->ctx);
     const bool big = !try_cluster && s->nt >= kTuneMinRows;
     const long long probe = s->nt >= kTuneMinRows ? 256 : 64;
@@ -954,10 +964,11 @@ static int solve_two_cyclic(cps_sys s, const double* b, double* x, double rtol, 
 // solve is hundreds of iterations, against which the colouring and the rows
 // cost nothing; a CP1 system converges in about eight) where one CG iteration
 // on S costs less than two of the loop the tuner chose.
-static int choose_two_cyclic(cps_sys s, const double* b, cudaStream_t stream, bool* take) {
+static int choose_two_cyclic(cps_sys s, cudaStream_t stream, bool* take) {
     *take = false;
     Tuning& t = s->tune[CPS_FP64];
     if (t.pinned || s->kind != CPS_KIND_CP2 || t.tc == 2) return CPS_OK;
+    const bool had_rows = s->sch.buf != nullptr;
     bool two = false;
     int rc = two_colour_order(s, stream, &two);
     if (rc == CPS_OK && two) rc = schur_setup(s, false, stream);
@@ -971,18 +982,23 @@ static int choose_two_cyclic(cps_sys s, const double* b, cudaStream_t stream, bo
         CPS_CUDA_TRY(s->ctx, cudaEventCreate(&e0));
         CPS_CUDA_TRY(s->ctx, cudaEventCreate(&e1));
         double us = 0.0, best = 0.0;
-        rc = probe_schur(s, b, s->nt >= kTuneMinRows ? 256 : 64, 0, false, e0, e1, stream, &us);
+        rc = probe_rhs(s, stream);
+        if (rc == CPS_OK)
+            rc = probe_schur(s, s->wb, s->nt >= kTuneMinRows ? 256 : 64, 0, false, e0, e1, stream,
+                             &us);
         cudaEventDestroy(e0);
         cudaEventDestroy(e1);
         if (rc) return rc;
+        if (us <= 0.0) return CPS_OK;           // did not run: nothing to remember
         for (double p : t.probe_us)
             if (p > 0.0 && (best == 0.0 || p < best)) best = p;
-        t.tc = us > 0.0 && (best == 0.0 || us < 2.0 * best) ? 1 : 2;
+        t.tc = best == 0.0 || us < 2.0 * best ? 1 : 2;
         t.tc_us = us;
         update_cached_tuning(s, CPS_FP64, [&](Tuning& c) {
             c.tc = t.tc;
             c.tc_us = t.tc_us;
         });
+        if (t.tc == 2 && !had_rows) free_schur(s);
     }
     *take = t.tc == 1;
     return CPS_OK;
@@ -992,9 +1008,8 @@ static int choose_two_cyclic(cps_sys s, const double* b, cudaStream_t stream, bo
 // large systems) of the graph-replayed streaming kernels and of the
 // persistent single-reduction launch on the scaled Schur rows (without and,
 // where the set-aside holds them, with its vectors in persisting L2) and keeps
-// the fastest.  bb is the right-hand side b in colour order.
-static int choose_ic0_path(cps_sys s, const Run<double>& v, const double* b, const double* bb,
-                           cudaStream_t stream) {
+// the fastest.  Overwrites wb and wx.
+static int choose_ic0_path(cps_sys s, const Run<double>& v, cudaStream_t stream) {
     Tuning& t = s->tune[CPS_FP64];
     t.ic0_done = true;
     t.ic0_path = 0;
@@ -1022,7 +1037,7 @@ static int choose_ic0_path(cps_sys s, const Run<double>& v, const double* b, con
     for (int ci = 0; ci < nc && rc == CPS_OK; ++ci) {
         const Cand c = cands[ci];
         double us = 0.0;
-        if (c.path == 1) rc = probe_schur(s, b, probe, 0, c.win != 0, e0, e1, stream, &us);
+        if (c.path == 1) rc = probe_schur(s, s->wb, probe, 0, c.win != 0, e0, e1, stream, &us);
         else rc = l2_set_aside(s, c.win, stream);
         for (int rep = 0; rep < 2 && rc == CPS_OK && c.path == 0; ++rep) {   // the first warms up
             if (cudaMemsetAsync(s->wx, 0, sizeof(double) * s->nt, stream) != cudaSuccess ||
@@ -1030,8 +1045,8 @@ static int choose_ic0_path(cps_sys s, const Run<double>& v, const double* b, con
                 rc = CPS_ERR_CUDA;
                 break;
             }
-            k_init64<<<s->grid, kBlock, 0, stream>>>(bb, s->wx, v.s, v.a, v.col, s->nt, v.y, v.r,
-                                                     v.p0, 0.0, probe, 0, s->partials, s->st);
+            k_init64<<<s->grid, kBlock, 0, stream>>>(s->wb, s->wx, v.s, v.a, v.col, s->nt, v.y,
+                                                     v.r, v.p0, 0.0, probe, 0, s->partials, s->st);
             CgState h{};
             enqueue_precond<double>(s, v, stream);
             k_copy<double><<<s->grid, kBlock, 0, stream>>>(v.p0, v.z, s->nt);
@@ -1094,12 +1109,12 @@ static int solve_fp64(cps_sys s, const double* b, double* x, double rtol, int64_
         if (rc) return rc;
     }
     if (!ic0 && !s->tune[CPS_FP64].path_done) {
-        int rc = choose_fp64_path(s, v, b, stream);
+        int rc = choose_fp64_path(s, v, stream);
         if (rc) return rc;
     }
     if (!ic0) {
         bool take = false;
-        int rc = choose_two_cyclic(s, b, stream, &take);
+        int rc = choose_two_cyclic(s, stream, &take);
         if (rc) return rc;
         if (take)
             return solve_two_cyclic(s, b, x, rtol, max_iter, 2, 0, false, stats, stream, keep_least);
@@ -1114,19 +1129,14 @@ static int solve_fp64(cps_sys s, const double* b, double* x, double rtol, int64_
         if (rc) return rc;
     }
     if (ic0) {
+        if (!s->tune[CPS_FP64].ic0_done) {
+            int rc = choose_ic0_path(s, v, stream);
+            if (rc) return rc;
+        }
         k_permute_in<<<g, kBlock, 0, stream>>>(b, x, s->perm, n, s->wb, s->wx);
         ++launches;
         bb = s->wb;
         xx = s->wx;
-        if (!s->tune[CPS_FP64].ic0_done) {
-            // the probe runs from x = 0 in wx: keep the caller's start in wbest
-            CPS_CUDA_TRY(s->ctx, cudaMemcpyAsync(s->wbest, s->wx, sizeof(double) * n,
-                                                 cudaMemcpyDeviceToDevice, stream));
-            int rc = choose_ic0_path(s, v, b, bb, stream);
-            if (rc) return rc;
-            CPS_CUDA_TRY(s->ctx, cudaMemcpyAsync(s->wx, s->wbest, sizeof(double) * n,
-                                                 cudaMemcpyDeviceToDevice, stream));
-        }
     }
     if (ic0 && s->ncolours == 2 && s->tune[CPS_FP64].ic0_path == 1 &&
         schur_setup(s, true, stream) == CPS_OK)
@@ -1359,7 +1369,8 @@ static int solve_reduced(cps_sys s, const double* b, double* x, double rtol, int
         // slot 0 graph, 1 persistent, 2 graph + window, 3 persistent + window,
         // 4 persistent single-reduction on the explicit rows, 5 the same + its
         // five vectors in persisting L2 (persistent at a few grid sizes)
-        k_permute_in<<<g, kBlock, 0, stream>>>(b, x, s->perm, n, s->wb, s->wx);
+        const int brc = probe_rhs(s, stream);
+        if (brc) return brc;
         const long long probe = nB >= kTuneMinRows ? 256 : 64;
         const bool try_win = nB >= kTuneMinRows && l2_window_fits(s, 2);
         const bool try_win5 = nB >= kTuneMinRows && l2_window_fits(s, 3);
@@ -1400,7 +1411,7 @@ static int solve_reduced(cps_sys s, const double* b, double* x, double rtol, int
             const int kind = kind_of(c.slot);
             const bool pers = kind != 0;
             double us = 0.0;
-            if (kind == 2) rc = probe_schur(s, b, probe, 0, c.win != 0, e0, e1, stream, &us);
+            if (kind == 2) rc = probe_schur(s, s->wb, probe, 0, c.win != 0, e0, e1, stream, &us);
             else rc = l2_set_aside(s, c.win, stream);
             for (int rep = 0; rep < 2 && rc == CPS_OK && kind != 2; ++rep) {
                 CPS_CUDA_TRY(s->ctx, cudaMemsetAsync(xx, 0, sizeof(double) * n, stream));

@@ -203,3 +203,33 @@ def test_unconverged_mixed_ensemble_returns_the_least_residual(ctx, mesh):
     assert all(t.rel_res > 1.0 for t in st)
     for s in systems:
         s.free()
+
+
+@pytest.mark.parametrize("pc", [cps.PC_JACOBI, cps.PC_IC0, cps.PC_REDUCED])
+@pytest.mark.parametrize("first", ["nan", "inf", "zero"])
+def test_the_first_right_hand_side_does_not_choose_the_loop(cuda_device, pc, first):
+    """A first solve that cannot iterate leaves the choice that any other one
+    does, to its own system and to the next one of its size."""
+    c = cps.Context(0)                                     # remembers no size yet
+    p = synth.channel_block_problem(60, seed=4)
+    good = torch.as_tensor(synth.rhs(p.mesh, 1), device="cuda")
+    bad = good.clone() if first != "zero" else torch.zeros_like(good)
+    if first != "zero":
+        bad[17] = float(first)
+    for rhs in (bad, good):
+        s = _assemble(c, p)
+        s.set_precond(pc)
+        s.solve(rhs, rtol=1e-10, check=False)
+        x, st = s.solve(good, rtol=1e-10)
+        assert st.rel_res <= 1e-10
+        tu = s.tuning()
+        probe = tu["probe_us_per_iter"]
+        # the loop on the Schur rows ran when it was timed, and was the faster one
+        if pc == cps.PC_JACOBI:
+            assert tu["two_cyclic"] and 1.0 < tu["two_cyclic_us_per_iter"] < 100.0
+        elif pc == cps.PC_IC0:
+            assert tu["ic0_persistent"] and 1.0 < probe["ic0_persistent"] < 100.0
+        else:
+            assert tu["reduced_single_reduction"] and 1.0 < probe["reduced_persistent_1red"] < 100.0
+        s.free()
+    c.close()
