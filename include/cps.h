@@ -352,7 +352,8 @@ int cps_cp2_kernel_times(cps_sys sys, float* ms);
  *     two-cyclic form: from a zero residual on one colour, two Jacobi-PCG
  *     iterations are one CG iteration on the other colour's Schur complement
  *     (half the unknowns), and stats->iters counts two for each (max_iter
- *     bounds that count);
+ *     bounds that count: the last iteration of an odd one runs on all cells,
+ *     and is left out in the one-launch ensemble and CP1 step);
  *   CPS_PATH_STREAM: graph-replayed streaming kernels, any size;
  *   CPS_PATH_CLUSTER (FP64 Jacobi only): the whole solve in one launch of a
  *     single thread-block cluster whose shared memory holds the system;

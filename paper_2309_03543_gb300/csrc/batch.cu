@@ -585,8 +585,8 @@ static int solve_batch_one_launch(const cps_sys* systems, int nsys, const double
         d.n = s->nt;
     }
     // An ensemble of two-coloured CP2 systems runs on their Schur rows, in either
-    // precision; any other on all cells.
-    bool tc = true;
+    // precision; any other on all cells, and any for fewer iterations than a step counts.
+    bool tc = max_iter >= 2;
     for (int i = 0; i < nsys && tc; ++i) {
         cps_sys s = systems[i];
         int rc = CPS_OK;

@@ -465,8 +465,9 @@ __device__ __forceinline__ bool kbp_solve(const BatchDesc& d, int64_t lo, int64_
 // are one CG iteration on S, half of the rows), by this block (tc null) or this
 // member's share (rank of k) of the red cells, of the black rows and of the
 // cells of either colour.  The recurrences, restarts, results and the return
-// value are kbp_solve's, iterations counted two a step; per step one pass over
-// the rows of S (80 B and 9 FP64 FMAs a row) and one over the vectors.  The
+// value are kbp_solve's, iterations counted two a step (max_iter at least 2; an
+// odd one's last iteration is not made); per step one pass over the rows of S (80 B
+// and 9 FP64 FMAs a row) and one over the vectors.  The
 // stop test runs on the steps whose low bits are all set in mask.
 __device__ __forceinline__ bool kbp_solve_tc(const BatchDesc& d, int rank, int k, TeamCtx* tc,
                                              double rtol, long long max_iter, int mask) {
@@ -557,7 +558,7 @@ __device__ __forceinline__ bool kbp_solve_tc(const BatchDesc& d, int rank, int k
             sc.it = 0;
             sc.ig = sc.c = 0.0;
             sc.flag = v3[1] == 0.0 ? 3
-                      : (v3[2] > sc.thresh2 && sc.budget > 0 && v3[0] > 0.0) ? 0 : 1;
+                      : (v3[2] > sc.thresh2 && sc.budget > 1 && v3[0] > 0.0) ? 0 : 1;
         }
         __syncthreads();
         if (sc.flag == 3) {           // b = 0: x = 0
@@ -611,7 +612,7 @@ __device__ __forceinline__ bool kbp_solve_tc(const BatchDesc& d, int rank, int k
             if (!ok) break;
             if (threadIdx.x == 0) {
                 const double g = g3[0], dl = g3[1];
-                bool halt = !(g > 0.0) || 2 * sc.it >= sc.budget;
+                bool halt = !(g > 0.0) || 2 * sc.it + 2 > sc.budget;
                 if (check) {
                     sc.rnorm2 = g3[2];
                     if (g3[2] <= sc.thresh2) halt = true;
@@ -691,11 +692,10 @@ __device__ __forceinline__ bool kbp_solve_tc(const BatchDesc& d, int rank, int k
         sum1(nn);
         if (!ok) break;
         if (threadIdx.x == 0) {
-            const long long left = max_iter - sc.total, made = 2 * sc.it;
-            sc.total += made < left ? made : left;
+            sc.total += 2 * sc.it;
             sc.it = 0;
             sc.rnorm2 = nn[0];
-            sc.flag = (sc.status != CPS_OK || nn[0] <= sc.thresh2 || sc.total >= max_iter) ? 1 : 0;
+            sc.flag = (sc.status != CPS_OK || nn[0] <= sc.thresh2 || sc.total + 1 >= max_iter) ? 1 : 0;
             sc.keep = round_ends(sc, d.best != nullptr, round == 7);
         }
         __syncthreads();

@@ -386,10 +386,12 @@ static int cp1_step_one_launch(cps_sys sx, cps_sys sy, double* du, double toll,
                                cps_cp1_stats* stats, cudaStream_t stream) {
     Cp1Data* c = sx->cp1;
     const int64_t nt = sx->nt;
-    // on the Schur rows where the cell graph has two colours (one for both systems)
-    bool tc = true;
+    // on the Schur rows where the cell graph has two colours (one for both systems) and
+    // a solve may make the two iterations that a step counts
+    bool tc = max_iter >= 2;
     cps_sys sys[2] = {sx, sy};
     for (cps_sys s : sys) {
+        if (!tc) break;
         int rc = two_colour_order(s, stream, &tc);
         if (rc == CPS_OK && tc) rc = schur_setup(s, false, stream);
         if (rc == CPS_ERR_NOMEM) {              // no room for the rows

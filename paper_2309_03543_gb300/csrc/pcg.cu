@@ -894,7 +894,7 @@ struct Least {
 
 // A whole solve on the explicit Schur rows (schur.cu; the caller has set them
 // up): `per` iterations of the solve's method per CG iteration on S (2 for
-// Jacobi, 1 for IC(0) and the reduced system).
+// Jacobi, 1 for IC(0) and the reduced system), max_iter a multiple of it.
 static int solve_two_cyclic(cps_sys s, const double* b, double* x, double rtol, int64_t max_iter,
                             int per, int grid, bool window, cps_stats* stats,
                             cudaStream_t stream, bool keep_least = false) {
@@ -914,7 +914,7 @@ static int solve_two_cyclic(cps_sys s, const double* b, double* x, double rtol, 
     // restarts from the true residual, as in solve_fp64
     for (int restart = 0; restart < 8; ++restart) {
         const int64_t left = max_iter - total;
-        int rc = schur_init(s, b, x, rtol, left / per + (left % per ? 1 : 0), stream);
+        int rc = schur_init(s, b, x, rtol, left / per, stream);
         if (rc == CPS_OK) rc = schur_run(s, grid, window, stream);
         if (rc == CPS_OK) rc = schur_back(s, b, stream);
         if (rc) return rc;
@@ -924,8 +924,7 @@ static int solve_two_cyclic(cps_sys s, const double* b, double* x, double rtol, 
         CPS_CUDA_TRY(s->ctx, cudaGetLastError());
         rc = read_state(s, stream, &h);
         if (rc) return rc;
-        const int64_t done = h.iter * per;
-        total += done < left ? done : left;
+        total += h.iter * per;
         status = h.status;
         if (status != CPS_OK || h.rnorm2 <= h.thresh2 || total >= max_iter) break;
         rc = least.offer(s, x, h.rnorm2, stream);
@@ -1112,12 +1111,19 @@ static int solve_fp64(cps_sys s, const double* b, double* x, double rtol, int64_
         int rc = choose_fp64_path(s, v, stream);
         if (rc) return rc;
     }
-    if (!ic0) {
+    if (!ic0 && max_iter >= 2) {
         bool take = false;
         int rc = choose_two_cyclic(s, stream, &take);
         if (rc) return rc;
-        if (take)
-            return solve_two_cyclic(s, b, x, rtol, max_iter, 2, 0, false, stats, stream, keep_least);
+        if (take) {
+            cps_stats two{};
+            rc = solve_two_cyclic(s, b, x, rtol, max_iter - max_iter % 2, 2, 0, false, &two, stream,
+                                  keep_least);
+            if (stats) *stats = two;
+            if (rc != CPS_ERR_NOT_CONVERGED || two.iters + 1 != max_iter) return rc;
+            total = two.iters;          // an odd bound's last iteration, on all cells
+            launches = two.launches;
+        }
     }
     const bool cluster = !ic0 && s->tune[CPS_FP64].path == 1;
     const bool persistent = !ic0 && (s->tune[CPS_FP64].path == 2 || s->tune[CPS_FP64].path == 4);
@@ -1138,7 +1144,7 @@ static int solve_fp64(cps_sys s, const double* b, double* x, double rtol, int64_
         bb = s->wb;
         xx = s->wx;
     }
-    if (ic0 && s->ncolours == 2 && s->tune[CPS_FP64].ic0_path == 1 &&
+    if (ic0 && max_iter >= 1 && s->ncolours == 2 && s->tune[CPS_FP64].ic0_path == 1 &&
         schur_setup(s, true, stream) == CPS_OK)
         return solve_two_cyclic(s, b, x, rtol, max_iter, 1, 0, s->tune[CPS_FP64].ic0_win != 0,
                                 stats, stream, keep_least);

@@ -233,3 +233,91 @@ def test_the_first_right_hand_side_does_not_choose_the_loop(cuda_device, pc, fir
             assert tu["reduced_single_reduction"] and 1.0 < probe["reduced_persistent_1red"] < 100.0
         s.free()
     c.close()
+
+
+def test_max_iter_bounds_the_iterations_made(ctx):
+    """On a system whose Jacobi solves count two iterations a step: none leaves x
+    as it is, one is the steepest descent step, an odd bound makes one more than
+    the even one below and not as many as the next (the energy norm of the error
+    falls with every iteration made)."""
+    p = synth.channel_block_problem(40, seed=4)
+    s = _assemble(ctx, p)
+    A = oracle.assemble_problem(p)
+    b = torch.as_tensor(synth.rhs(p.mesh, 1), device="cuda")
+    s.solve(b, rtol=1e-10)
+    assert s.tuning()["two_cyclic"]
+    xs, _ = s.solve(b, rtol=1e-12, check=False)
+    x0 = xs + 1e-3 * xs.norm() / np.sqrt(p.mesh.nt) * torch.sin(torch.arange(p.mesh.nt, device="cuda").double())
+
+    def energy(x):
+        e = (x - xs).cpu().numpy()
+        return float(e @ A.matvec(e))
+
+    f = []
+    for k in range(10):
+        x, st = s.solve(b, x=x0.clone(), rtol=1e-13, max_iter=k, check=False)
+        assert st.iters == k and st.status == cps._cps.ERR_NOT_CONVERGED
+        r = b.cpu().numpy() - A.matvec(x.cpu().numpy())
+        assert abs(np.linalg.norm(r) / float(b.norm()) - st.rel_res) < 1e-6 * st.rel_res
+        f.append(energy(x))
+        if k == 0:
+            assert float((x - x0).norm()) <= 4e-16 * float(x0.norm())
+        if k == 1:
+            r0 = b - s.matvec(x0)
+            d = s.export_matrix()[0]
+            z = r0 / d
+            x1 = x0 + (r0 @ z) / (z @ s.matvec(z)) * z
+            assert float((x - x1).norm()) <= 1e-12 * float((x1 - x0).norm()) + 1e-15 * float(x1.norm())
+    assert all(f[k + 1] < f[k] for k in range(2, 9))
+    assert f[1] < f[0] and f[2] < f[0]
+    s.free()
+
+
+@pytest.mark.parametrize("sizes", [[600], [30000, 600]])
+def test_max_iter_bounds_the_ensembles_iterations(ctx, sizes):
+    probs = [synth.ensemble_member_problem(nt, seed=70 + i) for i, nt in enumerate(sizes)]
+    systems = [_assemble(ctx, p) for p in probs]
+    bs = [torch.as_tensor(synth.rhs(p.mesh, 80), device="cuda") for p in probs]
+
+    def run(k):
+        xs = [0.5 * torch.ones_like(b) for b in bs]
+        return xs, cps.solve_batch(systems, bs, xs, rtol=1e-13, max_iter=k, check=False)
+
+    for k in (0, 1):
+        xs, st = run(k)
+        assert all(t.iters == k for t in st)
+        if k == 0:
+            assert all(bool(torch.all((x - 0.5).abs() <= 1e-15)) for x in xs)
+    for k in (2, 6, 7, 9):
+        xs, st = run(k)
+        assert all(t.iters == k - k % 2 for t in st)
+        for u, v in zip(xs, run(k - k % 2)[0]):            # no work beyond what is counted
+            assert torch.equal(u, v)
+    for s in systems:
+        s.free()
+
+
+def test_max_iter_bounds_the_cp1_steps_solves(ctx):
+    p = _walls(synth.channel_block_problem(24, seed=6))
+    du_b = synth.cell_vector_field(p.mesh, 9, mean=(0.01, -0.02), scale=0.05)
+    sx, sy = _cp1_pair(ctx, p)
+    for k in (0, 1, 2, 3):
+        # the uncoupled sweep only: two solves
+        _, st = cps.cp1_step(sx, sy, du_b, max_outer=0, rtol=1e-15, max_iter=k, check=False)
+        assert st["solve_iters"] == 2 * (k if k < 2 else 2)
+    sx.free()
+    sy.free()
+
+
+@pytest.mark.parametrize("path", [cps.PATH_AUTO, cps.PATH_PERSISTENT_1RED])
+def test_ic0_solve_of_no_iteration_leaves_x(ctx, path):
+    p = synth.channel_block_problem(40, seed=4)
+    s = _assemble(ctx, p)
+    s.set_precond(cps.PC_IC0)
+    s.set_solver_path(path)
+    b = torch.as_tensor(synth.rhs(p.mesh, 1), device="cuda")
+    s.solve(b, rtol=1e-6)
+    x0 = torch.sin(torch.arange(p.mesh.nt, device="cuda").double())
+    x, st = s.solve(b, x=x0.clone(), max_iter=0, check=False)
+    assert st.iters == 0 and float((x - x0).norm()) <= 4e-16 * float(x0.norm())
+    s.free()
