@@ -226,6 +226,31 @@ int cps_set_batch_path(cps_ctx ctx, int path) {
 int cps_set_solver_path(cps_sys sys, int path) {
     if (!sys) return CPS_ERR_ARG;
     cps::Tuning& t = sys->tune[CPS_FP64];
+    const int var = path == CPS_PATH_CLUSTER_SSTEP3   ? 4
+                    : path == CPS_PATH_CLUSTER_SSTEP2 ? 3
+                    : path == CPS_PATH_CLUSTER_PIPE   ? 2
+                    : path == CPS_PATH_CLUSTER_1RED   ? 1
+                    : path == CPS_PATH_CLUSTER        ? 0
+                                                      : -1;
+    // a refused pin changes nothing (but for IC(0), which then runs without the window)
+    if (path < CPS_PATH_AUTO || path > CPS_PATH_CLUSTER_SSTEP3) return CPS_ERR_ARG;
+    if ((path == CPS_PATH_STREAM_1RED_L2 || path == CPS_PATH_PERSISTENT_L2 ||
+         path == CPS_PATH_STREAM_L2) && !cps::l2_vectors_fit(sys)) {
+        cps::set_error(sys->ctx, "set_solver_path: the persisting L2 set-aside cannot hold r, p, q");
+        return CPS_ERR_ARG;
+    }
+    if (path == CPS_PATH_PERSISTENT_1RED_L2 && !cps::l2_window_fits_mode(sys, 3)) {
+        cps::set_error(sys->ctx, "set_solver_path: the persisting L2 set-aside cannot hold "
+                                 "the five vectors of the single-reduction loop");
+        t.ic0_done = true;
+        t.ic0_path = 1;
+        t.ic0_win = 0;
+        return CPS_ERR_ARG;
+    }
+    if (var >= 0 && sys->nt > cps::cluster_max_rows(sys->ctx, var)) {
+        cps::set_error(sys->ctx, "set_solver_path: system too large for one cluster");
+        return CPS_ERR_ARG;
+    }
     t.pinned = path != CPS_PATH_AUTO;
     if (path >= CPS_PATH_STREAM && path <= CPS_PATH_PERSISTENT_1RED_L2) {
         // IC(0) in a two-colour order: the persistent single-reduction loop
@@ -233,7 +258,7 @@ int cps_set_solver_path(cps_sys sys, int path) {
         // the others
         t.ic0_done = true;
         t.ic0_path = (path == CPS_PATH_PERSISTENT_1RED || path == CPS_PATH_PERSISTENT_1RED_L2) ? 1 : 0;
-        t.ic0_win = path == CPS_PATH_PERSISTENT_1RED_L2 && cps::l2_window_fits_mode(sys, 3) ? 3 : 0;
+        t.ic0_win = path == CPS_PATH_PERSISTENT_1RED_L2 ? 3 : 0;
     }
     if (path == CPS_PATH_AUTO) {
         t.ic0_done = false;
@@ -252,23 +277,10 @@ int cps_set_solver_path(cps_sys sys, int path) {
         t.red_win = 0;
     } else if (path == CPS_PATH_STREAM_1RED || path == CPS_PATH_STREAM_1RED_L2) {
         // with L2: all five vectors of the loop where the set-aside holds them, else r, p, q
-        int win = 0;
-        if (path == CPS_PATH_STREAM_1RED_L2) {
-            win = cps::l2_window_fits_mode(sys, 3) ? 3 : 2;
-            if (!cps::l2_vectors_fit(sys)) {
-                cps::set_error(sys->ctx, "set_solver_path: the persisting L2 set-aside cannot hold r, p, q");
-                return CPS_ERR_ARG;
-            }
-        }
         t.path_done = true;
         t.path = 3;
-        t.l2win = win;
+        t.l2win = path == CPS_PATH_STREAM_1RED ? 0 : (cps::l2_window_fits_mode(sys, 3) ? 3 : 2);
     } else if (path == CPS_PATH_PERSISTENT_1RED || path == CPS_PATH_PERSISTENT_1RED_L2) {
-        if (path == CPS_PATH_PERSISTENT_1RED_L2 && !cps::l2_window_fits_mode(sys, 3)) {
-            cps::set_error(sys->ctx, "set_solver_path: the persisting L2 set-aside cannot hold "
-                                     "the five vectors of the single-reduction loop");
-            return CPS_ERR_ARG;
-        }
         t.path_done = true;
         t.path = 4;
         t.l2win = path == CPS_PATH_PERSISTENT_1RED_L2 ? 3 : 0;
@@ -277,57 +289,27 @@ int cps_set_solver_path(cps_sys sys, int path) {
         t.red_path = 2;
         t.red_win = path == CPS_PATH_PERSISTENT_1RED_L2 ? 3 : 0;
         t.red_pgrid = 0;
-    } else if (path == CPS_PATH_PERSISTENT) {
+    } else if (path == CPS_PATH_PERSISTENT || path == CPS_PATH_PERSISTENT_L2) {
         t.path_done = true;
         t.path = 2;
-        t.l2win = 0;
+        t.l2win = path == CPS_PATH_PERSISTENT_L2 ? 2 : 0;
         t.red_done = true;
         t.red_path = 1;
-        t.red_win = 0;
-        t.pgrid = 0;
-        t.red_pgrid = 0;
-    } else if (path == CPS_PATH_PERSISTENT_L2) {
-        if (!cps::l2_vectors_fit(sys)) {
-            cps::set_error(sys->ctx, "set_solver_path: the persisting L2 set-aside cannot hold r, p, q");
-            return CPS_ERR_ARG;
-        }
-        t.path_done = true;
-        t.path = 2;
-        t.l2win = 2;
-        t.red_done = true;
-        t.red_path = 1;
-        t.red_win = 2;
+        t.red_win = path == CPS_PATH_PERSISTENT_L2 ? 2 : 0;
         t.pgrid = 0;
         t.red_pgrid = 0;
     } else if (path == CPS_PATH_STREAM_L2) {
-        if (!cps::l2_vectors_fit(sys)) {
-            cps::set_error(sys->ctx, "set_solver_path: the persisting L2 set-aside cannot hold r, p, q");
-            return CPS_ERR_ARG;
-        }
         t.path_done = true;
         t.path = 0;
         t.l2win = 2;
         t.red_done = true;
         t.red_path = 0;
         t.red_win = 2;
-    } else if (path == CPS_PATH_CLUSTER || path == CPS_PATH_CLUSTER_1RED ||
-               path == CPS_PATH_CLUSTER_PIPE || path == CPS_PATH_CLUSTER_SSTEP2 ||
-               path == CPS_PATH_CLUSTER_SSTEP3) {
-        const int var = path == CPS_PATH_CLUSTER_SSTEP3   ? 4
-                        : path == CPS_PATH_CLUSTER_SSTEP2 ? 3
-                        : path == CPS_PATH_CLUSTER_PIPE   ? 2
-                        : path == CPS_PATH_CLUSTER_1RED   ? 1
-                                                          : 0;
-        if (sys->nt > cps::cluster_max_rows(sys->ctx, var)) {
-            cps::set_error(sys->ctx, "set_solver_path: system too large for one cluster");
-            return CPS_ERR_ARG;
-        }
+    } else {
         t.path_done = true;
         t.path = 1;
         t.l2win = 0;
         t.cluster_variant = var;
-    } else {
-        return CPS_ERR_ARG;
     }
     return CPS_OK;
 }

@@ -321,3 +321,21 @@ def test_ic0_solve_of_no_iteration_leaves_x(ctx, path):
     x, st = s.solve(b, x=x0.clone(), max_iter=0, check=False)
     assert st.iters == 0 and float((x - x0).norm()) <= 4e-16 * float(x0.norm())
     s.free()
+
+
+def test_a_refused_pin_changes_nothing(ctx):
+    p = synth.channel_block_problem(200, seed=4)           # no cluster holds 79,202 cells
+    s = _assemble(ctx, p)
+    b = torch.as_tensor(synth.rhs(p.mesh, 1), device="cuda")
+    x, st = s.solve(b, rtol=1e-10)
+    before = s.tuning()
+    assert before["two_cyclic"]
+    for path in (-1, 14, 99, cps.PATH_CLUSTER, cps.PATH_CLUSTER_1RED, cps.PATH_CLUSTER_SSTEP2):
+        with pytest.raises(cps.CpsError):
+            s.set_solver_path(path)
+        assert s.tuning() == before
+        x2, st2 = s.solve(b, rtol=1e-10)
+        assert st2.iters == st.iters and torch.equal(x, x2)
+        _, st3 = s.solve(b, rtol=1e-10, precision=cps.MIXED)
+        assert st3.refinements == 1                        # the FP64 loop
+    s.free()
