@@ -421,7 +421,7 @@ void free_sys(cps_sys s) {
     free_cp2(s);
     free_cp1(s);
     free_schur(s);
-    void* bufs[] = {s->slab, s->perm, s->iperm, s->pa,   s->pcol, s->pl,      s->pdinv,
+    void* bufs[] = {s->slab, s->perm,   s->pa,   s->pcol, s->pl,      s->pdinv,
                     s->pdiag, s->ps,  s->pa32,  s->pl32, s->pdinv32, s->ps32, s->gsync};
     for (void* b : bufs)
         if (b) cudaFree(b);

@@ -587,19 +587,18 @@ static int solve_batch_one_launch(const cps_sys* systems, int nsys, const double
     // An ensemble of two-coloured CP2 systems runs on their Schur rows, in either
     // precision; any other on all cells, and any for fewer iterations than a step counts.
     bool tc = max_iter >= 2;
-    for (int i = 0; i < nsys && tc; ++i) {
-        cps_sys s = systems[i];
-        int rc = CPS_OK;
-        if (s->kind != CPS_KIND_CP2) tc = false;
-        else rc = two_colour_order(s, stream, &tc);
-        if (rc == CPS_OK && tc) rc = schur_setup(s, false, stream);
+    for (int i = 0; i < nsys; ++i) tc = tc && systems[i]->kind == CPS_KIND_CP2;
+    if (tc) {
+        const int rc = two_cyclic_setup(systems, nsys, stream, &tc);
         if (rc == CPS_ERR_NOMEM) {              // no room for the rows
             cudaGetLastError();
             tc = false;
         } else if (rc) {
             return rc;
         }
-        if (!tc) break;
+    }
+    for (int i = 0; i < nsys && tc; ++i) {
+        cps_sys s = systems[i];
         hd[i].perm = s->perm;
         hd[i].iperm = s->iperm;
         hd[i].nR = s->colour_start[1];

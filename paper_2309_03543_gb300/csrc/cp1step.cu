@@ -389,18 +389,15 @@ static int cp1_step_one_launch(cps_sys sx, cps_sys sy, double* du, double toll,
     // on the Schur rows where the cell graph has two colours (one for both systems) and
     // a solve may make the two iterations that a step counts
     bool tc = max_iter >= 2;
-    cps_sys sys[2] = {sx, sy};
-    for (cps_sys s : sys) {
-        if (!tc) break;
-        int rc = two_colour_order(s, stream, &tc);
-        if (rc == CPS_OK && tc) rc = schur_setup(s, false, stream);
+    const cps_sys sys[2] = {sx, sy};
+    if (tc) {
+        const int rc = two_cyclic_setup(sys, 2, stream, &tc);
         if (rc == CPS_ERR_NOMEM) {              // no room for the rows
             cudaGetLastError();
             tc = false;
         } else if (rc) {
             return rc;
         }
-        if (!tc) break;
     }
     const void* kernel = tc      ? (const void*)k_cp1_step<2>
                          : mixed ? (const void*)k_cp1_step<1>

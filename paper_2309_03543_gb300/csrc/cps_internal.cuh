@@ -326,15 +326,15 @@ struct cps_sys_s {
     double* dxi = nullptr;      // [nt]
     int32_t* slot_kind = nullptr;   // [3*nt] 0 no-flux, 1 interior, 2 Dirichlet
 
-    // Colour order of the cells (perm, iperm; ncolours 0: not ordered, -1:
-    // two colours do not suffice and no other order was asked for) and IC(0)
+    // Colour order of the cells (perm, iperm; ncolours 0: not ordered, -1: not
+    // two colours, and no other order was asked for) and IC(0)
     // in it (scaled matrix, unit diagonal), each set up on demand.
     bool factored = false;
     cps::SchurData sch;
     int ncolours = 0;
     int64_t colour_start[17] = {0};
     int32_t* perm = nullptr;    // [nt] colour order -> mesh order
-    int32_t* iperm = nullptr;   // [nt] mesh order -> colour order
+    int32_t* iperm = nullptr;   // [nt] mesh order -> colour order (same allocation)
     double* pa = nullptr;       // [3*nt] permuted scaled off-diagonals
     int32_t* pcol = nullptr;    // [3*nt] permuted columns
     double* pl = nullptr;       // [3*nt] IC(0) factor entries per slot
@@ -406,7 +406,7 @@ int assemble_impl(cps_ctx ctx, const double* xy, int64_t nv, const int32_t* tri,
                   int field_loc, int kind, double nu, double dt, cps_sys* out,
                   cudaStream_t stream);
 int precond_impl(cps_sys sys, int precond, cudaStream_t stream);
-int two_colour_order(cps_sys s, cudaStream_t stream, bool* ok);
+int two_cyclic_setup(const cps_sys* systems, int n, cudaStream_t stream, bool* ok);
 void free_schur(cps_sys s);
 int schur_setup(cps_sys s, bool scaled, cudaStream_t stream);
 int schur_init(cps_sys s, const double* b, const double* x, double rtol, long long budget,

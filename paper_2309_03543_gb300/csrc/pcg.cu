@@ -969,8 +969,7 @@ static int choose_two_cyclic(cps_sys s, cudaStream_t stream, bool* take) {
     if (t.pinned || s->kind != CPS_KIND_CP2 || t.tc == 2) return CPS_OK;
     const bool had_rows = s->sch.buf != nullptr;
     bool two = false;
-    int rc = two_colour_order(s, stream, &two);
-    if (rc == CPS_OK && two) rc = schur_setup(s, false, stream);
+    int rc = two_cyclic_setup(&s, 1, stream, &two);
     if (rc == CPS_ERR_NOMEM) {              // no room for the rows: the loop on all cells
         cudaGetLastError();
         return CPS_OK;

@@ -339,3 +339,43 @@ def test_a_refused_pin_changes_nothing(ctx):
         _, st3 = s.solve(b, rtol=1e-10, precision=cps.MIXED)
         assert st3.refinements == 1                        # the FP64 loop
     s.free()
+
+
+def test_first_calls_on_fresh_systems_pay_little(ctx):
+    """The Schur rows are set up by a system's first solve: for an ensemble of small
+    systems in less time than a call takes (2.1 ms before there were rows, 1.1
+    with them, the set-up in between)."""
+    first, later = [], []
+    for rep in range(6):
+        probs = [synth.ensemble_member_problem(512, seed=200 + i) for i in range(16)]
+        systems = [_assemble(ctx, p) for p in probs]
+        bs = [torch.as_tensor(synth.rhs(p.mesh, 80), device="cuda") for p in probs]
+        for call in range(3):
+            xs = [torch.zeros_like(b) for b in bs]
+            torch.cuda.synchronize()
+            t = time.perf_counter()
+            cps.solve_batch(systems, bs, xs, rtol=1e-10)
+            torch.cuda.synchronize()
+            if rep:
+                (later if call else first).append(time.perf_counter() - t)
+        for s in systems:
+            s.free()
+    print("first", np.median(first), "later", np.median(later))
+    assert np.median(first) < 2.2 * np.median(later)
+
+
+def test_a_graph_of_more_colours_keeps_no_order(ctx):
+    """8 bytes a cell that no loop would read: the colouring decides before the order
+    is allocated (722,000 cells: 5.8 MB)."""
+    p = synth.defect_problem(600, seed=3)
+    s = _assemble(ctx, p)
+    b = torch.as_tensor(synth.rhs(p.mesh, 1), device="cuda")
+    x = torch.zeros_like(b)
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    s.solve(b, x=x, rtol=1e-3)
+    torch.cuda.synchronize()
+    held = before - torch.cuda.mem_get_info()[0]
+    print("held", held)
+    assert not s.tuning()["two_cyclic"] and held < 5 << 20
+    s.free()
