@@ -38,7 +38,9 @@ __global__ void k_cp1_coeffs(const double* __restrict__ xy, const int32_t* __res
                              const double* __restrict__ area, const double* __restrict__ eps,
                              const double* __restrict__ kinv, int64_t nt, int64_t nv,
                              bool per_vertex, bool logk, double nu, double dt,
-                             double* __restrict__ T, double* __restrict__ mass, int* err) {
+                             double* __restrict__ T, double* __restrict__ mass, int* err,
+                             float* coupling2) {
+    float most = 0.0f;           // Mbar_12^2 / (Mbar_11 Mbar_22)
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nt;
          e += (int64_t)gridDim.x * blockDim.x) {
         const int64_t v[3] = {tri[3 * e], tri[3 * e + 1], tri[3 * e + 2]};
@@ -75,7 +77,11 @@ __global__ void k_cp1_coeffs(const double* __restrict__ xy, const int32_t* __res
         mass[e] = mb[0] * a;
         mass[nt + e] = mb[1] * a;
         mass[2 * nt + e] = mb[2] * a;
+        const float m12 = (float)mb[1];          // binary32: a size, and FP64 divides are slow
+        most = fmaxf(most, (m12 / (float)mb[0]) * (m12 / (float)mb[2]));
     }
+    most = __int_as_float(__reduce_max_sync(0xffffffffu, __float_as_int(most)));
+    if ((threadIdx.x & 31) == 0) atomicMax(reinterpret_cast<int*>(coupling2), __float_as_int(most));
 }
 
 // lap_k = -nu L du_breve_k for both components; a boundary slot (col = e) has a
@@ -344,24 +350,28 @@ int cp1_setup_impl(cps_sys sx, cps_sys sy, const double* xy, const int32_t* tri,
     sx->cp1 = c;
 
     double *ccx = nullptr, *ccy = nullptr, *area = nullptr;
-    int* err = nullptr;
-    int h_err = 0;
+    int* err = nullptr;          // and the coupling
+    struct {
+        int err;
+        float coupling2;
+    } h{0, 0.0f};
     auto A = [&](void** p, size_t b) { return cudaMallocAsync(p, b, stream); };
     ce = A((void**)&ccx, sizeof(double) * nt);
     if (ce == cudaSuccess) ce = A((void**)&ccy, sizeof(double) * nt);
     if (ce == cudaSuccess) ce = A((void**)&area, sizeof(double) * nt);
-    if (ce == cudaSuccess) ce = A((void**)&err, sizeof(int));
-    if (ce == cudaSuccess) ce = cudaMemsetAsync(err, 0, sizeof(int), stream);
+    if (ce == cudaSuccess) ce = A((void**)&err, sizeof(h));
+    if (ce == cudaSuccess) ce = cudaMemsetAsync(err, 0, sizeof(h), stream);
     if (ce == cudaSuccess) {
         const int g = sx->grid;
         k_cell_geometry<<<g, kBlock, 0, stream>>>(xy, tri, nt, nv, area, ccx, ccy, err);
         k_cp1_coeffs<<<g, kBlock, 0, stream>>>(xy, tri, sx->col, sx->slot_kind, ccx, ccy, area,
                                                eps, kinv, nt, nv,
                                                sx->field_loc == CPS_PER_VERTEX, sx->logk, sx->nu,
-                                               sx->dt, c->T, c->mass, err);
+                                               sx->dt, c->T, c->mass, err,
+                                               reinterpret_cast<float*>(err + 1));
         ce = cudaGetLastError();
         if (ce == cudaSuccess)
-            ce = cudaMemcpyAsync(&h_err, err, sizeof(int), cudaMemcpyDeviceToHost, stream);
+            ce = cudaMemcpyAsync(&h, err, sizeof(h), cudaMemcpyDeviceToHost, stream);
     }
     void* tmp[] = {ccx, ccy, area, err};
     for (void* p : tmp)
@@ -373,9 +383,10 @@ int cp1_setup_impl(cps_sys sx, cps_sys sy, const double* xy, const int32_t* tri,
         return fail(sx, ce == cudaErrorMemoryAllocation ? CPS_ERR_NOMEM : CPS_ERR_CUDA,
                     std::string("cp1_setup: ") + cudaGetErrorString(ce));
     }
-    if (h_err != 0) {
+    c->coupling2 = h.coupling2;
+    if (h.err != 0) {
         free_cp1(sx);
-        return fail(sx, h_err, "cp1_setup: mesh or fields do not match the systems (or bad input)");
+        return fail(sx, h.err, "cp1_setup: mesh or fields do not match the systems (or bad input)");
     }
     return CPS_OK;
 }
@@ -386,12 +397,17 @@ static int cp1_step_one_launch(cps_sys sx, cps_sys sy, double* du, double toll,
                                cps_cp1_stats* stats, cudaStream_t stream) {
     Cp1Data* c = sx->cp1;
     const int64_t nt = sx->nt;
-    // on the Schur rows where the cell graph has two colours (one for both systems) and
-    // a solve may make the two iterations that a step counts
-    bool tc = max_iter >= 2;
+    // On the Schur rows where the cell graph has two colours and a solve may make the
+    // two iterations that a step counts.  To set a pair's rows up costs what one to two
+    // and a half sweeps on all cells lose (3k cells 0.10 ms against 0.10 a sweep, 0.8M
+    // 0.65 against 0.28): a first step does it that will make more sweeps, each coupled one
+    // bringing the change down by about the coupling's size, and else (an isotropic
+    // tensor settles in one: 0.33 ms a step at 3k cells, 0.73 with the set-up) the fifth.
+    const bool many = (c->coupling2 > toll && max_outer >= 2) || c->cell_steps >= 4;
+    bool tc = max_iter >= 2 && (many || (sx->sch.buf && sy->sch.buf));
     const cps_sys sys[2] = {sx, sy};
     if (tc) {
-        const int rc = two_cyclic_setup(sys, 2, stream, &tc);
+        const int rc = two_cyclic_setup_pair(sx, sy, stream, &tc);
         if (rc == CPS_ERR_NOMEM) {              // no room for the rows
             cudaGetLastError();
             tc = false;
@@ -399,6 +415,7 @@ static int cp1_step_one_launch(cps_sys sx, cps_sys sy, double* du, double toll,
             return rc;
         }
     }
+    if (!tc && c->cell_steps < 4) ++c->cell_steps;
     const void* kernel = tc      ? (const void*)k_cp1_step<2>
                          : mixed ? (const void*)k_cp1_step<1>
                                  : (const void*)k_cp1_step<0>;

@@ -163,6 +163,8 @@ struct Cp1Data {
     void* dev = nullptr;         // one-launch step: team state, system descriptors, statistics
     void* hstats = nullptr;      // pinned copy of the one-launch statistics
     int path = 0;                // 0 one launch (Jacobi systems), 1 host-driven sweeps
+    double coupling2 = 0.0;      // largest Mbar_12^2 / (Mbar_11 Mbar_22) of the cells
+    int cell_steps = 0;          // one-launch steps made on all cells so far
     int64_t nt = 0;
 };
 
@@ -407,6 +409,7 @@ int assemble_impl(cps_ctx ctx, const double* xy, int64_t nv, const int32_t* tri,
                   cudaStream_t stream);
 int precond_impl(cps_sys sys, int precond, cudaStream_t stream);
 int two_cyclic_setup(const cps_sys* systems, int n, cudaStream_t stream, bool* ok);
+int two_cyclic_setup_pair(cps_sys x, cps_sys y, cudaStream_t stream, bool* ok);
 void free_schur(cps_sys s);
 int schur_setup(cps_sys s, bool scaled, cudaStream_t stream);
 int schur_init(cps_sys s, const double* b, const double* x, double rtol, long long budget,

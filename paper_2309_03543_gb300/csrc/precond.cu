@@ -533,6 +533,50 @@ int two_cyclic_setup(const cps_sys* systems, int n, cudaStream_t stream, bool* o
     return CPS_OK;
 }
 
+__global__ void k_same_columns(const int32_t* __restrict__ u, const int32_t* __restrict__ v,
+                               int64_t m, int* differ) {
+    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < m;
+         k += (int64_t)gridDim.x * blockDim.x)
+        if (u[k] != v[k]) *differ = 1;
+}
+
+// The same for two systems of one size, which share a cell graph as a rule (the x
+// and y systems of a mesh): y takes x's order if their columns are the same.
+int two_cyclic_setup_pair(cps_sys x, cps_sys y, cudaStream_t stream, bool* ok) {
+    const cps_sys both[2] = {x, y};
+    if (x->ncolours != 0 || y->ncolours != 0 || x->nt != y->nt)
+        return two_cyclic_setup(both, 2, stream, ok);
+    *ok = false;
+    int rc = enqueue_two_colours(x, stream);
+    if (rc) return rc;
+    int* differ = scratch_of(y).flags;
+    int* h = reinterpret_cast<int*>(y->hst);
+    CPS_CUDA_TRY(x->ctx, cudaMemsetAsync(differ, 0, sizeof(int), stream));
+    k_same_columns<<<grid_for(x->ctx, 3 * x->nt), kBlock, 0, stream>>>(x->col, y->col, 3 * x->nt,
+                                                                       differ);
+    CPS_CUDA_TRY(x->ctx, cudaGetLastError());
+    CPS_CUDA_TRY(x->ctx, cudaMemcpyAsync(h, differ, sizeof(int), cudaMemcpyDeviceToHost, stream));
+    CPS_CUDA_TRY(x->ctx, cudaStreamSynchronize(stream));
+    const bool same = *h == 0;
+    if (!has_two_colours(x)) {
+        if (same) y->ncolours = -1;
+        return CPS_OK;
+    }
+    rc = finish_two_colours(x, stream);
+    if (rc) return rc;
+    if (same) {
+        rc = alloc_order(y);
+        if (rc) return rc;
+        const size_t bytes = (size_t)(reinterpret_cast<char*>(x->iperm + x->nt) -
+                                      reinterpret_cast<char*>(x->perm));
+        CPS_CUDA_TRY(x->ctx, cudaMemcpyAsync(y->perm, x->perm, bytes, cudaMemcpyDeviceToDevice,
+                                             stream));
+        for (int k = 0; k < 3; ++k) y->colour_start[k] = x->colour_start[k];
+        y->ncolours = 2;
+    }
+    return two_cyclic_setup(both, 2, stream, ok);
+}
+
 // Permutes the matrix into the colour order and factors it.
 static int factor_ic0(cps_sys s, cudaStream_t stream) {
     int rc = alloc_ic0(s);

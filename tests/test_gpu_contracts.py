@@ -52,7 +52,7 @@ def test_cp1_step_with_one_zero_component(ctx, n, zero):
     du_b[zero] = 0.0
     o = oracle.cp1_step(p, du_b, toll=1e-4, rtol=1e-13)
     sx, sy = _cp1_pair(ctx, p)
-    for _ in range(3):
+    for _ in range(7):                                     # on all cells, then on the Schur rows
         start = torch.full((2, p.mesh.nt), 0.5, dtype=torch.float64, device="cuda")
         du, st = cps.cp1_step(sx, sy, du_b, du=start, toll=1e-4, rtol=1e-12)
         d = du.cpu().numpy()
@@ -301,6 +301,7 @@ def test_max_iter_bounds_the_cp1_steps_solves(ctx):
     p = _walls(synth.channel_block_problem(24, seed=6))
     du_b = synth.cell_vector_field(p.mesh, 9, mean=(0.01, -0.02), scale=0.05)
     sx, sy = _cp1_pair(ctx, p)
+    cps.cp1_step(sx, sy, du_b)                             # a coupled pair: on the Schur rows
     for k in (0, 1, 2, 3):
         # the uncoupled sweep only: two solves
         _, st = cps.cp1_step(sx, sy, du_b, max_outer=0, rtol=1e-15, max_iter=k, check=False)
@@ -379,3 +380,59 @@ def test_a_graph_of_more_colours_keeps_no_order(ctx):
     print("held", held)
     assert not s.tuning()["two_cyclic"] and held < 5 << 20
     s.free()
+
+
+@pytest.mark.parametrize("n", [40, 150])
+def test_first_cp1_step_of_a_pair_pays_little(ctx, n):
+    """A pair that settles in one coupled sweep (isotropic) makes its first steps on
+    all cells: they take less than twice the later ones on the Schur rows (1.3
+    times; with the rows set up by the first step, 2.9 times)."""
+    p = _walls(synth.centred_block_problem(n, seed=2))
+    du_b = torch.as_tensor(synth.cell_vector_field(p.mesh, 3, mean=(0.02, 0.01), scale=0.05),
+                           device="cuda")
+    times = []
+    for rep in range(6):
+        sx, sy = _cp1_pair(ctx, p)
+        t = []
+        for step in range(8):
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            _, st = cps.cp1_step(sx, sy, du_b)
+            t.append(time.perf_counter() - t0)
+            assert st["outer"] == 1
+        if rep:
+            times.append(t)
+        sx.free()
+        sy.free()
+    t = np.median(np.array(times), axis=0)
+    print("steps", 1e3 * t)
+    assert t[0] < 2.0 * min(t[5:])
+
+
+@pytest.mark.parametrize("shuffled", [False, True])
+def test_a_pair_whose_systems_number_their_cells_differently(ctx, shuffled):
+    """The y system's order is its own where its columns are not the x system's: the
+    solve of each of them on the Schur rows matches the oracle's."""
+    p = _walls(synth.channel_block_problem(30, seed=6))
+    m = p.mesh
+    q = p
+    if shuffled:
+        order = np.random.default_rng(3).permutation(m.nt)
+        back = np.argsort(order)
+        q = dataclasses.replace(p, mesh=dataclasses.replace(
+            m, tri=np.ascontiguousarray(m.tri[order]),
+            dirichlet=(back[m.dirichlet // 3] * 3 + m.dirichlet % 3).astype(np.int32)))
+    sx = _assemble(ctx, p, cps.KIND_CP1_X)
+    sy = _assemble(ctx, q, cps.KIND_CP1_Y)
+    cps.cp1_setup(sx, sy, m.xy, m.tri, p.eps, p.kinv)
+    du_b = synth.cell_vector_field(m, 9, mean=(0.01, -0.02), scale=0.05)
+    cps.cp1_step(sx, sy, du_b, max_outer=3, check=False)   # sets the rows up
+    du, _ = cps.cp1_step(sx, sy, du_b, max_outer=0, rtol=1e-12, check=False)
+    f = (p.eps, p.kinv, p.field_loc)
+    T, _, isd, nbr = oracle.side_coefficients(m.xy, m.tri, m.dirichlet, *f, oracle.CP1_X, p.nu, p.dt)
+    for k, (s, r, kind) in enumerate(((sx, p, oracle.CP1_X), (sy, q, oracle.CP1_Y))):
+        A = oracle.assemble(m.xy, r.mesh.tri, r.mesh.dirichlet, *f, kind, p.nu, p.dt)
+        lap = -oracle.cp1_laplacian(T, nbr, isd, du_b[k])
+        assert np.linalg.norm(A.matvec(du[k].cpu().numpy()) - lap) <= 1e-11 * np.linalg.norm(lap)
+    sx.free()
+    sy.free()
