@@ -597,10 +597,12 @@ static void fill_stats(cps_stats* stats, int64_t iters, double rel, int status, 
 // k_init64 left: with the vectors in shared memory where they fit (schur.cu),
 // else streamed (persistent.cu).
 static int persistent_1red(cps_sys s, const Run<double>& v, int grid, const void* base,
-                           size_t bytes, cudaStream_t stream) {
+                           size_t bytes, cudaStream_t stream, int64_t* launches) {
+    ++*launches;
     if (jacobi_resident(s)) return jacobi_run(s, grid, base, bytes, stream);
     k_gear_start<<<s->grid, kBlock, 0, stream>>>(v.a, v.col, v.r, v.p1, v.p0, v.q, s->nt,
                                                  s->partials, s->st);
+    ++*launches;
     CPS_CUDA_TRY(s->ctx, cudaGetLastError());
     return persistent_solve(s, 2, v.a, v.col, v.s, v.y, v.r, v.p0, v.q, v.p1, s->nt, 0, base,
                             bytes, grid, stream);
@@ -706,7 +708,7 @@ static int choose_fp64_path(cps_sys s, const Run<double>& v, cudaStream_t stream
                                                          v.p0, 0.0, probe, 1, s->partials, s->st);
                 const void* base = c.win ? l2_window_base(s, c.win) : nullptr;
                 const size_t bytes = c.win ? l2_window_bytes(s, c.win) : 0;
-                rc = c.path == 4 ? persistent_1red(s, v, c.grid, base, bytes, stream)
+                rc = c.path == 4 ? persistent_1red(s, v, c.grid, base, bytes, stream, &dummy)
                                  : persistent_solve(s, 0, v.a, v.col, v.s, v.y, v.r, v.p0, v.q,
                                                     nullptr, s->nt, 0, base, bytes, c.grid,
                                                     stream);
@@ -1186,11 +1188,11 @@ static int solve_fp64(cps_sys s, const double* b, double* x, double rtol, int64_
             const void* base = window ? l2_window_base(s, window) : nullptr;
             const size_t bytes = window ? l2_window_bytes(s, window) : 0;
             const int pg = s->tune[CPS_FP64].pgrid;
-            int rc = pgear ? persistent_1red(s, v, pg, base, bytes, stream)
+            int rc = pgear ? persistent_1red(s, v, pg, base, bytes, stream, &launches)
                            : persistent_solve(s, 0, v.a, v.col, v.s, v.y, v.r, v.p0, v.q, nullptr,
                                               n, 0, base, bytes, pg, stream);
             if (rc) return rc;
-            ++launches;
+            if (!pgear) ++launches;
             rc = read_state(s, stream, &h);
             if (rc) return rc;
             total += h.iter;

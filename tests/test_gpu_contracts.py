@@ -436,3 +436,16 @@ def test_a_pair_whose_systems_number_their_cells_differently(ctx, shuffled):
         assert np.linalg.norm(A.matvec(du[k].cpu().numpy()) - lap) <= 1e-11 * np.linalg.norm(lap)
     sx.free()
     sy.free()
+
+
+@pytest.mark.parametrize("n,launches", [(400, 3), (900, 4)])
+def test_launches_of_the_persistent_loop_are_counted(ctx, n, launches):
+    """Start, loop and end; above 1.44M cells the streamed loop has a kernel of its
+    own before it."""
+    p = synth.centred_block_problem(n, seed=1)
+    s = _assemble(ctx, p)
+    s.set_solver_path(cps.PATH_PERSISTENT_1RED)
+    b = torch.as_tensor(synth.rhs(p.mesh, 2), device="cuda")
+    _, st = s.solve(b, rtol=1e-6)                          # one run: far from the FP64 floor
+    assert st.launches == launches
+    s.free()
