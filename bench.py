@@ -113,6 +113,7 @@ def traffic_for(tf: dict, n: int):
 # step: the row of S (diagonal 8, six values 48, six columns 24) and x, r, p, q
 # read and written once (64); one step is two Jacobi iterations of all cells.
 BYTES_PER_ROW_STEP_SCHUR = 144
+BYTES_PER_ROW_S = 80           # of which the row of S
 
 
 def loop_name(tf: dict) -> str:
@@ -120,7 +121,11 @@ def loop_name(tf: dict) -> str:
     if tf.get("two_cyclic"):
         return ("k_resident_cg (two-cyclic form of Jacobi-PCG: CG on the explicit Schur complement "
                 "of one colour in one cooperative launch, two Jacobi iterations a step)")
-    if tf.get("persistent_single_reduction"):
+    if tf.get("resident_vectors"):
+        kname = (f"k_resident_cg (whole Jacobi-PCG solve in one cooperative launch, "
+                 f"Chronopoulos-Gear recurrences, {tf['resident_vectors']} vectors"
+                 f"{' and the matrix rows' if tf.get('resident_rows') else ''} in shared memory)")
+    elif tf.get("persistent_single_reduction"):
         kname = ("k_persistent_gear (whole Jacobi-PCG solve in one cooperative launch, "
                  "Chronopoulos-Gear recurrences)")
     elif tf["persistent"]:
@@ -149,9 +154,15 @@ def loop_name(tf: dict) -> str:
 
 
 def loop_bytes(tf: dict) -> int:
-    """Bytes per cell per iteration the chosen FP64 Jacobi loop moves."""
+    """Bytes per cell per iteration the chosen FP64 Jacobi loop moves (outside of
+    shared memory, where it keeps vectors or rows there)."""
     if tf.get("two_cyclic"):
         return BYTES_PER_ROW_STEP_SCHUR // 4
+    if tf.get("resident_vectors"):
+        # the rows (values 24, columns 12), r written and gathered (16), then what is
+        # not resident: w written and read (16), r read by its owner (8)
+        v = tf["resident_vectors"]
+        return (0 if tf.get("resident_rows") else 36) + 16 + (16 if v < 4 else 0) + (8 if v < 5 else 0)
     single = tf["stream_single_reduction"] or tf.get("persistent_single_reduction")
     return BYTES_PER_CELL_ITER_FP64_1RED if single else BYTES_PER_CELL_ITER_FP64
 
@@ -168,7 +179,7 @@ def method_bytes(name: str, tf: dict) -> float:
 
 
 def roofline(tf: dict, nt: int, iters: int, seconds: float, peak: float, peak_kind: str,
-             n: int) -> dict:
+             n: int, l2_bytes: float = 129e6) -> dict:
     """Roofline of one FP64 Jacobi-PCG iteration: achieved = the method's
     108 algorithmic bytes per cell x cells / (solve time / iterations); the
     solve time is the whole timed solve (start-up, stop tests and the final
@@ -179,8 +190,11 @@ def roofline(tf: dict, nt: int, iters: int, seconds: float, peak: float, peak_ki
         # the method's bytes are those of CG on S: half of the rows, and half
         # of the steps that the iteration count says
         achieved = bpc * nt / per_iter / 1e9
-        return {"bound": "fp64 issue (matrix and vectors stay in L2 and shared memory at this "
-                         "size); bytes are CG's on S", "kernel": loop_name(tf),
+        rows = BYTES_PER_ROW_S * nt / 2        # half of the cells are rows of S
+        bound = ("fp64 issue (the rows of S, {:.0f} MB, stay in L2 or shared memory)"
+                 if rows <= l2_bytes else
+                 "fp64 issue (the rows of S, {:.0f} MB, come from HBM)").format(rows / 1e6)
+        return {"bound": bound + "; bytes are CG's on S", "kernel": loop_name(tf),
                 "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                 "peak_kind": peak_kind, "bytes_per_cell_iter": bpc,
                 "algorithmic_bytes_per_iter": bpc * nt, "us_per_iter": 1e6 * per_iter,
@@ -190,7 +204,9 @@ def roofline(tf: dict, nt: int, iters: int, seconds: float, peak: float, peak_ki
     achieved = BYTES_PER_CELL_ITER_METHOD * nt / per_iter / 1e9
     loop_achieved = bpc * nt / per_iter / 1e9
     traffic = traffic_for(tf, n)
-    return {"bound": "hbm", "kernel": loop_name(tf),
+    bound = ("fp64 issue and the two grid-wide waits of an iteration (vectors in shared memory, "
+             "the matrix rows there or in L2)" if tf.get("resident_vectors") else "hbm")
+    return {"bound": bound, "kernel": loop_name(tf),
             "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
             "peak_kind": peak_kind, "bytes_per_cell_iter": BYTES_PER_CELL_ITER_METHOD,
             "algorithmic_bytes_per_iter": BYTES_PER_CELL_ITER_METHOD * nt,

@@ -498,6 +498,12 @@ int cps_get_tuning(cps_sys sys, int precision, int32_t* unroll, int32_t* grid, i
  * Errors: CPS_ERR_ARG. */
 int cps_get_two_cyclic(cps_sys sys, int32_t* taken, double* us_per_iter);
 
+/* What the single-reduction persistent launch on all cells, where it is chosen
+ * or pinned for FP64 Jacobi, keeps in shared memory over the iterations: how
+ * many of its five vectors (0: it streams them) and whether the matrix rows.
+ * Either output may be NULL.  Errors: CPS_ERR_ARG. */
+int cps_get_resident(cps_sys sys, int32_t* vectors, int32_t* rows);
+
 /* Allocation-free solve of a matrix the caller already holds in the padded
  * ELL form that cps_export_matrix writes (no counterpart in the paper; it is
  * an interface for callers that cannot allocate device memory).  Such callers

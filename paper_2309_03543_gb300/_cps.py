@@ -88,6 +88,7 @@ SIGNATURES = {
     "cps_get_tuning": (_I, [_P, _I, _P, _P, _P, _P, _P]),
     "cps_get_gear_shape": (_I, [_P, _P, _P, _P]),
     "cps_get_two_cyclic": (_I, [_P, _P, _P]),
+    "cps_get_resident": (_I, [_P, _P, _P]),
     "cps_set_solver_path": (_I, [_P, _I]),
     "cps_set_batch_path": (_I, [_P, _I]),
     "cps_set_cp1_path": (_I, [_P, _I]),

@@ -155,7 +155,11 @@ class System:
         tc, tus = ctypes.c_int32(), ctypes.c_double()
         self.ctx.check(self.ctx.lib.cps_get_two_cyclic(self.handle, ctypes.byref(tc),
                                                       ctypes.byref(tus)), "cps_get_two_cyclic")
+        rv, rr = ctypes.c_int32(), ctypes.c_int32()
+        self.ctx.check(self.ctx.lib.cps_get_resident(self.handle, ctypes.byref(rv),
+                                                    ctypes.byref(rr)), "cps_get_resident")
         return {"unroll": list(u), "grid": list(g), "block": list(bl),
+                "resident_vectors": rv.value, "resident_rows": bool(rr.value),
                 "two_cyclic": bool(tc.value), "two_cyclic_us_per_iter": tus.value,
                 "cluster": bool(f[0]),
                 "cluster_recurrence": (None, "textbook", "single_reduction", "pipelined", "s_step2",

@@ -405,6 +405,18 @@ int cps_get_two_cyclic(cps_sys sys, int32_t* taken, double* us_per_iter) {
     return CPS_OK;
 }
 
+int cps_get_resident(cps_sys sys, int32_t* vectors, int32_t* rows) {
+    if (!sys) return CPS_ERR_ARG;
+    int rc = set_device(sys->ctx);
+    if (rc) return rc;
+    const cps::Tuning& t = sys->tune[CPS_FP64];
+    bool mat = false;
+    const int v = t.path_done && t.path == 4 ? cps::jacobi_resident(sys, &mat) : 0;
+    if (vectors) *vectors = v;
+    if (rows) *rows = mat ? 1 : 0;
+    return CPS_OK;
+}
+
 int cps_matvec(cps_sys sys, const double* x, double* y, void* stream) {
     CallRange range_("cps_matvec");
     if (!sys) return CPS_ERR_ARG;

@@ -884,16 +884,19 @@ int schur_run(cps_sys s, int grid, bool window, cudaStream_t stream) {
                            window ? schur_window_bytes(s) : 0, stream);
 }
 
-// Whether jacobi_run takes this system: p, s and y of a block's rows have to fit
+// Whether jacobi_run takes this system (the vectors then in shared memory, and in
+// *rows whether the rows are too; else 0): p, s and y of a block's rows have to fit
 // its shared memory (up to 1.44M cells on 152 SMs).  With fewer resident the L1
 // that is left does not hold the gathers: at 2.09M cells p and s resident took
 // 48.1 us an iteration, k_persistent_gear (nothing resident, the L1 whole) 42.5;
 // at 0.98M 21.8 against 23.1, at 0.4M 11.6 against 13.8, at 33k 5.7 against 7.8.
-bool jacobi_resident(cps_sys s) {
+int jacobi_resident(cps_sys s, bool* rows) {
     const int G = resident_grid(s, s->nt);
     size_t smem = 0;
-    return pick_form(3, true, ((((s->nt + G - 1) / G) + 31) & ~(int64_t)31), s->ctx->smem_optin,
-                     &smem) != nullptr;
+    const Form* f = pick_form(3, true, ((((s->nt + G - 1) / G) + 31) & ~(int64_t)31),
+                              s->ctx->smem_optin, &smem);
+    if (rows) *rows = f && f->mat;
+    return f ? f->res : 0;
 }
 
 // FP64 Jacobi on all cells from the state k_init64 left (y, r), the same loop on

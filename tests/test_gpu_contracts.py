@@ -449,3 +449,15 @@ def test_launches_of_the_persistent_loop_are_counted(ctx, n, launches):
     _, st = s.solve(b, rtol=1e-6)                          # one run: far from the FP64 floor
     assert st.launches == launches
     s.free()
+
+
+@pytest.mark.parametrize("n,vectors,rows", [(200, 5, True), (900, 0, False)])
+def test_what_the_persistent_loop_keeps_on_chip_is_reported(ctx, n, vectors, rows):
+    s = _assemble(ctx, synth.centred_block_problem(n, seed=1))
+    assert s.tuning()["resident_vectors"] == 0             # not chosen yet
+    s.set_solver_path(cps.PATH_PERSISTENT_1RED)
+    tu = s.tuning()
+    assert tu["resident_vectors"] == vectors and tu["resident_rows"] == rows
+    s.set_solver_path(cps.PATH_STREAM)
+    assert s.tuning()["resident_vectors"] == 0
+    s.free()
