@@ -988,7 +988,20 @@ __device__ __forceinline__ bool kbp_solve_mixed(const BatchDesc& d, int64_t lo, 
             }
             __syncthreads();
         }
-        if (!ok || sm.flag == 2) break;
+        if (!ok) break;
+        if (sm.flag == 2) {
+            // after replaced residuals: the binary32 run's rounding floor, not the matrix
+            if (sm.updates > 1) {
+                if (sm.rnorm2 > sm.best)
+                    for (int64_t e = lo + threadIdx.x; e < hi; e += kBB) x[e] = d.best[e];
+                __syncthreads();
+                if (threadIdx.x == 0) {
+                    sm.status = CPS_ERR_NOT_CONVERGED;
+                    if (sm.rnorm2 > sm.best) sm.rnorm2 = sm.best;
+                }
+            }
+            break;
+        }
         // x += S^-1 d in FP64 (own rows), then every member's x is final
         // before the next residual reads it at neighbours
         for (int64_t e = lo + threadIdx.x; e < hi; e += kBB) x[e] += (double)dy[e] / S[e];

@@ -1641,6 +1641,12 @@ static int solve_mixed(cps_sys s, const double* b, double* x, double rtol, int64
         }
         if (h.status != CPS_OK) {
             status = h.status;
+            // p.Ap <= 0 after replaced residuals: the binary32 run is at its rounding
+            // floor (a matrix that is not SPD shows in the first one)
+            if (status == CPS_ERR_NOT_SPD && updates > 1) {
+                status = CPS_ERR_NOT_CONVERGED;
+                restore = true;
+            }
             break;
         }
         k_flush_y<float><<<g, kBlock, 0, stream>>>(v.y, v.p0, v.p1, n, s->st);
