@@ -415,10 +415,10 @@ int schur_setup(cps_sys s, bool scaled, cudaStream_t stream);
 int schur_init(cps_sys s, const double* b, const double* x, double rtol, long long budget,
                cudaStream_t stream);
 int schur_back(cps_sys s, const double* b, cudaStream_t stream);
-int schur_run(cps_sys s, int grid, bool window, cudaStream_t stream);
+int schur_run(cps_sys s, bool window, cudaStream_t stream);
 int ensure_gsync(cps_sys s);
 int jacobi_resident(cps_sys s, bool* rows = nullptr);
-int jacobi_run(cps_sys s, int grid, const void* win, size_t win_bytes, cudaStream_t stream);
+int jacobi_run(cps_sys s, const void* win, size_t win_bytes, cudaStream_t stream);
 size_t schur_window_bytes(cps_sys s);
 int true_residual2(cps_sys s, const double* b, const double* x, double* r2, cudaStream_t stream);
 int solve_impl(cps_sys sys, const double* b, double* x, double rtol, int64_t max_iter,

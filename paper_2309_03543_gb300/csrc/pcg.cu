@@ -596,16 +596,16 @@ static void fill_stats(cps_stats* stats, int64_t iters, double rel, int status, 
 // The persistent single-reduction Jacobi loop on all cells from the state
 // k_init64 left: with the vectors in shared memory where they fit (schur.cu),
 // else streamed (persistent.cu).
-static int persistent_1red(cps_sys s, const Run<double>& v, int grid, const void* base,
-                           size_t bytes, cudaStream_t stream, int64_t* launches) {
+static int persistent_1red(cps_sys s, const Run<double>& v, const void* base, size_t bytes,
+                           cudaStream_t stream, int64_t* launches) {
     ++*launches;
-    if (jacobi_resident(s)) return jacobi_run(s, grid, base, bytes, stream);
+    if (jacobi_resident(s)) return jacobi_run(s, base, bytes, stream);
     k_gear_start<<<s->grid, kBlock, 0, stream>>>(v.a, v.col, v.r, v.p1, v.p0, v.q, s->nt,
                                                  s->partials, s->st);
     ++*launches;
     CPS_CUDA_TRY(s->ctx, cudaGetLastError());
     return persistent_solve(s, 2, v.a, v.col, v.s, v.y, v.r, v.p0, v.q, v.p1, s->nt, 0, base,
-                            bytes, grid, stream);
+                            bytes, 0, stream);
 }
 
 // The probes' right-hand side, in wb: 0x3F bytes, a small positive constant.  Not the
@@ -708,7 +708,7 @@ static int choose_fp64_path(cps_sys s, const Run<double>& v, cudaStream_t stream
                                                          v.p0, 0.0, probe, 1, s->partials, s->st);
                 const void* base = c.win ? l2_window_base(s, c.win) : nullptr;
                 const size_t bytes = c.win ? l2_window_bytes(s, c.win) : 0;
-                rc = c.path == 4 ? persistent_1red(s, v, c.grid, base, bytes, stream, &dummy)
+                rc = c.path == 4 ? persistent_1red(s, v, base, bytes, stream, &dummy)
                                  : persistent_solve(s, 0, v.a, v.col, v.s, v.y, v.r, v.p0, v.q,
                                                     nullptr, s->nt, 0, base, bytes, c.grid,
                                                     stream);
@@ -818,9 +818,9 @@ static int choose_fp64_path(cps_sys s, const Run<double>& v, cudaStream_t stream
 }
 
 // Microseconds per iteration of the explicit Schur loop (schur.cu) over a
-// short run from x = 0 on `grid` blocks (0: the default), with or without its
-// vectors in persisting L2; 0 where it cannot run here.
-static int probe_schur(cps_sys s, const double* b, long long probe, int grid, bool window,
+// short run from x = 0, with or without its vectors in persisting L2; 0 where it
+// cannot run here.
+static int probe_schur(cps_sys s, const double* b, long long probe, bool window,
                        cudaEvent_t e0, cudaEvent_t e1, cudaStream_t stream, double* us) {
     *us = 0.0;
     int rc = l2_set_aside(s, window ? 5 : 0, stream);
@@ -829,7 +829,7 @@ static int probe_schur(cps_sys s, const double* b, long long probe, int grid, bo
     for (int rep = 0; rep < 2; ++rep) {          // the first one warms up
         CPS_CUDA_TRY(s->ctx, cudaEventRecord(e0, stream));
         rc = schur_init(s, b, s->wx, 0.0, probe, stream);
-        if (rc == CPS_OK) rc = schur_run(s, grid, window, stream);
+        if (rc == CPS_OK) rc = schur_run(s, window, stream);
         CgState h{};
         if (rc == CPS_OK) rc = read_state(s, stream, &h);
         if (rc) return rc;
@@ -898,8 +898,8 @@ struct Least {
 // up): `per` iterations of the solve's method per CG iteration on S (2 for
 // Jacobi, 1 for IC(0) and the reduced system), max_iter a multiple of it.
 static int solve_two_cyclic(cps_sys s, const double* b, double* x, double rtol, int64_t max_iter,
-                            int per, int grid, bool window, cps_stats* stats,
-                            cudaStream_t stream, bool keep_least = false) {
+                            int per, bool window, cps_stats* stats, cudaStream_t stream,
+                            bool keep_least = false) {
     Least least;
     least.on = keep_least;
     if (keep_least)
@@ -917,7 +917,7 @@ static int solve_two_cyclic(cps_sys s, const double* b, double* x, double rtol, 
     for (int restart = 0; restart < 8; ++restart) {
         const int64_t left = max_iter - total;
         int rc = schur_init(s, b, x, rtol, left / per, stream);
-        if (rc == CPS_OK) rc = schur_run(s, grid, window, stream);
+        if (rc == CPS_OK) rc = schur_run(s, window, stream);
         if (rc == CPS_OK) rc = schur_back(s, b, stream);
         if (rc) return rc;
         k_final64<<<s->grid, kBlock, 0, stream>>>(b, s->wy, s->s, s->a, s->col, n, x, s->partials,
@@ -984,7 +984,7 @@ static int choose_two_cyclic(cps_sys s, cudaStream_t stream, bool* take) {
         double us = 0.0, best = 0.0;
         rc = probe_rhs(s, stream);
         if (rc == CPS_OK)
-            rc = probe_schur(s, s->wb, s->nt >= kTuneMinRows ? 256 : 64, 0, false, e0, e1, stream,
+            rc = probe_schur(s, s->wb, s->nt >= kTuneMinRows ? 256 : 64, false, e0, e1, stream,
                              &us);
         cudaEventDestroy(e0);
         cudaEventDestroy(e1);
@@ -1037,7 +1037,7 @@ static int choose_ic0_path(cps_sys s, const Run<double>& v, cudaStream_t stream)
     for (int ci = 0; ci < nc && rc == CPS_OK; ++ci) {
         const Cand c = cands[ci];
         double us = 0.0;
-        if (c.path == 1) rc = probe_schur(s, s->wb, probe, 0, c.win != 0, e0, e1, stream, &us);
+        if (c.path == 1) rc = probe_schur(s, s->wb, probe, c.win != 0, e0, e1, stream, &us);
         else rc = l2_set_aside(s, c.win, stream);
         for (int rep = 0; rep < 2 && rc == CPS_OK && c.path == 0; ++rep) {   // the first warms up
             if (cudaMemsetAsync(s->wx, 0, sizeof(double) * s->nt, stream) != cudaSuccess ||
@@ -1118,7 +1118,7 @@ static int solve_fp64(cps_sys s, const double* b, double* x, double rtol, int64_
         if (rc) return rc;
         if (take) {
             cps_stats two{};
-            rc = solve_two_cyclic(s, b, x, rtol, max_iter - max_iter % 2, 2, 0, false, &two, stream,
+            rc = solve_two_cyclic(s, b, x, rtol, max_iter - max_iter % 2, 2, false, &two, stream,
                                   keep_least);
             if (stats) *stats = two;
             if (rc != CPS_ERR_NOT_CONVERGED || two.iters + 1 != max_iter) return rc;
@@ -1147,7 +1147,7 @@ static int solve_fp64(cps_sys s, const double* b, double* x, double rtol, int64_
     }
     if (ic0 && max_iter >= 1 && s->ncolours == 2 && s->tune[CPS_FP64].ic0_path == 1 &&
         schur_setup(s, true, stream) == CPS_OK)
-        return solve_two_cyclic(s, b, x, rtol, max_iter, 1, 0, s->tune[CPS_FP64].ic0_win != 0,
+        return solve_two_cyclic(s, b, x, rtol, max_iter, 1, s->tune[CPS_FP64].ic0_win != 0,
                                 stats, stream, keep_least);
     CgState h{};
     int status = CPS_OK;
@@ -1188,7 +1188,7 @@ static int solve_fp64(cps_sys s, const double* b, double* x, double rtol, int64_
             const void* base = window ? l2_window_base(s, window) : nullptr;
             const size_t bytes = window ? l2_window_bytes(s, window) : 0;
             const int pg = s->tune[CPS_FP64].pgrid;
-            int rc = pgear ? persistent_1red(s, v, pg, base, bytes, stream, &launches)
+            int rc = pgear ? persistent_1red(s, v, base, bytes, stream, &launches)
                            : persistent_solve(s, 0, v.a, v.col, v.s, v.y, v.r, v.p0, v.q, nullptr,
                                               n, 0, base, bytes, pg, stream);
             if (rc) return rc;
@@ -1418,7 +1418,7 @@ static int solve_reduced(cps_sys s, const double* b, double* x, double rtol, int
             const int kind = kind_of(c.slot);
             const bool pers = kind != 0;
             double us = 0.0;
-            if (kind == 2) rc = probe_schur(s, s->wb, probe, 0, c.win != 0, e0, e1, stream, &us);
+            if (kind == 2) rc = probe_schur(s, s->wb, probe, c.win != 0, e0, e1, stream, &us);
             else rc = l2_set_aside(s, c.win, stream);
             for (int rep = 0; rep < 2 && rc == CPS_OK && kind != 2; ++rep) {
                 CPS_CUDA_TRY(s->ctx, cudaMemsetAsync(xx, 0, sizeof(double) * n, stream));
@@ -1473,7 +1473,7 @@ static int solve_reduced(cps_sys s, const double* b, double* x, double rtol, int
     const int win = tu.red_win;
     if (kind == 2 && schur_setup(s, false, stream) != CPS_OK) kind = 1;   // no room for the rows
     if (kind == 2) {
-        return solve_two_cyclic(s, b, x, rtol, max_iter, 1, tu.red_pgrid, win != 0, stats, stream);
+        return solve_two_cyclic(s, b, x, rtol, max_iter, 1, win != 0, stats, stream);
     }
     k_permute_in<<<g, kBlock, 0, stream>>>(b, x, s->perm, n, s->wb, s->wx);
     ++launches;

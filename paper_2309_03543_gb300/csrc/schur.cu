@@ -860,13 +860,12 @@ int schur_back(cps_sys s, const double* b, cudaStream_t stream) {
 // Bytes of the five vectors (the L2 window of the loop).
 size_t schur_window_bytes(cps_sys s) { return sizeof(double) * 5 * (size_t)s->sch.ld; }
 
-// The CG run from schur_init's state as one cooperative launch of `grid`
-// blocks (0: one per SM), with the five vectors in persisting L2 if window
-// (the caller holds the set-aside).  State in s->st.
-int schur_run(cps_sys s, int grid, bool window, cudaStream_t stream) {
+// The CG run from schur_init's state as one cooperative launch, with the five
+// vectors in persisting L2 if window (the caller holds the set-aside).  State in
+// s->st.
+int schur_run(cps_sys s, bool window, cudaStream_t stream) {
     SchurData& h = s->sch;
-    int G = resident_grid(s, h.nB);
-    if (grid > 0 && grid < G) G = grid;
+    const int G = resident_grid(s, h.nB);
     SchurArgs P{};
     P.v = h.v;
     P.c = h.c;
@@ -902,9 +901,8 @@ int jacobi_resident(cps_sys s, bool* rows) {
 // FP64 Jacobi on all cells from the state k_init64 left (y, r), the same loop on
 // the scaled matrix's own rows (s = A p in q, w = A r in p1), with r, p, q, y, p1
 // in persisting L2 over win_bytes from win.
-int jacobi_run(cps_sys s, int grid, const void* win, size_t win_bytes, cudaStream_t stream) {
-    int G = resident_grid(s, s->nt);
-    if (grid > 0 && grid < G) G = grid;
+int jacobi_run(cps_sys s, const void* win, size_t win_bytes, cudaStream_t stream) {
+    const int G = resident_grid(s, s->nt);
     SchurArgs P{};
     P.v = s->a;
     P.c = s->col;
