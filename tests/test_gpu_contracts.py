@@ -452,8 +452,9 @@ def test_launches_of_the_persistent_loop_are_counted(ctx, n, launches):
 
 
 @pytest.mark.parametrize("n,vectors,rows", [(200, 5, True), (900, 0, False)])
-def test_what_the_persistent_loop_keeps_on_chip_is_reported(ctx, n, vectors, rows):
-    s = _assemble(ctx, synth.centred_block_problem(n, seed=1))
+def test_what_the_persistent_loop_keeps_on_chip_is_reported(cuda_device, n, vectors, rows):
+    c = cps.Context(0)                                     # remembers no size yet
+    s = _assemble(c, synth.centred_block_problem(n, seed=1))
     assert s.tuning()["resident_vectors"] == 0             # not chosen yet
     s.set_solver_path(cps.PATH_PERSISTENT_1RED)
     tu = s.tuning()
@@ -461,3 +462,4 @@ def test_what_the_persistent_loop_keeps_on_chip_is_reported(ctx, n, vectors, row
     s.set_solver_path(cps.PATH_STREAM)
     assert s.tuning()["resident_vectors"] == 0
     s.free()
+    c.close()
