@@ -357,7 +357,8 @@ struct TeamPlan {
 // teams[t].sys (rows split in multiples of 32).  Then every block takes whole
 // systems in the order `order` (largest estimated work first) from the
 // counter *next until none is left.  FP64 or mixed precision.
-// FORM: 0 FP64 and 1 mixed Jacobi on all cells, 2 every system on its Schur rows.
+// FORM: 0 FP64 and 1 mixed Jacobi on all cells, 2 every system on its Schur rows;
+// 3 and 4 are 0 and 2 for CPS_MIXED, which returns the iterate with the least residual.
 template <int FORM>
 __global__ void __launch_bounds__(kBB, 2) kb_one_launch(const BatchDesc* __restrict__ dd,
                                                         const int* __restrict__ order, int nqueue,
@@ -394,14 +395,14 @@ __global__ void __launch_bounds__(kBB, 2) kb_one_launch(const BatchDesc* __restr
             if (s_k >= nqueue) return;
             d = dd + order[s_k];
         }
-        if (FORM == 2) {
-            kbp_solve_tc(*d, rank, k, tc, rtol, max_iter, 7);
+        if (FORM == 2 || FORM == 4) {
+            kbp_solve_tc<FORM == 4>(*d, rank, k, tc, rtol, max_iter, 7);
         } else {
             const int64_t rows = k == 1 ? d->n : ((d->n + k - 1) / k + 31) / 32 * 32;
             const int64_t lo = min(d->n, (int64_t)rank * rows);
             const int64_t hi = min(d->n, lo + rows);
             if (FORM == 1) kbp_solve_mixed(*d, lo, hi, tc, rtol, max_iter);
-            else kbp_solve(*d, lo, hi, tc, rtol, max_iter);
+            else kbp_solve<FORM == 3>(*d, lo, hi, tc, rtol, max_iter);
         }
     }
 }
@@ -615,8 +616,10 @@ static int solve_batch_one_launch(const cps_sys* systems, int nsys, const double
         if (least) hd[i].start = systems[i]->wx;
     }
     if (least) mixed = false;
-    const void* kernel = tc      ? (const void*)kb_one_launch<2>
+    const void* kernel = tc      ? (least ? (const void*)kb_one_launch<4>
+                                          : (const void*)kb_one_launch<2>)
                          : mixed ? (const void*)kb_one_launch<1>
+                         : least ? (const void*)kb_one_launch<3>
                                  : (const void*)kb_one_launch<0>;
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kBB, 0) !=

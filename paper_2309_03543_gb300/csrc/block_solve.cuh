@@ -28,7 +28,7 @@ struct BatchDesc {
     double* t;                    // one-launch solve only: w = Ahat r
     const float* a32;             // one-launch mixed solve: binary32 matrix and S
     const float* s32;
-    double* best;                 // the best FP64 iterate (FP64 loops: null unless CPS_MIXED)
+    double* best;                 // the best FP64 iterate (CPS_MIXED)
     double* start;                // the caller's x (FP64 loops under CPS_MIXED)
     double* partials;
     CgState* st;
@@ -211,12 +211,12 @@ struct SolveScalars {
     int keep;                     // this round's x is the least so far
 };
 
-// Thread 0, at a round's end (rnorm2 and flag set; keep: CPS_MIXED, which returns
-// the iterate with the least true residual where rtol is not reached): 1 x becomes
+// Thread 0, at a round's end (rnorm2 and flag set) of a solve that keeps the iterate
+// with the least true residual (CPS_MIXED, where rtol is not reached): 1 x becomes
 // the best iterate, 2 the solve's last round ended above it (rnorm2 set to its
 // residual): x is replaced, 0 neither.
-__device__ __forceinline__ int round_ends(SolveScalars& sc, bool keep, bool last) {
-    if (!keep || sc.status != CPS_OK || sc.rnorm2 <= sc.thresh2) return 0;
+__device__ __forceinline__ int round_ends(SolveScalars& sc, bool last) {
+    if (sc.status != CPS_OK || sc.rnorm2 <= sc.thresh2) return 0;
     if (sc.rnorm2 <= sc.best) {
         sc.best = sc.rnorm2;
         return 1;
@@ -270,7 +270,10 @@ __device__ __forceinline__ int round_ends(SolveScalars& sc, bool keep, bool last
 // Restarts from the true residual (at most 8 rounds).  The result and the
 // status go to the system's CgState (iter, rnorm2, bnorm2, status; done = 2),
 // written by the block that holds row 0.  Returns false if a team wait ran
-// out (the status is then CPS_ERR_TIMEOUT).
+// out (the status is then CPS_ERR_TIMEOUT).  KEEP: the iterate with the least true
+// residual of the rounds is returned, through d.best (a form of its own: in the
+// kernels that do not keep it its code costs 1%).
+template <bool KEEP>
 __device__ __forceinline__ bool kbp_solve(const BatchDesc& d, int64_t lo, int64_t hi,
                                           TeamCtx* tc, double rtol, long long max_iter) {
     __shared__ SolveScalars sc;
@@ -438,12 +441,12 @@ __device__ __forceinline__ bool kbp_solve(const BatchDesc& d, int64_t lo, int64_
             sc.it = 0;
             sc.rnorm2 = nn[0];
             sc.flag = (sc.status != CPS_OK || nn[0] <= sc.thresh2 || sc.total >= max_iter) ? 1 : 0;
-            sc.keep = round_ends(sc, d.best != nullptr, round == 7);
+            if (KEEP) sc.keep = round_ends(sc, round == 7);
         }
         __syncthreads();
-        if (sc.keep == 1)
+        if (KEEP && sc.keep == 1)
             for (int64_t e = lo + threadIdx.x; e < hi; e += kBB) d.best[e] = d.x[e];
-        if (sc.keep == 2)
+        if (KEEP && sc.keep == 2)
             for (int64_t e = lo + threadIdx.x; e < hi; e += kBB) d.x[e] = d.best[e];
         if (sc.flag) break;
     }
@@ -469,6 +472,7 @@ __device__ __forceinline__ bool kbp_solve(const BatchDesc& d, int64_t lo, int64_
 // odd one's last iteration is not made); per step one pass over the rows of S (80 B
 // and 9 FP64 FMAs a row) and one over the vectors.  The
 // stop test runs on the steps whose low bits are all set in mask.
+template <bool KEEP>
 __device__ __forceinline__ bool kbp_solve_tc(const BatchDesc& d, int rank, int k, TeamCtx* tc,
                                              double rtol, long long max_iter, int mask) {
     __shared__ SolveScalars sc;
@@ -696,10 +700,10 @@ __device__ __forceinline__ bool kbp_solve_tc(const BatchDesc& d, int rank, int k
             sc.it = 0;
             sc.rnorm2 = nn[0];
             sc.flag = (sc.status != CPS_OK || nn[0] <= sc.thresh2 || sc.total + 1 >= max_iter) ? 1 : 0;
-            sc.keep = round_ends(sc, d.best != nullptr, round == 7);
+            if (KEEP) sc.keep = round_ends(sc, round == 7);
         }
         __syncthreads();
-        if (sc.keep) {
+        if (KEEP && sc.keep) {
             double* to = sc.keep == 1 ? d.best : d.x;
             const double* from = sc.keep == 1 ? d.x : d.best;
             for (int i = rlo + (int)threadIdx.x; i < rhi; i += kBB) to[perm[i]] = from[perm[i]];

@@ -228,10 +228,10 @@ __global__ void __launch_bounds__(kBB, 2) k_cp1_step(Cp1DevArgs P) {
         if (!ok) break;
         // the two solves, each by the whole grid, warm-started from du
         for (int k = 0; k < 2 && ok; ++k)
-            ok = (FORM == 2   ? kbp_solve_tc(P.sys[k], (int)blockIdx.x, G, &s_tc, P.rtol,
+            ok = (FORM == 2   ? kbp_solve_tc<false>(P.sys[k], (int)blockIdx.x, G, &s_tc, P.rtol,
                                              P.max_iter, 0)
                   : FORM == 1 ? kbp_solve_mixed(P.sys[k], lo, hi, &s_tc, P.rtol, P.max_iter)
-                              : kbp_solve(P.sys[k], lo, hi, &s_tc, P.rtol, P.max_iter)) && ok;
+                              : kbp_solve<false>(P.sys[k], lo, hi, &s_tc, P.rtol, P.max_iter)) && ok;
         if (!ok) break;
         // every block: the change sums of its rows (du final everywhere after
         // the team sum that ends each solve), one exact team sum; the solves'
@@ -448,7 +448,7 @@ static int cp1_step_one_launch(cps_sys sx, cps_sys sy, double* du, double toll,
         d.t = s->wp1;
         d.a32 = s->a32;
         d.s32 = s->s32;
-        d.best = tc || !mixed ? nullptr : s->wbest;
+        d.best = s->wbest;
         d.partials = s->partials;
         d.st = s->st;
         d.n = nt;
