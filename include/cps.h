@@ -321,8 +321,11 @@ int cps_cp1_setup(cps_sys sys_x, cps_sys sys_y, const double* xy, const int32_t*
  * systems use the Jacobi preconditioner the whole outer iteration runs by
  * default in one cooperative launch: each sweep's right-hand sides, both
  * solves (the single-reduction Jacobi CG of cps_solve_batch, FP64 or mixed,
- * by all the launch's blocks), the change test and the stop decision on the
- * device, the statistics read once at the end; otherwise (or after
+ * by all the launch's blocks; in FP64 on the Schur rows, with a stop test every
+ * step, where the cell graph has two colours: from the first step of a pair
+ * whose coupling lets it expect more than two coupled sweeps, else from its
+ * fifth), the change test and the stop decision on the device, the statistics
+ * read once at the end; otherwise (or after
  * cps_set_cp1_path(sys_x, CPS_CP1_HOST)) each solve is a cps_solve and the
  * change sums are read back after every sweep.  Errors: as cps_solve
  * (CPS_ERR_TIMEOUT: a device-side wait of the one launch ran out);
