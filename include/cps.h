@@ -200,14 +200,13 @@ int cps_solve(cps_sys sys, const double* b, double* x, double rtol, int64_t max_
  * complements (two Jacobi iterations a step, counted as two; see
  * CPS_PATH_AUTO).  Else the iteration is the single-reduction
  * (Chronopoulos-Gear) form of Jacobi CG, restarted from the true residual up to
- * 8 times.  A team
- * wait that runs out (about one second) gives CPS_ERR_TIMEOUT.  With
- * cps_set_batch_path(ctx, CPS_BATCH_GRAPH) instead one launch per phase for
+ * 8 times.  A team wait that runs out (about one second) gives
+ * CPS_ERR_TIMEOUT.  With cps_set_batch_path(ctx, CPS_BATCH_GRAPH) instead one launch per phase for
  * all systems, a per-system convergence mask, and iteration chunks replayed
  * from a CUDA graph (a system of more than 33,554,432 cells is rejected there
  * with CPS_ERR_ARG -- solve it alone).  CPS_MIXED with other systems among
- * them: by default the same one launch, each system (or team) running the single solve's refinement with
- * every decision on the device -- binary32 textbook CG inner iterations with
+ * them: by default the same one launch, each system (or team) running the
+ * single solve's refinement with every decision on the device -- binary32 textbook CG inner iterations with
  * FP64 inner products, an FP64 true residual after each, the best FP64
  * iterate kept (stats.refinements = residual replacements); with
  * CPS_BATCH_GRAPH instead each system's solve (whose residual replacements
