@@ -397,9 +397,15 @@ __device__ __forceinline__ void tagged_allreduce(const double (&v)[NV], unsigned
                 const int sh = E - Eq;
                 t = lane < nq ? s_g[k][lane] : 0;
                 if (sh > 0) t = sh > 61 ? 0 : (t + (1LL << (sh - 1))) >> sh;
-                static_assert(kPollPer <= 8, "the lanes of the sum");
-#pragma unroll
-                for (int d = 4; d > 0; d >>= 1) t += __shfl_down_sync(0xffffffffu, t, d);
+                // at most 2^58 a lane: biased into three limbs of 20 bits (as in
+                // warp_sum_fixed; a tree of 64-bit shuffles takes twice as long)
+                const unsigned long long u = (unsigned long long)t + (1ULL << 59);
+                const unsigned int mask = (1u << 20) - 1u;
+                const unsigned long long s0 = __reduce_add_sync(0xffffffffu, (unsigned)u & mask);
+                const unsigned long long s1 =
+                    __reduce_add_sync(0xffffffffu, (unsigned)(u >> 20) & mask);
+                const unsigned long long s2 = __reduce_add_sync(0xffffffffu, (unsigned)(u >> 40));
+                t = (long long)(s0 + (s1 << 20) + (s2 << 40) - (32ULL << 59));
             }
         }
         if (q == 0) {
